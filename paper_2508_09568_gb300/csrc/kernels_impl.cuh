@@ -2,6 +2,8 @@
 #pragma once
 
 #include <algorithm>
+#include <utility>
+#include <vector>
 
 #include "mhd_adjoint.cuh"
 #include "mhd_aux.cuh"
@@ -25,37 +27,98 @@ static StepArgs<R> to_args(const StepHostArgs& h) {
     a.work = h.work;
     a.dt_ptr = h.dt_ptr;
     a.dt_val = h.dt_val;
-    a.gamma = h.gamma;
-    a.eps = h.eps;
-    for (int d = 0; d < 3; ++d) a.dxi[d] = h.dxi[d];
+    a.gamma = R(h.gamma);
+    a.gm1 = R(h.gamma - 1.0);
+    a.gm1i = R(1.0 / (h.gamma - 1.0));
+    a.eps = R(h.eps);
+    for (int d = 0; d < 3; ++d) {
+        a.dxi[d] = h.dxi[d];
+        a.dxir[d] = R(h.dxi[d]);
+    }
     a.limiter = h.limiter;
     a.riemann = h.riemann;
     a.err = h.err;
     return a;
 }
 
-template <typename R, int NDIM, int TX, int TY, int NT, int MINB = 1, bool PREFETCH = false>
+// The chunks of a 3D plane shared out to the warps (StepPlan), longest first to the least loaded
+// warp, for every number of in-plane flux chunks moved to phase A; the split with the shortest
+// two phases is taken.  Costs in cycles of a chunk with four
+// warps per scheduler running, measured (FP32, 32x8).
+template <typename C>
+static StepPlan make_plan() {
+    constexpr int PREP = 2480, FACE = 1450, EDGE = 1400, CONV = 620, UPD = 700;
+    auto share = [](std::vector<std::pair<int, int>> tasks, StepPlan& P, int phase) {
+        std::stable_sort(tasks.begin(), tasks.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
+        int load[StepPlan::MAXW] = {}, top = 0;
+        std::vector<std::pair<int, int>> list[StepPlan::MAXW];
+        for (const auto& t : tasks) {
+            const int w = (int)(std::min_element(load, load + C::NWARP) - load);
+            list[w].push_back(t);
+            load[w] += t.first;
+            top = std::max(top, load[w]);
+        }
+        for (int w = 0; w < StepPlan::MAXW; ++w) {
+            // the short, latency-bound chunks at another place in the list of each warp of a
+            // scheduler (warps w, w + 4, ...), so that the others have work meanwhile
+            auto& L = list[w];
+            if (L.size() > 1) std::rotate(L.begin(), L.end() - (w / 4) % (int)L.size(), L.end());
+            if ((int)L.size() > 8 * C::NQ - (C::NQ > 1)) return 1 << 30;
+            P.t[phase][w][0] = P.t[phase][w][1] = ~0ull;
+            for (size_t k = 0; k < L.size(); ++k)
+                P.t[phase][w][k / 8] ^= (255ull ^ (unsigned long long)L[k].second) << (8 * (k % 8));
+        }
+        return top;
+    };
+    StepPlan best{};
+    int least = 1 << 30;
+    for (int x = 0; x <= C::IEZ::N; ++x) {
+        std::vector<std::pair<int, int>> A, B;
+        for (int q = 0; q < C::NZ; ++q) A.emplace_back(q < C::IFZ::N ? FACE : EDGE, C::NI + q);
+        for (int q = 0; q < C::IPR::N; ++q) B.emplace_back(PREP, C::NI + C::NZ + q);
+        for (int q = 0; q < C::NI; ++q) {
+            const int cost = q < C::IFX::N + C::IFY::N ? FACE : EDGE;
+            if (q >= C::NI - x) A.emplace_back(cost, q);
+            else B.emplace_back(cost, q);
+        }
+        for (int q = 0; q < C::ICV::N; ++q) A.emplace_back(CONV, C::NI + C::NZ + C::IPR::N + q);
+        for (int q = 0; q < C::IUP::N; ++q) B.emplace_back(UPD, C::NI + C::NZ + C::IPR::N + C::ICV::N + q);
+        StepPlan P{};
+        const int a = share(A, P, 0), b = share(B, P, 1);
+        if (a < (1 << 30) && b < (1 << 30) && a + b < least) {
+            least = a + b;
+            best = P;
+        }
+    }
+    return best;
+}
+
+template <typename R, int NDIM, int TX, int TY, int NT, int MINB = 1>
 struct StepInst {
-    using C = StepCfg<R, NDIM, TX, TY, NT>;
-    static_assert(C::SMEM_BYTES * MINB <= 227 * 1024, "tile too large for shared memory");
+    using C = StepCfg<R, NDIM, TX, TY, NT, MINB>;
+    static_assert((C::SMEM_BYTES + 1024) * MINB <= 228 * 1024, "tile too large for shared memory");
+    static_assert(C::NI + C::NZ + C::IPR::N + C::ICV::N + C::IUP::N < 255 && C::NWARP >= 4 * (NDIM == 3) &&
+                      C::NWARP <= StepPlan::MAXW,
+                  "chunk numbers are bytes");
     static cudaError_t prepare() {
-        cudaError_t e = cudaFuncSetAttribute(step_kernel<R, NDIM, TX, TY, NT, MINB, PREFETCH, false>,
+        cudaError_t e = cudaFuncSetAttribute(step_kernel<R, NDIM, TX, TY, NT, MINB, false>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
         if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(step_kernel<R, NDIM, TX, TY, NT, MINB, PREFETCH, true>,
+        return cudaFuncSetAttribute(step_kernel<R, NDIM, TX, TY, NT, MINB, true>,
                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
     }
     static cudaError_t occupancy(int* blocks) {
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, step_kernel<R, NDIM, TX, TY, NT, MINB, PREFETCH, false>,
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, step_kernel<R, NDIM, TX, TY, NT, MINB, false>,
                                                              NT, C::SMEM_BYTES);
     }
     // asynchronous stepping (a.slice set) runs its own instantiation
     static cudaError_t launch(const void* args, int grid, cudaStream_t s) {
         const StepArgs<R> a = to_args<R>(*static_cast<const StepHostArgs*>(args));
+        static const StepPlan plan = NDIM == 3 ? make_plan<C>() : StepPlan{};
         if (a.slice)
-            step_kernel<R, NDIM, TX, TY, NT, MINB, PREFETCH, true><<<grid, NT, C::SMEM_BYTES, s>>>(a);
+            step_kernel<R, NDIM, TX, TY, NT, MINB, true><<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
         else
-            step_kernel<R, NDIM, TX, TY, NT, MINB, PREFETCH, false><<<grid, NT, C::SMEM_BYTES, s>>>(a);
+            step_kernel<R, NDIM, TX, TY, NT, MINB, false><<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
         return cudaGetLastError();
     }
     static StepLaunch entry() {

@@ -28,20 +28,13 @@ template <typename R>
 MHD_HD R fmin1(R a, R b) { return a <= b ? a : b; }
 
 // Limited undivided slope from the two one-sided differences a = q_i - q_{i-1},
-// b = q_{i+1} - q_i (Sec. 2.1.4).  limiter 0: minmod, 1: monotonised central.
-// Zero when a*b <= 0; otherwise the selected candidate (ties: the first).
+// b = q_{i+1} - q_i (Sec. 2.1.4).  limiter 0: minmod, 1: monotonised central (the smallest of
+// 2a, 2b and (a + b)/2 in magnitude).  Zero when a and b differ in sign or one is 0.
 template <typename R>
 MHD_HD R limited(R a, R b, int limiter) {
-    R pick;
-    if (limiter == 0) {
-        pick = sel(le(rabs(a), rabs(b)), a, b);
-    } else {
-        const R c = R(0.5) * (a + b);
-        const R a2 = a + a, b2 = b + b;
-        const R m2v = sel(le(rabs(a2), rabs(b2)), a2, b2);
-        pick = sel(le(rabs(c), rabs(m2v)), c, m2v);
-    }
-    return sel(gt(a * b, R(0)), pick, R(0));
+    const R m = minmod_(a, b);
+    if (limiter == 0) return m;
+    return minmod_(R(0.5) * (a + b), m + m);
 }
 
 // Fast magnetosonic speed along a normal with field component bn (transverse bt1, bt2).
@@ -110,7 +103,7 @@ MHD_HD void hancock_dw(const R q[8], const R dW[3][8], const R dxi[3], R hdt, R 
     const R u = q[Q_U], v = q[Q_V], w = q[Q_W], rho = q[Q_RHO], P = q[Q_P];
     const R us = u * dxi[0], vs = v * dxi[1], ws = w * dxi[2];
     const R divu = fma_(dxi[0], dW[0][Q_U], fma_(dxi[1], dW[1][Q_V], dxi[2] * dW[2][Q_W]));
-    const R ri = rdiv(R(1), rho);
+    const R ri = rcp_(rho);
     auto adv = [&](int k) { return fma_(us, dW[0][k], fma_(vs, dW[1][k], ws * dW[2][k])); };
     out[0] = rho - hdt * fma_(rho, divu, adv(Q_RHO));
     out[4] = P - hdt * fma_(gamma * P, divu, adv(Q_P));
@@ -124,107 +117,145 @@ MHD_HD void hancock_dw(const R q[8], const R dW[3][8], const R dxi[3], R hdt, R 
     }
 }
 
+// Fast speeds as the double-precision Riemann solvers of the step take them: 2 rho c_f^2 = s + sqrt(disc) with
+// s = gamma P + B^2 and disc = (gamma P - B^2)^2 + 4 gamma P Bt^2 (Bt^2 the transverse part of
+// B^2): the value of fast_speed with the density divided out once at the end and both terms of
+// disc non-negative, so that nothing cancels when gamma P ~ Bn^2 and B is along n.  disc's
+// first term and s do not depend on the direction: a corner's two speeds share them.
+// Returns 2 rho c_f^2.
+template <typename R>
+MHD_HD R fast_h(R gP4, R s, R dd, R bt2) {
+    return s + rsqrt_(fma_(gP4, bt2, dd));
+}
+
 // HLLD flux (Sec. 2.1.2; Miyoshi & Kusano 2005) through a face with normal field bn.
 // Left/right states: rho, un, ut1, ut2, P, bt1, bt2.  F receives the fluxes of
 // (rho, rho*un, rho*ut1, rho*ut2, E) of the region covering x/t = 0.
 // Wave speeds S_L = min(un_L, un_R) - max(cf_L, cf_R), S_R = max(..) + max(..);
 // the star state is degenerate when |D| <= eps*bn^2 (then transverse v, B keep their
-// outer values); ties at x/t = 0 take the left state.  Every lane takes the same path:
-// the states of all regions are formed and the one at x/t = 0 is selected.
+// outer values); ties at x/t = 0 take the left state.  Every lane takes the same path.
+// The contact speed decides the side (left when S_M >= 0 or S_L >= 0), so what only one side
+// needs (energies, v.B, the Alfven speed) is formed once, from the selected side.
+//
+// The two precisions end differently.  Single precision forms F + S (U* - U) + S* (U** - U*)
+// in that order, whose rounding runs are compared by.  Double precision, where the FP64 pipe
+// bounds every kernel, takes the ideal-MHD flux function at the selected region's state and
+// total pressure instead, which the jump conditions make equal (in the star regions the normal
+// velocity is S_M and the total pressure p_T*), and the shared form of the fast speed: about a
+// third fewer FP64 operations.
 template <typename R>
 MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[5]) {
+    constexpr bool F64 = sizeof(R) == 8;
     const R zero = R(0), half = R(0.5);
     const R bn2 = bn * bn;
-    // outer states
     const R rl = L[0], ul = L[1], vl = L[2], wl = L[3], pl = L[4], byl = L[5], bzl = L[6];
     const R rr = Rt[0], ur = Rt[1], vr = Rt[2], wr = Rt[3], pr = Rt[4], byr = Rt[5], bzr = Rt[6];
-    const R b2l = fma_(byl, byl, fma_(bzl, bzl, bn2)), b2r = fma_(byr, byr, fma_(bzr, bzr, bn2));
+    R b2l, b2r, cmax;
+    if constexpr (F64) {
+        const R btl = fma_(byl, byl, bzl * bzl), btr = fma_(byr, byr, bzr * bzr), g4 = R(4) * gamma;
+        b2l = bn2 + btl;
+        b2r = bn2 + btr;
+        // the larger fast speed with one square root for the two sides (the root is monotone)
+        const R dfl = fma_(gamma, pl, -b2l), dfr = fma_(gamma, pr, -b2r);
+        const R hl = fast_h(g4 * pl, fma_(gamma, pl, b2l), dfl * dfl, btl);
+        const R hr = fast_h(g4 * pr, fma_(gamma, pr, b2r), dfr * dfr, btr);
+        cmax = rsqrt_(half * fmax_(hl * rcp_(rl), hr * rcp_(rr)));
+    } else {
+        b2l = fma_(byl, byl, fma_(bzl, bzl, bn2));
+        b2r = fma_(byr, byr, fma_(bzr, bzr, bn2));
+        cmax = fmax_(fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl), fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr));
+    }
     const R ptl = fma_(half, b2l, pl), ptr = fma_(half, b2r, pr);
-    const R el = fma_(pl, gm1i, half * fma_(rl, fma_(ul, ul, fma_(vl, vl, wl * wl)), b2l));
-    const R er = fma_(pr, gm1i, half * fma_(rr, fma_(ur, ur, fma_(vr, vr, wr * wr)), b2r));
-    const R cfl = fast_speed(rdiv(R(1), rl), gamma * pl, bn, byl, bzl);
-    const R cfr = fast_speed(rdiv(R(1), rr), gamma * pr, bn, byr, bzr);
-    const R vbl = fma_(ul, bn, fma_(vl, byl, wl * bzl)), vbr = fma_(ur, bn, fma_(vr, byr, wr * bzr));
-    const R cmax = fmax_(cfl, cfr);
     const R sl = fmin_(ul, ur) - cmax;
     const R sr = fmax_(ul, ur) + cmax;
     const R sul = sl - ul, sur = sr - ur;
     const R dl = sul * rl, dr = sur * rr;
-    const R deni = rdiv(R(1), dr - dl);
+    const R deni = rcp_(dr - dl);
     const R sm = (fma_(dr, ur, -dl * ul) - ptr + ptl) * deni;
-    const R pts = fma_(dl * dr, ur - ul, fma_(dr, ptl, -dl * ptr)) * deni;
 
-    // star states
+    // star states (transverse velocity and field)
     const R sml = sl - sm, smr = sr - sm;
-    const R sli = rdiv(R(1), sml), sri = rdiv(R(1), smr);
+    const R sli = rcp_(sml), sri = rcp_(smr);
     const R rsl = dl * sli, rsr = dr * sri;
     const R Dl = fma_(dl, sml, -bn2), Dr = fma_(dr, smr, -bn2);
-    const auto degl = le(rabs(Dl), eps * bn2), degr = le(rabs(Dr), eps * bn2);
-    const R Dli = sel(degl, zero, rdiv(R(1), Dl)), Dri = sel(degr, zero, rdiv(R(1), Dr));
-    const R nul = bn * (sm - ul) * Dli, nur = bn * (sm - ur) * Dri;
-    const R nbl = fma_(dl, sul, -bn2) * Dli, nbr = fma_(dr, sur, -bn2) * Dri;
-    const R vsl = sel(degl, vl, fma_(-byl, nul, vl)), wsl = sel(degl, wl, fma_(-bzl, nul, wl));
-    const R vsr = sel(degr, vr, fma_(-byr, nur, vr)), wsr = sel(degr, wr, fma_(-bzr, nur, wr));
-    const R bysl = sel(degl, byl, byl * nbl), bzsl = sel(degl, bzl, bzl * nbl);
-    const R bysr = sel(degr, byr, byr * nbr), bzsr = sel(degr, bzr, bzr * nbr);
-    const R vbsl = fma_(sm, bn, fma_(vsl, bysl, wsl * bzsl)), vbsr = fma_(sm, bn, fma_(vsr, bysr, wsr * bzsr));
-    const R esl = fma_(sul, el, fma_(-ptl, ul, fma_(pts, sm, bn * (vbl - vbsl)))) * sli;
-    const R esr = fma_(sur, er, fma_(-ptr, ur, fma_(pts, sm, bn * (vbr - vbsr)))) * sri;
+    const R epb = eps * bn2;
+    const auto degl = le(rabs(Dl), epb), degr = le(rabs(Dr), epb);
+    const R Dli = sel(degl, zero, rcp_(Dl)), Dri = sel(degr, zero, rcp_(Dr));
+    const R nul = bn * (sm - ul) * Dli, nur = bn * (sm - ur) * Dri;   // 0 when degenerate
+    const R nbl = sel(degl, R(1), fma_(dl, sul, -bn2) * Dli), nbr = sel(degr, R(1), fma_(dr, sur, -bn2) * Dri);
+    const R vsl = fma_(-byl, nul, vl), wsl = fma_(-bzl, nul, wl);
+    const R vsr = fma_(-byr, nur, vr), wsr = fma_(-bzr, nur, wr);
+    const R bysl = byl * nbl, bzsl = bzl * nbl;
+    const R bysr = byr * nbr, bzsr = bzr * nbr;
 
-    // double-star states
+    // double-star states (sign of bn: at bn = 0 their region has zero width and is never the
+    // one selected, so the value there does not matter)
     const R sql = rsqrt_(rsl), sqr = rsqrt_(rsr);
-    const R abn = rabs(bn);
-    const R ssl = sm - rdiv(abn, sql), ssr = sm + rdiv(abn, sqr);
-    // sign of bn (+-1; at bn = 0 the double-star region has zero width, ssl = sm = ssr, and
-    // is never the one selected, so its value there does not matter)
     const R sgn = copysign(R(1), bn);
-    const R isum = rdiv(R(1), sql + sqr);
+    const R isum = rcp_(sql + sqr);
     const R vss = fma_(sql, vsl, fma_(sqr, vsr, (bysr - bysl) * sgn)) * isum;
     const R wss = fma_(sql, wsl, fma_(sqr, wsr, (bzsr - bzsl) * sgn)) * isum;
     const R sq2 = sql * sqr * sgn;
     const R byss = fma_(sql, bysr, fma_(sqr, bysl, sq2 * (vsr - vsl))) * isum;
     const R bzss = fma_(sql, bzsr, fma_(sqr, bzsl, sq2 * (wsr - wsl))) * isum;
-    const R vbss = fma_(sm, bn, fma_(vss, byss, wss * bzss));
-    const R essl = fma_(-sql * sgn, vbsl - vbss, esl);
-    const R essr = fma_(sqr * sgn, vbsr - vbss, esr);
 
-    // region at x/t = 0 (priority: the leftmost wave with speed >= 0):
-    // L (sl >= 0), *L, **L, **R, *R, R
-    const auto gl = ge(sl, zero), gsl = ge(ssl, zero), gm = ge(sm, zero), gsr = ge(ssr, zero), gr = ge(sr, zero);
-    const auto left = mor(gl, mor(gsl, gm));                       // L, *L or **L
-    const auto outer = mor(gl, mnot(mor(gsl, mor(gm, mor(gsr, gr)))));   // L or R
-    const auto dstar = mand(mnot(mor(gl, gsl)), mor(gm, gsr));    // **L or **R
-    // flux of the outer state on the chosen side
+    // the side of x/t = 0 and what is needed of it
+    const auto gl = ge(sl, zero), left = mor(gl, ge(sm, zero));
+    const R S = sel(left, sl, sr), su = sel(left, sul, sur), si = sel(left, sli, sri);
     const R r0 = sel(left, rl, rr), u0 = sel(left, ul, ur), v0 = sel(left, vl, vr), w0 = sel(left, wl, wr);
-    const R by0 = sel(left, byl, byr), bz0 = sel(left, bzl, bzr), pt0 = sel(left, ptl, ptr);
-    const R e0 = sel(left, el, er), vb0 = sel(left, vbl, vbr);
-    const R m0 = r0 * u0;
-    R f0 = m0;
-    R f1 = fma_(m0, u0, pt0 - bn2);
-    R f2v = fma_(m0, v0, -by0 * bn);
-    R f3 = fma_(m0, w0, -bz0 * bn);
-    R f4 = fma_(e0 + pt0, u0, -bn * vb0);
-    // F* = F + S (U* - U)
-    const R S = sel(left, sl, sr);
-    const R rs = sel(left, rsl, rsr);
-    const R vs = sel(left, vsl, vsr), ws = sel(left, wsl, wsr), es = sel(left, esl, esr);
-    const R us1 = rs * sm, us2 = rs * vs, us3 = rs * ws;
-    const R g0 = fma_(S, rs - r0, f0);
-    const R g1 = fma_(S, us1 - m0, f1);
-    const R g2 = fma_(S, fma_(-r0, v0, us2), f2v);
-    const R g3 = fma_(S, fma_(-r0, w0, us3), f3);
-    const R g4 = fma_(S, es - e0, f4);
-    // F** = F* + S* (U** - U*); the density and normal momentum are unchanged
-    const R Ss = sel(left, ssl, ssr);
-    const R ess = sel(left, essl, essr);
-    const R h2 = fma_(Ss, fma_(rs, vss, -us2), g2);
-    const R h3 = fma_(Ss, fma_(rs, wss, -us3), g3);
-    const R h4 = fma_(Ss, ess - es, g4);
-    F[0] = sel(outer, f0, g0);
-    F[1] = sel(outer, f1, g1);
-    F[2] = sel(outer, f2v, sel(dstar, h2, g2));
-    F[3] = sel(outer, f3, sel(dstar, h3, g3));
-    F[4] = sel(outer, f4, sel(dstar, h4, g4));
+    const R p0 = sel(left, pl, pr), by0 = sel(left, byl, byr), bz0 = sel(left, bzl, bzr);
+    const R b20 = sel(left, b2l, b2r), pt0 = sel(left, ptl, ptr);
+    const R rs = sel(left, rsl, rsr), vs = sel(left, vsl, vsr), ws = sel(left, wsl, wsr);
+    const R bys = sel(left, bysl, bysr), bzs = sel(left, bzsl, bzsr);
+    const R sq = sel(left, -sql, sqr);
+    R pts;
+    if constexpr (F64) pts = fma_(sel(left, dl, dr), sm - u0, pt0);
+    else pts = fma_(dl * dr, ur - ul, fma_(dr, ptl, -dl * ptr)) * deni;
+    const R e0 = fma_(p0, gm1i, half * fma_(r0, fma_(u0, u0, fma_(v0, v0, w0 * w0)), b20));
+    const R vb0 = fma_(u0, bn, fma_(v0, by0, w0 * bz0));
+    const R vbs = fma_(sm, bn, fma_(vs, bys, ws * bzs)), vbss = fma_(sm, bn, fma_(vss, byss, wss * bzss));
+    const R es = fma_(su, e0, fma_(-pt0, u0, fma_(pts, sm, bn * (vb0 - vbs)))) * si;
+    const R ess = fma_(sq * sgn, vbs - vbss, es);
+    const R sa = sm + rdiv(rabs(bn), sq);   // Alfven speed of the side (sq < 0 on the left)
+
+    // region: outer (L, R), star or double star
+    const auto outer = sel(left, gl, mnot(ge(S, zero)));
+    const auto dstar = mand(mnot(outer), sel(left, mnot(ge(sa, zero)), ge(sa, zero)));
+    if constexpr (F64) {
+        const R rf = sel(outer, r0, rs), uf = sel(outer, u0, sm), ptf = sel(outer, pt0, pts);
+        const R vf = sel(dstar, vss, sel(outer, v0, vs)), wf = sel(dstar, wss, sel(outer, w0, ws));
+        const R byf = sel(dstar, byss, sel(outer, by0, bys)), bzf = sel(dstar, bzss, sel(outer, bz0, bzs));
+        const R ef = sel(dstar, ess, sel(outer, e0, es)), vbf = sel(dstar, vbss, sel(outer, vb0, vbs));
+        const R m = rf * uf;
+        F[0] = m;
+        F[1] = fma_(m, uf, ptf - bn2);
+        F[2] = fma_(m, vf, -byf * bn);
+        F[3] = fma_(m, wf, -bzf * bn);
+        F[4] = fma_(ef + ptf, uf, -bn * vbf);
+    } else {
+        // flux of the outer state, F* = F + S (U* - U), F** = F* + S* (U** - U*) (the density
+        // and normal momentum of ** are those of *)
+        const R m0 = r0 * u0;
+        const R f0 = m0;
+        const R f1 = fma_(m0, u0, pt0 - bn2);
+        const R f2v = fma_(m0, v0, -by0 * bn);
+        const R f3 = fma_(m0, w0, -bz0 * bn);
+        const R f4 = fma_(e0 + pt0, u0, -bn * vb0);
+        const R us1 = rs * sm, us2 = rs * vs, us3 = rs * ws;
+        const R g0 = fma_(S, rs - r0, f0);
+        const R g1 = fma_(S, us1 - m0, f1);
+        const R g2 = fma_(S, fma_(-r0, v0, us2), f2v);
+        const R g3 = fma_(S, fma_(-r0, w0, us3), f3);
+        const R g4 = fma_(S, es - e0, f4);
+        const R h2 = fma_(sa, fma_(rs, vss, -us2), g2);
+        const R h3 = fma_(sa, fma_(rs, wss, -us3), g3);
+        const R h4 = fma_(sa, ess - es, g4);
+        F[0] = sel(outer, f0, g0);
+        F[1] = sel(outer, f1, g1);
+        F[2] = sel(outer, f2v, sel(dstar, h2, g2));
+        F[3] = sel(outer, f3, sel(dstar, h3, g3));
+        F[4] = sel(outer, f4, sel(dstar, h4, g4));
+    }
 }
 
 // HLL flux (Harten, Lax & van Leer 1983; the simple solver of the paper's mockup, Sec. 2.4)
@@ -282,22 +313,35 @@ template <typename R>
 MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, const Corner<R>& NE, R gamma) {
     R ap[4], am[4], bp[4], bm[4];
     const Corner<R>* st[4] = {&SW, &SE, &NW, &NE};
+    const R g4 = R(4) * gamma;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const Corner<R>& s = *st[k];
-        const R ri = rdiv(R(1), s.rho), gP = gamma * s.p;
-        const R cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
-        const R cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
+        R cfa, cfb;
+        if constexpr (sizeof(R) == 8) {
+            const R hri = R(0.5) * rcp_(s.rho), gP4 = g4 * s.p;
+            const R be2 = s.Be * s.Be;
+            const R ta = fma_(s.Bb, s.Bb, be2), tb = fma_(s.Ba, s.Ba, be2);   // transverse to a, to b
+            const R b2 = fma_(s.Ba, s.Ba, ta);
+            const R sf = fma_(gamma, s.p, b2), df = fma_(gamma, s.p, -b2);
+            const R dd = df * df;
+            cfa = rsqrt_(fast_h(gP4, sf, dd, ta) * hri);
+            cfb = rsqrt_(fast_h(gP4, sf, dd, tb) * hri);
+        } else {   // the rounding of fast_speed (see hlld)
+            const R ri = rcp_(s.rho), gP = gamma * s.p;
+            cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
+            cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
+        }
         ap[k] = s.ua + cfa;
         am[k] = s.ua - cfa;
         bp[k] = s.ub + cfb;
         bm[k] = s.ub - cfb;
     }
     const R zero = R(0);
-    const R sE = fmax_(fmax_(fmax_(ap[0], ap[1]), fmax_(ap[2], ap[3])), zero);
-    const R sW = fmin_(fmin_(fmin_(am[0], am[1]), fmin_(am[2], am[3])), zero);
-    const R sN = fmax_(fmax_(fmax_(bp[0], bp[1]), fmax_(bp[2], bp[3])), zero);
-    const R sS = fmin_(fmin_(fmin_(bm[0], bm[1]), fmin_(bm[2], bm[3])), zero);
+    const R sE = fmax3_(fmax3_(ap[0], ap[1], ap[2]), ap[3], zero);
+    const R sW = fmin3_(fmin3_(am[0], am[1], am[2]), am[3], zero);
+    const R sN = fmax3_(fmax3_(bp[0], bp[1], bp[2]), bp[3], zero);
+    const R sS = fmin3_(fmin3_(bm[0], bm[1], bm[2]), bm[3], zero);
     const R da = sE - sW, db = sN - sS;
     const R eSW = fma_(SW.ua, SW.Bb, -SW.ub * SW.Ba);
     const R eSE = fma_(SE.ua, SE.Bb, -SE.ub * SE.Ba);
@@ -305,7 +349,7 @@ MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, co
     const R eNE = fma_(NE.ua, NE.Bb, -NE.ub * NE.Ba);
     // [S_E (S_N E_SW - S_S E_NW) - S_W (S_N E_SE - S_S E_NE)] / (da db)
     const R num = fma_(sE, fma_(sN, eSW, -sS * eNW), -sW * fma_(sN, eSE, -sS * eNE));
-    const R ida = rdiv(R(1), da), idb = rdiv(R(1), db);
+    const R ida = rcp_(da), idb = rcp_(db);
     return fma_(sE * sW * ida, SE.Bb - SW.Bb, fma_(num * ida, idb, -(sN * sS * idb) * (NW.Ba - SW.Ba)));
 }
 

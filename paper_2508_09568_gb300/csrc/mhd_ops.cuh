@@ -87,6 +87,18 @@ MHD_HD float rdiv(float a, float b) {
 }
 MHD_HD double rdiv(double a, double b) { return a / b; }
 
+// 1 / x.  Single precision on the device: the hardware approximate reciprocal (1 ulp).
+MHD_HD float rcp_(float x) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+MHD_HD double rcp_(double x) { return 1.0 / x; }
+
 // x is finite (tested in its own precision: no conversion to double)
 MHD_HD bool finite_(float x) { return isfinite(x); }
 MHD_HD bool finite_(double x) { return isfinite(x); }
@@ -97,5 +109,45 @@ MHD_HD float fmax_(float a, float b) { return fmaxf(a, b); }
 MHD_HD float fmin_(float a, float b) { return fminf(a, b); }
 MHD_HD double fmax_(double a, double b) { return fmax(a, b); }
 MHD_HD double fmin_(double a, double b) { return fmin(a, b); }
+
+// Larger / smaller of three values (one instruction in single precision on sm_100 and later).
+MHD_HD float fmax3_(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("max.ftz.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+#else
+    return fmaxf(fmaxf(a, b), c);
+#endif
+}
+MHD_HD float fmin3_(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("min.ftz.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+#else
+    return fminf(fminf(a, b), c);
+#endif
+}
+MHD_HD double fmax3_(double a, double b, double c) { return fmax_(fmax_(a, b), c); }
+MHD_HD double fmin3_(double a, double b, double c) { return fmin_(fmin_(a, b), c); }
+
+// minmod(a, b): the argument of smaller magnitude when both have the same sign, else 0, i.e.
+// the median of a, b and 0.
+MHD_HD float minmod_(float a, float b) {
+    return fminf(fmaxf(a, fminf(b, 0.0f)), fmaxf(b, 0.0f));
+}
+MHD_HD double minmod_(double a, double b) {
+#ifdef __CUDA_ARCH__
+    // on the integer pipe (doubles of one sign order as their bits): the FP64 pipe, where a
+    // comparison costs as much as a product, is what bounds the FP64 kernels
+    const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
+    const long long m = 0x7fffffffffffffffll;
+    const long long pick = (ia & m) <= (ib & m) ? ia : ib;
+    return __longlong_as_double((ia ^ ib) < 0 ? 0ll : pick);
+#else
+    return a * b > 0.0 ? (fabs(a) <= fabs(b) ? a : b) : 0.0;
+#endif
+}
 
 }  // namespace mhd

@@ -1,0 +1,48 @@
+"""The 3D step on patches at the edges of its plane staging and of its lane maps: rows too wide for
+the bulk copies (element copies then), rows and volumes that are not multiples of 16 bytes (every
+offset of a staged block), tiles with ragged tails, patches of the smallest extents; every tile
+configuration against the oracle, with the parity bounds of one step, and bitwise the same."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import assert_parity, gpu_bunch, gpu_steps, interior_global, oracle_bunch, oracle_steps, rounded
+from paper_2508_09568_gb300 import capi
+from paper_2508_09568_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# (box, patch): 38 padded columns are the widest row staged in bulk
+SHAPES = {
+    "rows_38": ((32, 9, 4), (32, 9, 4)),
+    "rows_39": ((33, 9, 8), (33, 9, 4)),
+    "wide": ((70, 8, 5), (70, 8, 5)),
+    "odd_volume": ((42, 13, 9), (21, 13, 9)),
+    "odd_rows": ((31, 20, 10), (31, 10, 5)),
+    "smallest": ((6, 6, 6), (3, 3, 3)),
+    "flat_tiles": ((25, 17, 3), (25, 17, 3)),
+}
+
+
+@pytest.mark.parametrize("shape", list(SHAPES))
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32], ids=["f64", "f32"])
+@pytest.mark.parametrize("limiter", [0, 1], ids=["minmod", "mc"])
+def test_step_matches_oracle_in_every_configuration(shape, dtype, limiter):
+    ncell, patch = SHAPES[shape]
+    geom, U, meta = W.small_box(ncell=ncell, patch=patch, seed=31)
+    flat = rounded(W.to_patches(U, geom), dtype)
+    ob = oracle_bunch(geom, meta["gamma"], limiter=limiter, dtype=dtype)
+    dt = ob.cfl_dt(ob.fill_guards(ob.split(flat)))
+    ref = interior_global(oracle_steps(geom, flat, meta["gamma"], [dt], limiter=limiter, dtype=dtype), geom)
+    b = gpu_bunch(geom, flat, meta["gamma"], dtype, limiter=limiter)
+    first = None
+    for cfg in range(b.num_configs()):
+        for mode in (capi.MHD_MODE_PERSISTENT, capi.MHD_MODE_BUNCHED):
+            b.set_mode(mode, cfg)
+            b.upload(flat)
+            got = interior_global(gpu_steps(b, [dt]), geom)
+            if first is None:
+                first = got
+                assert_parity(got, ref, dtype, what=shape)
+            assert np.array_equal(got, first), (shape, cfg, mode)
+    assert b.error()[0] == 0
