@@ -4,15 +4,15 @@
 namespace mhd {
 
 static const StepLaunch kStepF32[] = {
-    StepInst<float, 3, 32, 8, 512>::entry(),
-    StepInst<float, 3, 16, 16, 512>::entry(),
-    StepInst<float, 3, 16, 16, 640>::entry(),
-    StepInst<float, 3, 16, 8, 256, 2>::entry(),
-    StepInst<float, 3, 8, 8, 128, 3>::entry(),
-    StepInst<float, 3, 16, 16, 384>::entry(),
-    StepInst<float, 3, 24, 8, 512>::entry(),
-    StepInst<float, 2, 16, 16, 256>::entry(),
-    StepInst<float, 2, 32, 8, 256>::entry(),
+    StepInst<float, 3, 32, 8, 512>::entry(5.07f, 5.07f),
+    StepInst<float, 3, 16, 16, 512>::entry(5.66f, 5.66f),
+    StepInst<float, 3, 16, 16, 640>::entry(5.32f, 5.32f),
+    StepInst<float, 3, 16, 8, 256, 2>::entry(3.5f, 4.5f),
+    StepInst<float, 3, 8, 8, 128, 3>::entry(2.0f, 3.0f),
+    StepInst<float, 3, 16, 16, 384>::entry(6.1f, 6.1f),
+    StepInst<float, 3, 24, 8, 512>::entry(4.76f, 4.76f),
+    StepInst<float, 2, 16, 16, 256>::entry(4.9f, 11.0f),
+    StepInst<float, 2, 32, 8, 256>::entry(4.35f, 9.5f),
     StepInst<float, 1, 64, 1, 64>::entry(),
 };
 

@@ -4,9 +4,10 @@
 namespace mhd {
 
 static const StepLaunch kStepF64[] = {
-    StepInst<double, 3, 8, 8, 128>::entry(),
-    StepInst<double, 2, 16, 16, 256>::entry(),
-    StepInst<double, 2, 8, 8, 128>::entry(),
+    StepInst<double, 3, 16, 8, 256>::entry(78.0f, 78.0f),
+    StepInst<double, 3, 8, 8, 128>::entry(52.0f, 52.0f),
+    StepInst<double, 2, 16, 16, 256>::entry(122.0f, 128.0f),
+    StepInst<double, 2, 8, 8, 128>::entry(41.5f, 50.0f),
     StepInst<double, 1, 64, 1, 64>::entry(),
 };
 

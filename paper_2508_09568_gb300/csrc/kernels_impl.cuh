@@ -22,6 +22,7 @@ static StepArgs<R> to_args(const StepHostArgs& h) {
     a.patches = h.patches;
     a.tiles = h.tiles;
     a.ntiles = h.ntiles;
+    a.nzb = h.nzb;
     a.ntiles_dev = h.ntiles_dev;
     a.dynamic = h.dynamic;
     a.work = h.work;
@@ -43,11 +44,13 @@ static StepArgs<R> to_args(const StepHostArgs& h) {
 
 // The chunks of a 3D plane shared out to the warps (StepPlan), longest first to the least loaded
 // warp, for every number of in-plane flux chunks moved to phase A; the split with the shortest
-// two phases is taken.  Costs in cycles of a chunk with four
-// warps per scheduler running, measured (FP32, 32x8).
+// two phases is taken.  Costs: cycles of a chunk with four
+// warps per scheduler running, measured (FP32, 32x8); FP64 operations (FP64, bound by that pipe).
 template <typename C>
 static StepPlan make_plan() {
-    constexpr int PREP = 2480, FACE = 1450, EDGE = 1400, CONV = 620, UPD = 700;
+    constexpr bool F64 = C::EQ == 2;
+    constexpr int PREP = F64 ? 330 : 2480, FACE = F64 ? 220 : 1450, EDGE = F64 ? 260 : 1400, CONV = F64 ? 40 : 620,
+                  UPD = F64 ? 45 : 700;
     auto share = [](std::vector<std::pair<int, int>> tasks, StepPlan& P, int phase) {
         std::stable_sort(tasks.begin(), tasks.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
         int load[StepPlan::MAXW] = {}, top = 0;
@@ -100,29 +103,28 @@ struct StepInst {
     static_assert(C::NI + C::NZ + C::IPR::N + C::ICV::N + C::IUP::N < 255 && C::NWARP >= 4 * (NDIM == 3) &&
                       C::NWARP <= StepPlan::MAXW,
                   "chunk numbers are bytes");
+    // whole columns, z-blocks (3D), asynchronous stepping (which may use z-blocks)
+    static constexpr auto whole = &step_kernel<R, NDIM, TX, TY, NT, MINB, false, false>;
+    static constexpr auto split = &step_kernel<R, NDIM, TX, TY, NT, MINB, NDIM == 3, false>;
+    static constexpr auto async = &step_kernel<R, NDIM, TX, TY, NT, MINB, NDIM == 3, true>;
     static cudaError_t prepare() {
-        cudaError_t e = cudaFuncSetAttribute(step_kernel<R, NDIM, TX, TY, NT, MINB, false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
-        if (e != cudaSuccess) return e;
-        return cudaFuncSetAttribute(step_kernel<R, NDIM, TX, TY, NT, MINB, true>,
-                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
+        for (auto k : {whole, split, async}) {
+            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
+            if (e != cudaSuccess) return e;
+        }
+        return cudaSuccess;
     }
     static cudaError_t occupancy(int* blocks) {
-        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, step_kernel<R, NDIM, TX, TY, NT, MINB, false>,
-                                                             NT, C::SMEM_BYTES);
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, whole, NT, C::SMEM_BYTES);
     }
-    // asynchronous stepping (a.slice set) runs its own instantiation
     static cudaError_t launch(const void* args, int grid, cudaStream_t s) {
         const StepArgs<R> a = to_args<R>(*static_cast<const StepHostArgs*>(args));
         static const StepPlan plan = NDIM == 3 ? make_plan<C>() : StepPlan{};
-        if (a.slice)
-            step_kernel<R, NDIM, TX, TY, NT, MINB, true><<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
-        else
-            step_kernel<R, NDIM, TX, TY, NT, MINB, false><<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
+        (a.slice ? async : a.nzb > 1 ? split : whole)<<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
         return cudaGetLastError();
     }
-    static StepLaunch entry() {
-        return StepLaunch{NDIM, C::TX, C::TY, NT, C::SMEM_BYTES, &prepare, &occupancy, &launch};
+    static StepLaunch entry(float plane_us = 1, float alone_us = 1) {
+        return StepLaunch{NDIM, C::TX, C::TY, NT, C::SMEM_BYTES, &prepare, &occupancy, &launch, plane_us, alone_us};
     }
 };
 

@@ -86,6 +86,7 @@ struct mhd_bunch {
         int4* d_nat = nullptr;
         int4* d_lpt = nullptr;
         int n = 0;
+        int nzb = 1;                         // z-blocks of the whole bunch's persistent launch
         std::vector<int4> nat_h;             // host copy of the natural order
         std::vector<int> first, count;   // per patch, in natural order
     };
@@ -142,11 +143,12 @@ struct mhd_bunch {
     cudaStream_t s_in = nullptr, s_out = nullptr;
     std::vector<cudaEvent_t> ev_in, ev_step, ev_out;
     int mode = MHD_MODE_PERSISTENT, config = -1;
+    int auto_config = 0;                 // configuration used when config is -1
     // MHD_MODE_MIXED: per configuration, the tiles (longest first) of the patches whose
     // size class was assigned that configuration by the autotuner (empty: not assigned)
     struct MixedTiles {
         int4* d_tiles = nullptr;
-        int n = 0;
+        int n = 0, nzb = 1;
     };
     std::vector<MixedTiles> mixed;
     // MHD_MODE_BUNCH_LISTS: the bunches of mhd_bunch_set_bunches (patch lists) and, per
@@ -154,7 +156,7 @@ struct mhd_bunch {
     std::vector<int> bunch_patches, bunch_start;
     struct BunchTiles {
         int4* d_tiles = nullptr;
-        std::vector<int> first, count;       // per bunch
+        std::vector<int> first, count, nzb;  // per bunch
     };
     std::vector<BunchTiles> btiles;
     // slab of a z-layer decomposition (mhd_bunch_set_slab): the handle owns layers
@@ -179,12 +181,77 @@ namespace {
 
 bool active(const mhd_bunch* b, int d) { return b->domain[d] > 1; }
 
-int default_config(const mhd_bunch* b) {
-    // first compiled configuration for this dimensionality
-    return b->cfg_index.empty() ? -1 : 0;
+const StepLaunch& step_cfg(const mhd_bunch* b, int k) { return b->K->step[b->cfg_index[k]]; }
+
+int default_config(const mhd_bunch* b) { return b->cfg_index.empty() ? -1 : b->auto_config; }
+
+// Estimated time (microseconds) of a persistent launch over n tiles of nz planes (most planes
+// nzmax) as nzb z-blocks each, on nsm SMs of occ resident CTAs.  A work item costs its planes and
+// the start of the march again (three planes converted, two prepared, one more level of fluxes:
+// about two and a half planes).  Equal items run in waves; otherwise the launch ends half a longest
+// item after an even share.
+double step_time(const StepLaunch& L, int nsm, int occ, int64_t n, double nz, int nzmax, bool equal, int nzb) {
+    const double start = L.ndim == 3 ? 2.5 : 0.0;
+    const double items = (double)n * nzb, slots = (double)nsm * occ;
+    const double item = nz / nzb + start, longest = (double)nzmax / nzb + start;
+    // CTAs that share an SM, and how much longer each takes for it
+    const double share = std::min<double>(occ, std::ceil(items / nsm));
+    const double plane = std::max<double>(L.alone_us, share * L.plane_us);
+    const double waves = equal ? std::ceil(items / slots) : std::max(1.0, items * item / slots / longest + 0.5);
+    return waves * (equal ? item : longest) * plane;
 }
 
-const StepLaunch& step_cfg(const mhd_bunch* b, int k) { return b->K->step[b->cfg_index[k]]; }
+constexpr int kMaxZBlocks = 16;
+
+// z-blocks per tile of a persistent launch over n tiles (3D): more than one where the tiles alone
+// leave SMs idle (a 64^3 box is 32 tiles of 32x8 columns on 152 SMs), at least four planes each
+int z_blocks(const StepLaunch& L, int nsm, int occ, int64_t n, double nz, int nzmin, int nzmax) {
+    if (L.ndim != 3 || n <= 0) return 1;
+    const bool equal = nzmin == nzmax;
+    int best = 1;
+    double least = step_time(L, nsm, occ, n, nz, nzmax, equal, 1);
+    for (int k = 2; k <= kMaxZBlocks && nzmin >= 4 * k; ++k) {
+        const double t = step_time(L, nsm, occ, n, nz, nzmax, equal, k);
+        if (t < 0.97 * least) {
+            least = t;
+            best = k;
+        }
+    }
+    return best;
+}
+
+// planes of the tiles of a launch: their number, mean and largest nz, and whether all are equal
+struct Planes {
+    int64_t n = 0;
+    int64_t sum = 0;
+    int most = 0, least = 1 << 30;
+    void add(int nz) {
+        ++n;
+        sum += nz;
+        most = std::max(most, nz);
+        least = std::min(least, nz);
+    }
+    double mean() const { return n ? (double)sum / (double)n : 0.0; }
+    bool equal() const { return most == least; }
+};
+
+int z_blocks(const mhd_bunch* b, const StepLaunch& L, int occ, const Planes& P) {
+    return z_blocks(L, b->nsm, occ, P.n, P.mean(), P.least, P.most);
+}
+
+// the tiles of configuration k of the patches patches[0..n-1] (null: 0..n-1)
+Planes planes_of(const mhd_bunch* b, int k, const int* patches, int n) {
+    Planes P;
+    for (int i = 0; i < n; ++i) {
+        const int p = patches ? patches[i] : i, nz = b->pn[3 * p + 2];
+        const int c = b->tiles[k].count[p];
+        P.n += c;
+        P.sum += (int64_t)c * nz;
+        P.most = std::max(P.most, nz);
+        P.least = std::min(P.least, nz);
+    }
+    return P;
+}
 
 void free_mixed(mhd_bunch* b) {
     for (auto& m : b->mixed) cudaFree(m.d_tiles);
@@ -340,6 +407,22 @@ int build_tiles(mhd_bunch* b) {
         CK(cudaMemcpy(T.d_nat, nat.data(), sizeof(int4) * T.n, cudaMemcpyHostToDevice));
         CK(cudaMemcpy(T.d_lpt, lpt.data(), sizeof(int4) * T.n, cudaMemcpyHostToDevice));
     }
+    // z-blocks of each configuration's launch over the whole bunch, and the configuration used when
+    // none is set: the shortest by step_time (the first one in 1D and 2D)
+    double least = 0;
+    for (size_t k = 0; k < b->cfg_index.size(); ++k) {
+        const StepLaunch& L = step_cfg(b, (int)k);
+        int occ = 1;
+        CK(L.occupancy(&occ));
+        occ = std::max(occ, 1);
+        const Planes P = planes_of(b, (int)k, nullptr, b->npatch);
+        b->tiles[k].nzb = z_blocks(b, L, occ, P);
+        const double t = step_time(L, b->nsm, occ, P.n, P.mean(), P.most, P.equal(), b->tiles[k].nzb);
+        if (k == 0 || t < least) {
+            least = t;
+            b->auto_config = (int)k;
+        }
+    }
     return MHD_OK;
 }
 
@@ -352,6 +435,7 @@ StepHostArgs step_args(mhd_bunch* b, const double* dt_ptr, double dt_val) {
     a.patches = b->d_patches;
     a.tiles = nullptr;
     a.ntiles = 0;
+    a.nzb = 1;
     a.ntiles_dev = nullptr;
     a.dynamic = 0;
     a.work = b->d_work;
@@ -483,8 +567,9 @@ int do_step(mhd_bunch* b, const double* dt_ptr, double dt_val) {
         for (size_t q = 0; q < BT.count.size(); ++q) {
             a.tiles = BT.d_tiles + BT.first[q];
             a.ntiles = BT.count[q];
+            a.nzb = BT.nzb[q];
             a.dynamic = 1;
-            CK(L.launch(&a, std::min(BT.count[q], b->nsm * occ), b->stream));
+            CK(L.launch(&a, std::min(BT.count[q] * a.nzb, b->nsm * occ), b->stream));
             b->launches++;
         }
     } else if (b->mode == MHD_MODE_MIXED && !b->mixed.empty()) {
@@ -499,17 +584,19 @@ int do_step(mhd_bunch* b, const double* dt_ptr, double dt_val) {
             occ = std::max(occ, 1);
             a.tiles = M.d_tiles;
             a.ntiles = M.n;
+            a.nzb = M.nzb;
             a.dynamic = 1;
-            CK(Lc.launch(&a, std::min(M.n, b->nsm * occ), b->stream));
+            CK(Lc.launch(&a, std::min(M.n * M.nzb, b->nsm * occ), b->stream));
             b->launches++;
         }
     } else {
         int occ = 1;
         CK(L.occupancy(&occ));
         occ = std::max(occ, 1);
-        const int grid = std::min(T.n, b->nsm * occ);
+        const int grid = std::min(T.n * T.nzb, b->nsm * occ);
         a.tiles = T.d_lpt;
         a.ntiles = T.n;
+        a.nzb = T.nzb;
         a.dynamic = 1;
         CK(L.launch(&a, grid, b->stream));
         b->launches++;
@@ -568,10 +655,13 @@ int autotune_mixed(mhd_bunch* b, int* chosen) {
             e = L.occupancy(&occ);
             if (e != cudaSuccess) break;
             StepHostArgs a = step_args(b, nullptr, 0.0);
+            Planes pl;
+            for (const int4& x : tl) pl.add(b->pn[3 * x.x + 2]);
             a.tiles = d_tmp;
             a.ntiles = (int)tl.size();
+            a.nzb = z_blocks(b, L, std::max(occ, 1), pl);
             a.dynamic = 1;
-            const int grid = std::min((int)tl.size(), b->nsm * std::max(occ, 1));
+            const int grid = std::min((int)tl.size() * a.nzb, b->nsm * std::max(occ, 1));
             for (int w = 0; w < 6 && e == cudaSuccess; ++w) {
                 if (w == 2) e = cudaEventRecord(e0, b->stream);
                 if (e == cudaSuccess) e = L.launch(&a, grid, b->stream);
@@ -603,6 +693,11 @@ int autotune_mixed(mhd_bunch* b, int* chosen) {
         CK(cudaMalloc(&b->mixed[c].d_tiles, sizeof(int4) * tl.size()));
         CK(cudaMemcpy(b->mixed[c].d_tiles, tl.data(), sizeof(int4) * tl.size(), cudaMemcpyHostToDevice));
         b->mixed[c].n = (int)tl.size();
+        Planes pl;
+        for (const int4& x : tl) pl.add(b->pn[3 * x.x + 2]);
+        int occ = 1;
+        CK(step_cfg(b, c).occupancy(&occ));
+        b->mixed[c].nzb = z_blocks(b, step_cfg(b, c), std::max(occ, 1), pl);
     }
     if (chosen) *chosen = pick[std::max_element(cells.begin(), cells.end()) - cells.begin()];
     return MHD_OK;
@@ -621,10 +716,18 @@ int do_step_range(mhd_bunch* b, const double* dt_ptr, int p0, int p1) {
     int occ = 1;
     CK(L.occupancy(&occ));
     occ = std::max(occ, 1);
+    Planes pl;
+    for (int p = p0; p < p1; ++p) {
+        pl.n += T.count[p];
+        pl.sum += (int64_t)T.count[p] * b->pn[3 * p + 2];
+        pl.most = std::max(pl.most, b->pn[3 * p + 2]);
+        pl.least = std::min(pl.least, b->pn[3 * p + 2]);
+    }
     a.tiles = T.d_nat + t0;
     a.ntiles = t1 - t0;
+    a.nzb = z_blocks(b, L, occ, pl);
     a.dynamic = 1;
-    CK(L.launch(&a, std::min(t1 - t0, b->nsm * occ), b->stream));
+    CK(L.launch(&a, std::min((t1 - t0) * a.nzb, b->nsm * occ), b->stream));
     b->launches++;
     return MHD_OK;
 }
@@ -1086,6 +1189,10 @@ int mhd_bunch_set_bunches(mhd_bunch* b, const int32_t* patches, const int32_t* s
             std::stable_sort(tl.begin(), tl.end(), [](const int4& x, const int4& y) { return x.w > y.w; });
             BT.first.push_back((int)all.size());
             BT.count.push_back((int)tl.size());
+            int occ = 1;
+            CK(step_cfg(b, (int)k).occupancy(&occ));
+            BT.nzb.push_back(z_blocks(b, step_cfg(b, (int)k), std::max(occ, 1),
+                                      planes_of(b, (int)k, patches + starts[q], starts[q + 1] - starts[q])));
             all.insert(all.end(), tl.begin(), tl.end());
         }
         CK(cudaMalloc(&BT.d_tiles, sizeof(int4) * all.size()));
@@ -1883,7 +1990,11 @@ int mhd_bunch_advance_async(mhd_bunch* b, double t_span, int max_rounds, int* ro
     a.ntiles = T.n;
     a.ntiles_dev = b->d_ntiles;
     a.dynamic = 1;
-    const int step_grid = std::min(T.n, b->nsm * occ);
+    // (a round's z-blocks are chosen in the kernel from its tile count, at least four planes each)
+    int nzmin = 1 << 30;
+    for (int p = 0; p < P; ++p) nzmin = std::min(nzmin, (int)b->pn[3 * p + 2]);
+    a.nzb = b->ndim == 3 ? std::max(1, std::min(kMaxZBlocks, nzmin / 4)) : 1;
+    const int step_grid = std::min(T.n * a.nzb, b->nsm * occ);
     const int list_blocks = std::max(1, 2 * b->nsm);
     // state stride of one patch (equal patches on a regular grid, for the table-driven fill)
     const int64_t pstride = P > 1 ? b->offs[1] - b->offs[0] : (int64_t)(b->state_bytes / b->rb);

@@ -36,6 +36,10 @@ struct StepLaunch {
     cudaError_t (*prepare)();                                   // opt in to large smem
     cudaError_t (*occupancy)(int* blocks_per_sm);
     cudaError_t (*launch)(const void* args, int grid, cudaStream_t s);
+    // time of one plane of a tile per SM, microseconds (measured on a GB300): with every resident CTA
+    // at work, and of a CTA alone on its SM; the default configuration and the number of z-blocks
+    // are chosen by them
+    float plane_us, alone_us;
 };
 
 // arguments of the adjoint step (see mhd_adjoint.cuh), precision independent
@@ -107,6 +111,7 @@ struct StepHostArgs {
     const PatchDev* patches;
     const int4* tiles;
     int ntiles;
+    int nzb;                 // 3D: z-blocks per tile (work items of a persistent launch)
     const int* ntiles_dev;   // asynchronous stepping: tile count read on the device (<= ntiles), or null
     int dynamic;
     int* work;

@@ -57,7 +57,7 @@ MHD_HD R fast_speed(R rho_inv, R gP, R bn, R bt1, R bt2) {
 // faces of the cell (Sec. 2.1 EOS: P = (gamma-1)(E - rho u^2/2 - B^2/2)).
 template <typename R>
 MHD_HD void cons_to_prim(R rho, R mx, R my, R mz, R E, R bxc, R byc, R bzc, R gm1, R q[8]) {
-    const R ri = rdiv(R(1), rho);
+    const R ri = rcp_(rho);
     const R u = mx * ri, v = my * ri, w = mz * ri;
     q[Q_RHO] = rho;
     q[Q_U] = u;
@@ -80,7 +80,7 @@ template <typename R>
 MHD_HD void hancock(const R q[8], const R D[3][8], R hdt, R gamma, R out[5]) {
     const R u = q[Q_U], v = q[Q_V], w = q[Q_W], rho = q[Q_RHO], P = q[Q_P];
     const R divu = D[0][Q_U] + D[1][Q_V] + D[2][Q_W];
-    const R ri = rdiv(R(1), rho);
+    const R ri = rcp_(rho);
     // advective derivative u . grad of primitive k
     auto adv = [&](int k) { return fma_(u, D[0][k], fma_(v, D[1][k], w * D[2][k])); };
     out[0] = rho - hdt * fma_(rho, divu, adv(Q_RHO));
@@ -179,7 +179,7 @@ MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[
     const R rsl = dl * sli, rsr = dr * sri;
     const R Dl = fma_(dl, sml, -bn2), Dr = fma_(dr, smr, -bn2);
     const R epb = eps * bn2;
-    const auto degl = le(rabs(Dl), epb), degr = le(rabs(Dr), epb);
+    const auto degl = le_mag_(rabs(Dl), epb), degr = le_mag_(rabs(Dr), epb);
     const R Dli = sel(degl, zero, rcp_(Dl)), Dri = sel(degr, zero, rcp_(Dr));
     const R nul = bn * (sm - ul) * Dli, nur = bn * (sm - ur) * Dri;   // 0 when degenerate
     const R nbl = sel(degl, R(1), fma_(dl, sul, -bn2) * Dli), nbr = sel(degr, R(1), fma_(dr, sur, -bn2) * Dri);
@@ -200,7 +200,7 @@ MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[
     const R bzss = fma_(sql, bzsr, fma_(sqr, bzsl, sq2 * (wsr - wsl))) * isum;
 
     // the side of x/t = 0 and what is needed of it
-    const auto gl = ge(sl, zero), left = mor(gl, ge(sm, zero));
+    const auto gl = nonneg_(sl), left = mor(gl, nonneg_(sm));
     const R S = sel(left, sl, sr), su = sel(left, sul, sur), si = sel(left, sli, sri);
     const R r0 = sel(left, rl, rr), u0 = sel(left, ul, ur), v0 = sel(left, vl, vr), w0 = sel(left, wl, wr);
     const R p0 = sel(left, pl, pr), by0 = sel(left, byl, byr), bz0 = sel(left, bzl, bzr);
@@ -216,11 +216,14 @@ MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[
     const R vbs = fma_(sm, bn, fma_(vs, bys, ws * bzs)), vbss = fma_(sm, bn, fma_(vss, byss, wss * bzss));
     const R es = fma_(su, e0, fma_(-pt0, u0, fma_(pts, sm, bn * (vb0 - vbs)))) * si;
     const R ess = fma_(sq * sgn, vbs - vbss, es);
-    const R sa = sm + rdiv(rabs(bn), sq);   // Alfven speed of the side (sq < 0 on the left)
+    R sa;   // Alfven speed of the side (sq < 0 on the left)
+    if constexpr (F64) sa = fma_(rabs(bn), rcp_(sq), sm);
+    else sa = sm + rdiv(rabs(bn), sq);
 
     // region: outer (L, R), star or double star
-    const auto outer = sel(left, gl, mnot(ge(S, zero)));
-    const auto dstar = mand(mnot(outer), sel(left, mnot(ge(sa, zero)), ge(sa, zero)));
+    const auto outer = sel(left, gl, mnot(nonneg_(S)));
+    const auto ahead = nonneg_(sa);
+    const auto dstar = mand(mnot(outer), sel(left, mnot(ahead), ahead));
     if constexpr (F64) {
         const R rf = sel(outer, r0, rs), uf = sel(outer, u0, sm), ptf = sel(outer, pt0, pts);
         const R vf = sel(dstar, vss, sel(outer, v0, vs)), wf = sel(dstar, wss, sel(outer, w0, ws));
@@ -272,8 +275,8 @@ MHD_HD void hll(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R F[5]) {
     const R ptl = fma_(half, b2l, pl), ptr = fma_(half, b2r, pr);
     const R el = fma_(pl, gm1i, half * fma_(rl, fma_(ul, ul, fma_(vl, vl, wl * wl)), b2l));
     const R er = fma_(pr, gm1i, half * fma_(rr, fma_(ur, ur, fma_(vr, vr, wr * wr)), b2r));
-    const R cfl = fast_speed(rdiv(R(1), rl), gamma * pl, bn, byl, bzl);
-    const R cfr = fast_speed(rdiv(R(1), rr), gamma * pr, bn, byr, bzr);
+    const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
+    const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
     const R vbl = fma_(ul, bn, fma_(vl, byl, wl * bzl)), vbr = fma_(ur, bn, fma_(vr, byr, wr * bzr));
     const R cmax = fmax_(cfl, cfr);
     const R sl = fmin_(ul, ur) - cmax;
@@ -285,9 +288,9 @@ MHD_HD void hll(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R F[5]) {
                      fma_(el + ptl, ul, -bn * vbl)};
     const R FR[5] = {mr, fma_(mr, ur, ptr - bn2), fma_(mr, vr, -byr * bn), fma_(mr, wr, -bzr * bn),
                      fma_(er + ptr, ur, -bn * vbr)};
-    const R di = rdiv(R(1), sr - sl);
+    const R di = rcp_(sr - sl);
     const R slr = sl * sr;
-    const auto gl = ge(sl, zero), gr = ge(sr, zero);
+    const auto gl = nonneg_(sl), gr = nonneg_(sr);
 #pragma unroll
     for (int c = 0; c < 5; ++c) {
         const R fh = fma_(sr, FL[c], fma_(-sl, FR[c], slr * (UR[c] - UL[c]))) * di;
@@ -337,11 +340,8 @@ MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, co
         bp[k] = s.ub + cfb;
         bm[k] = s.ub - cfb;
     }
-    const R zero = R(0);
-    const R sE = fmax3_(fmax3_(ap[0], ap[1], ap[2]), ap[3], zero);
-    const R sW = fmin3_(fmin3_(am[0], am[1], am[2]), am[3], zero);
-    const R sN = fmax3_(fmax3_(bp[0], bp[1], bp[2]), bp[3], zero);
-    const R sS = fmin3_(fmin3_(bm[0], bm[1], bm[2]), bm[3], zero);
+    const R sE = max0_(ap[0], ap[1], ap[2], ap[3]), sW = min0_(am[0], am[1], am[2], am[3]);
+    const R sN = max0_(bp[0], bp[1], bp[2], bp[3]), sS = min0_(bm[0], bm[1], bm[2], bm[3]);
     const R da = sE - sW, db = sN - sS;
     const R eSW = fma_(SW.ua, SW.Bb, -SW.ub * SW.Ba);
     const R eSE = fma_(SE.ua, SE.Bb, -SE.ub * SE.Ba);

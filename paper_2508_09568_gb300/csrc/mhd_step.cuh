@@ -258,6 +258,7 @@ template <typename R>
 struct Tile {
     PatchDev pt;
     int x0, y0, wx, wy;   // low corner in the patch, columns inside the patch
+    int z0, z1;           // planes updated (the z-block)
     const R* Uc;          // state read
     R* Un;                // state written
     R hdt, dtdx[3];
@@ -514,6 +515,7 @@ struct StepArgs {
     const PatchDev* __restrict__ patches;
     const int4* __restrict__ tiles;
     int ntiles;
+    int nzb;              // 3D: z-blocks of a tile, each a work item (ASYNC: chosen from the tile count)
     const int* ntiles_dev;  // ASYNC: tile count written by the device scheduler (null: ntiles)
     int dynamic;          // 1: pull tiles from *work (persistent), 0: one tile per CTA
     int* work;            // [0] next tile, [1] finished CTAs
@@ -746,9 +748,13 @@ struct ChunkList {
 // on a half-filled pass and whose prep left four of sixteen warps idle.  FP64 is bound by the FP64
 // pipe (see mhd_math.cuh).
 //
+// ZB: work items are z-blocks of tiles (a launch of fewer tiles than SMs: the 64^3 box of 32^3
+// patches, 32 tiles, took 172 us and takes 58); an instantiation of its own, whose block bounds cost
+// the whole-column step 1.5 %.
+//
 // ASYNC: asynchronous stepping (a.slice, a.dt_patch): per-tile slice choice and dt; a
 // separate instantiation so that the synchronous step keeps its kernel-wide constants.
-template <typename R, int NDIM, int TX, int TY, int NT, int MINB, bool ASYNC>
+template <typename R, int NDIM, int TX, int TY, int NT, int MINB, bool ZB, bool ASYNC>
 __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan plan) {
     using C = StepCfg<R, NDIM, TX, TY, NT, MINB>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -775,10 +781,15 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
     }
     __syncthreads();
     int t = s_tile;
-    int ntiles = a.ntiles;
+    int ntiles = a.ntiles, nzb = ZB ? a.nzb : 1;
     if constexpr (ASYNC) {
         if (a.ntiles_dev) ntiles = min(*a.ntiles_dev, a.ntiles);
+        // a round of few tiles: as many z-blocks as fill the grid (a.nzb: the most a patch takes)
+        if constexpr (ZB) nzb = max(1, min(a.nzb, (int)gridDim.x / max(ntiles, 1)));
     }
+    ntiles *= nzb;   // work items: z-block item % nzb of tile item / nzb
+    // first plane of z-block k
+    auto zblock = [&](int nz, int k) { return ZB ? nz * k / nzb : nz * k; };
     // the state that holds U^n of a patch
     auto source = [&](int p) -> const R* {
         if constexpr (ASYNC) return a.slice[p] ? a.Unew : a.U;
@@ -786,16 +797,17 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
     };
     // the first planes of a tile on their way: -2, -1 and 0 into the prep slots, which no phase
     // reads between the last phase A of one tile and the first phase B of the next, 1 into raw
-    auto begin = [&](int tile) {
+    auto begin = [&](int item) {
         if constexpr (C::STAGED) {
-            if (tile < ntiles) {
-                const int4 tl = a.tiles[tile];
+            if (item < ntiles) {
+                const int4 tl = a.tiles[ZB ? item / nzb : item];
                 const PatchDev pt = a.patches[tl.x];
                 const R* U = source(tl.x);
                 const Stage g = stage_of<R, C>(pt, tl.y, tl.z);
+                const int z0 = zblock(pt.nz, ZB ? item % nzb : 0);
                 for (int k = 0; k < 3; ++k)
-                    stage_plane<R, C>(U, pt, g, tl.y, k - 2, S.prep + k * C::RAWN, &s_bar[0], 9 * k);
-                stage_plane<R, C>(U, pt, g, tl.y, 1, S.raw, &s_bar[1], 27);
+                    stage_plane<R, C>(U, pt, g, tl.y, z0 + k - 2, S.prep + k * C::RAWN, &s_bar[0], 9 * k);
+                stage_plane<R, C>(U, pt, g, tl.y, z0 + 1, S.raw, &s_bar[1], 27);
             }
         }
     };
@@ -806,10 +818,12 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
         // what the tile's chunks need of it, in shared memory (they would hold some forty
         // registers through every chunk)
         if (threadIdx.x == 0) {
-            const int4 tl = a.tiles[t];
+            const int4 tl = a.tiles[ZB ? t / nzb : t];
             Tile<R>& T = sT;
             T.pt = a.patches[tl.x];
             T.x0 = tl.y;
+            T.z0 = zblock(T.pt.nz, ZB ? t % nzb : 0);
+            T.z1 = zblock(T.pt.nz, ZB ? t % nzb + 1 : 1);
             T.y0 = tl.z;
             T.wx = min(C::TX, T.pt.nx - tl.y);
             T.wy = C::AY ? min(C::TY, T.pt.ny - tl.z) : 1;
@@ -826,7 +840,7 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
         const Tile<R> T = sT;
 
         if constexpr (C::AZ) {
-            const int nz = T.pt.nz;
+            const int z0 = ZB ? T.z0 : 0, z1 = ZB ? T.z1 : T.pt.nz;
             const bool bulk = C::STAGED && T.g.bulk;
             int tnext = ntiles;
             if constexpr (C::STAGED) {
@@ -839,35 +853,35 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
                 }
             }
             for (int q = wid; q < 3 * C::ICV::N; q += C::NWARP) {
-                const int k = q / C::ICV::N;   // plane k - 2
-                convert_chunk<R, C>(T, S.prep + k * C::RAWN, k - 2, S.W((k + 1) % 3), q - k * C::ICV::N, a.gm1);
+                const int k = q / C::ICV::N;   // plane z0 + k - 2
+                convert_chunk<R, C>(T, S.prep + k * C::RAWN, z0 + k - 2, S.W((z0 + k + 1) % 3), q - k * C::ICV::N, a.gm1);
             }
             __syncthreads();
             auto phase = [&](int c, auto Bc) -> bool {
                 constexpr bool B = decltype(Bc)::value;
                 if (!B) {
-                    if (a.dynamic && c == nz && threadIdx.x == 0) s_tile = atomicAdd(&a.work[0], 1);
-                } else if (c == nz) {
+                    if (a.dynamic && c == z1 && threadIdx.x == 0) s_tile = atomicAdd(&a.work[0], 1);
+                } else if (c == z1) {
                     if (a.dynamic) tnext = s_tile;
                     begin(tnext);
                 } else if constexpr (C::STAGED) {
-                    if (c >= -1 && c + 3 <= nz + 1) stage_plane<R, C>(T.Uc, T.pt, T.g, T.x0, c + 3, S.raw, &s_bar[1], 0);
+                    if (c >= z0 - 1 && c + 3 <= z1 + 1) stage_plane<R, C>(T.Uc, T.pt, T.g, T.x0, c + 3, S.raw, &s_bar[1], 0);
                 }
                 const int ci = B ? c : c - 1;   // plane of the in-plane chunks
                 ChunkList<C::NQ> list(plan.t[B][wid]);
                 bool waited = false;
                 for (int q; (q = list.next()) != 255;) {
                     if (q < C::NI) {
-                        if (ci >= 0 && ci < nz) {
+                        if (ci >= z0 && ci < z1) {
                             if constexpr (B) flux_inplane<R, C>(S.P(ci & 1), S.I(ci & 1), q, a.gamma, a.gm1i, a.eps, a.riemann);
                             else flux_ez<R, C>(S.P(ci & 1), S.I(ci & 1), q - C::IFX::N - C::IFY::N, a.gamma);
                         }
                     } else if (q < C::NI + C::NZ) {
-                        if (c >= 0)
+                        if (c >= z0)
                             flux_interplane<R, C>(S.P((c + 1) & 1), S.P(c & 1), S.Z(c & 1), q - C::NI, a.gamma, a.gm1i,
                                                   a.eps, a.riemann);
                     } else if (q < C::NI + C::NZ + C::IPR::N) {
-                        if (c < nz) {
+                        if (c < z1) {
                             PrepCtx<R, C> X;
                             X.Wm = S.W((c + 3) % 3);
                             X.W0 = S.W((c + 4) % 3);
@@ -878,20 +892,20 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
                             prep_chunk<R, C>(X, S.P((c + 1) & 1), q - C::NI - C::NZ, a.limiter);
                         }
                     } else if (q < C::NI + C::NZ + C::IPR::N + C::ICV::N) {
-                        if (c < nz) {
+                        if (c < z1) {
                             if constexpr (C::STAGED) {
                                 if (bulk && !waited && !mbar_wait(&s_bar[1], par1)) s_fail = 1;
                                 waited = true;
                             }
                             convert_chunk<R, C>(T, S.raw, c + 2, S.W((c + 5) % 3), q - C::NI - C::NZ - C::IPR::N, a.gm1);
                         }
-                    } else if (c >= 1) {
+                    } else if (c > z0) {
                         update_chunk<R, C>(S, T, c - 1, a.err, q - C::NI - C::NZ - C::IPR::N - C::ICV::N);
                     }
                 }
                 if (!B) {
-                    par1 ^= c < nz && bulk;
-                } else if (c == nz) {
+                    par1 ^= c < z1 && bulk;
+                } else if (c == z1) {
                     return true;
                 } else if constexpr (C::STAGED) {
                     if (!bulk) cp_async_wait_all();
@@ -905,9 +919,9 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
                 }
                 return false;
             };
-            if (!phase(-2, std::true_type()))
+            if (!phase(z0 - 2, std::true_type()))
 #pragma unroll 1
-                for (int c = -1; c <= nz; ++c) {
+                for (int c = z0 - 1; c <= z1; ++c) {
                     if (phase(c, std::false_type())) break;
                     if (phase(c, std::true_type())) break;
                 }

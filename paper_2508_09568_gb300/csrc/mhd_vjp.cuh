@@ -511,7 +511,7 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
         const R b2 = bn2 + by * by + bz * bz;
         pt[k] = p + R(0.5) * b2;
         e[k] = p * gm1i + R(0.5) * r * (u * u + v * v + w * w) + R(0.5) * b2;
-        cf[k] = fast_speed(rdiv(R(1), r), gamma * p, bn, by, bz);
+        cf[k] = fast_speed(rcp_(r), gamma * p, bn, by, bz);
         vb[k] = u * bn + v * by + w * bz;
         U[k][0] = r;
         U[k][1] = r * u;
