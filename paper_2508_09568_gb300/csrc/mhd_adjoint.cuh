@@ -14,7 +14,8 @@
 // index, so each thread handles one face or edge; the slope kernel is capped at 128
 // registers and the other cell kernels at 85.
 //
-// Work arrays (fields of one value per padded cell; index coff[p] + (z*Y + y)*X + x):
+// Work arrays (fields of one value per padded cell, index coff[p] + (z*Y + y)*X + x, in blocks of
+// 32 cells, see fat):
 //   W(8) primitives, DW(24) slopes [d][k], FS(6) face-field slopes, EN(3) time-n edge
 //   EMFs, BH(3) predicted low-face fields, WH(8) predicted cell state; and the same 52
 //   fields again for their cotangents.  The state cotangent lives in the output buffer.
@@ -34,8 +35,8 @@ struct AdjArgs {
     const R* U;          // padded U^n with filled ghosts (state layout)
     const R* lam_next;   // cotangent of U^{n+1} (state layout; interior entries used)
     R* lam;              // cotangent of U^n (state layout), accumulated
-    R* F;                // forward work fields [AF_N][ncell]
-    R* G;                // cotangent work fields [AF_N][ncell]
+    R* F;                // forward work fields [(ncell + 31) / 32][AF_N][32]
+    R* G;                // cotangent work fields, likewise
     int64_t ncell;       // cells of all padded patches
     const PatchDev* patches;
     int npatch;
@@ -68,17 +69,26 @@ __device__ __forceinline__ void unit(int d, int& ox, int& oy, int& oz) {
         const int x1 = pt.gx + pt.nx - 1 + (HI), y1 = pt.gy + pt.ny - 1 + (HI),                \
                   z1 = pt.gz + pt.nz - 1 + (HI);                                               \
         const int ex = x1 - x0 + 1, ey = y1 - y0 + 1, ez = z1 - z0 + 1;                        \
-        const int64_t cnt = (int64_t)ex * ey * ez;                                             \
-        for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < cnt;              \
-             k += (int64_t)gridDim.x * blockDim.x) {                                           \
-            const int x = x0 + (int)(k % ex), y = y0 + (int)((k / ex) % ey),                   \
-                      z = z0 + (int)(k / ((int64_t)ex * ey));                                  \
+        /* 32-bit item numbers (the work arrays of 2^31 cells would need 890 GB): the 64-bit       \
+           divisions cost more instructions than some of the kernels' arithmetic */              \
+        const unsigned cnt = (unsigned)ex * ey * ez;                                           \
+        for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < cnt;                      \
+             k += gridDim.x * blockDim.x) {                                                    \
+            const unsigned kr = k / (unsigned)ex, kp = kr / (unsigned)ey;                      \
+            const int x = x0 + (int)(k - kr * ex), y = y0 + (int)(kr - kp * ey),               \
+                      z = z0 + (int)kp;                                                        \
             __VA_ARGS__                                                                        \
         }                                                                                      \
     }
 
+// field f of the cell with index i: blocks of 32 cells, the fields of a block one after the other, so
+// that a warp's access to a field is contiguous and every field of a cell lies at a constant offset
+// from one address (with one array per field each of the 105 accesses of an edge had its own 64-bit
+// address arithmetic)
 template <typename R>
-__device__ __forceinline__ R* fld(R* base, int f, int64_t ncell) { return base + (int64_t)f * ncell; }
+__device__ __forceinline__ R& fat(R* base, int f, int64_t i) {
+    return base[(int64_t)((unsigned)i >> 5) * (AF_N * 32) + f * 32 + ((unsigned)i & 31u)];
+}
 
 // the state variable v of the cell with field index i (state layout: 8 vars per patch)
 template <typename R>
@@ -102,27 +112,31 @@ __global__ void adj_fwd_prim(AdjArgs<R> a) {
         const R bzc = R(0.5) * (u[sidx<R>(pt, C, 7, i)] + u[sidx<R>(pt, C, 7, C.at(x, y, z + 1))]);
         cons_to_prim(u[sidx<R>(pt, C, 0, i)], u[sidx<R>(pt, C, 1, i)], u[sidx<R>(pt, C, 2, i)],
                      u[sidx<R>(pt, C, 3, i)], u[sidx<R>(pt, C, 4, i)], bxc, byc, bzc, gm1, q);
-        for (int v = 0; v < 8; ++v) fld(a.F, AF_W + v, a.ncell)[i] = q[v];
+        for (int v = 0; v < 8; ++v) fat(a.F, AF_W + v, i) = q[v];
     })
 }
 
 template <typename R>
-__global__ void adj_fwd_slopes(AdjArgs<R> a) {
+__global__ void __launch_bounds__(256, 4) adj_fwd_slopes(AdjArgs<R> a) {
     ADJ_FOR_REGION(a, -1, 2, {
         const int64_t i = C.at(x, y, z);
         const bool inner = x <= pt.gx + pt.nx && y <= pt.gy + pt.ny && z <= pt.gz + pt.nz;
+#pragma unroll
         for (int d = 0; d < 3; ++d) {
             int ox, oy, oz;
             unit(d, ox, oy, oz);
             const int64_t im = C.at(x - ox, y - oy, z - oz), ip = C.at(x + ox, y + oy, z + oz);
             if (inner)
                 for (int k = 0; k < 8; ++k) {
-                    const R* w = fld(a.F, AF_W + k, a.ncell);
-                    fld(a.F, AF_DW + 8 * d + k, a.ncell)[i] = limited(w[i] - w[im], w[ip] - w[i], a.limiter);
+                    const R wi = fat(a.F, AF_W + k, i);
+                    fat(a.F, AF_DW + 8 * d + k, i) =
+                        limited(wi - fat(a.F, AF_W + k, im), fat(a.F, AF_W + k, ip) - wi, a.limiter);
                 }
         }
         // transverse slopes of the three low face fields
+#pragma unroll
         for (int c = 0; c < 3; ++c)
+#pragma unroll
             for (int kk = 0; kk < 2; ++kk) {
                 const int t = (c + kk + 1) % 3;
                 int ox, oy, oz;
@@ -130,7 +144,7 @@ __global__ void adj_fwd_slopes(AdjArgs<R> a) {
                 const R bm = a.U[sidx<R>(pt, C, 5 + c, C.at(x - ox, y - oy, z - oz))];
                 const R b0 = a.U[sidx<R>(pt, C, 5 + c, i)];
                 const R bp = a.U[sidx<R>(pt, C, 5 + c, C.at(x + ox, y + oy, z + oz))];
-                fld(a.F, AF_FS + 2 * c + kk, a.ncell)[i] = limited(b0 - bm, bp - b0, a.limiter);
+                fat(a.F, AF_FS + 2 * c + kk, i) = limited(b0 - bm, bp - b0, a.limiter);
             }
     })
 }
@@ -146,10 +160,10 @@ __device__ __forceinline__ R en_value(const AdjArgs<R>& a, const PatchDev& pt, c
     unit(B, bx, by, bz);
     const int64_t c0 = C.at(x, y, z), cA = C.at(x - ax, y - ay, z - az), cB = C.at(x - bx, y - by, z - bz),
                   cAB = C.at(x - ax - bx, y - ay - by, z - az - bz);
-    const R* ua = fld(a.F, AF_W + 1 + A, a.ncell);
-    const R* ub = fld(a.F, AF_W + 1 + B, a.ncell);
-    const R va = R(0.25) * (ua[c0] + ua[cA] + ua[cB] + ua[cAB]);
-    const R vb = R(0.25) * (ub[c0] + ub[cA] + ub[cB] + ub[cAB]);
+    auto mean = [&](int f) {
+        return R(0.25) * (fat(a.F, f, c0) + fat(a.F, f, cA) + fat(a.F, f, cB) + fat(a.F, f, cAB));
+    };
+    const R va = mean(AF_W + 1 + A), vb = mean(AF_W + 1 + B);
     const R Ba = R(0.5) * (a.U[sidx<R>(pt, C, 5 + A, c0)] + a.U[sidx<R>(pt, C, 5 + A, cB)]);
     const R Bb = R(0.5) * (a.U[sidx<R>(pt, C, 5 + B, c0)] + a.U[sidx<R>(pt, C, 5 + B, cA)]);
     if (va_out) {
@@ -165,7 +179,7 @@ template <typename R>
 __global__ void adj_fwd_en(AdjArgs<R> a) {
     ADJ_FOR_REGION(a, -1, 2, {
         const int64_t i = C.at(x, y, z);
-        for (int e = 0; e < 3; ++e) fld(a.F, AF_EN + e, a.ncell)[i] = en_value(a, pt, C, e, x, y, z);
+        for (int e = 0; e < 3; ++e) fat(a.F, AF_EN + e, i) = en_value(a, pt, C, e, x, y, z);
     })
 }
 
@@ -190,21 +204,19 @@ __global__ void adj_fwd_bh(AdjArgs<R> a) {
             int ax, ay, az, bx, by, bz;
             unit(A, ax, ay, az);
             unit(B, bx, by, bz);
-            const R* EA = fld(a.F, AF_EN + A, a.ncell);
-            const R* EB = fld(a.F, AF_EN + B, a.ncell);
             // dB_c/dt = d_A E_B - d_B E_A
-            const R t = hdt * R(a.dxi[A]) * (EB[C.at(x + ax, y + ay, z + az)] - EB[i]) -
-                        hdt * R(a.dxi[B]) * (EA[C.at(x + bx, y + by, z + bz)] - EA[i]);
-            fld(a.F, AF_BH + c, a.ncell)[i] = a.U[sidx<R>(pt, C, 5 + c, i)] + t;
+            const R t = hdt * R(a.dxi[A]) * (fat(a.F, AF_EN + B, C.at(x + ax, y + ay, z + az)) - fat(a.F, AF_EN + B, i)) -
+                        hdt * R(a.dxi[B]) * (fat(a.F, AF_EN + A, C.at(x + bx, y + by, z + bz)) - fat(a.F, AF_EN + A, i));
+            fat(a.F, AF_BH + c, i) = a.U[sidx<R>(pt, C, 5 + c, i)] + t;
         }
     })
 }
 
 template <typename R>
 __device__ __forceinline__ void load_q_D(const AdjArgs<R>& a, int64_t i, R q[8], R D[3][8]) {
-    for (int k = 0; k < 8; ++k) q[k] = fld(a.F, AF_W + k, a.ncell)[i];
+    for (int k = 0; k < 8; ++k) q[k] = fat(a.F, AF_W + k, i);
     for (int d = 0; d < 3; ++d)
-        for (int k = 0; k < 8; ++k) D[d][k] = fld(a.F, AF_DW + 8 * d + k, a.ncell)[i] * R(a.dxi[d]);
+        for (int k = 0; k < 8; ++k) D[d][k] = fat(a.F, AF_DW + 8 * d + k, i) * R(a.dxi[d]);
 }
 
 template <typename R>
@@ -215,12 +227,11 @@ __global__ void adj_fwd_wh(AdjArgs<R> a) {
         R q[8], D[3][8], out[5];
         load_q_D(a, i, q, D);
         hancock(q, D, hdt, gamma, out);
-        for (int k = 0; k < 5; ++k) fld(a.F, AF_WH + k, a.ncell)[i] = out[k];
+        for (int k = 0; k < 5; ++k) fat(a.F, AF_WH + k, i) = out[k];
         for (int c = 0; c < 3; ++c) {
             int ox, oy, oz;
             unit(c, ox, oy, oz);
-            const R* bh = fld(a.F, AF_BH + c, a.ncell);
-            fld(a.F, AF_WH + 5 + c, a.ncell)[i] = R(0.5) * (bh[i] + bh[C.at(x + ox, y + oy, z + oz)]);
+            fat(a.F, AF_WH + 5 + c, i) = R(0.5) * (fat(a.F, AF_BH + c, i) + fat(a.F, AF_BH + c, C.at(x + ox, y + oy, z + oz)));
         }
     })
 }
@@ -230,7 +241,7 @@ __global__ void adj_fwd_wh(AdjArgs<R> a) {
 // ---------------------------------------------------------------------------------------
 template <typename R>
 __device__ __forceinline__ void aadd(R* p, R v) {
-    if (v != R(0)) atomicAdd(p, v);
+    if (nonzero_(v)) atomicAdd(p, v);
 }
 
 // cotangent of U^{n+1} at a state entry if it is an interior cell / owned face, else 0
@@ -252,66 +263,64 @@ __global__ void adj_init(AdjArgs<R> a) {
 
 // faces: the HLLD flux through the low c-face of cells with normal index in [g, g+n] and
 // transverse indices in the interior
-template <typename R>
-__global__ void __launch_bounds__(256, 2) adj_faces(AdjArgs<R> a) {
+template <typename R, int c>
+__device__ __forceinline__ void adj_face(const AdjArgs<R>& a, const PatchDev& pt, const Cell& C, int x, int y, int z) {
+    constexpr int t1 = (c + 1) % 3, t2 = (c + 2) % 3, ox = c == 0, oy = c == 1, oz = c == 2;
+    const int v3[3] = {x, y, z};
+    const int lim[3] = {pt.gx + pt.nx, pt.gy + pt.ny, pt.gz + pt.nz};
+    if (v3[t1] >= lim[t1] || v3[t2] >= lim[t2]) return;
     const R gamma = R(a.gamma), gm1i = R(1.0 / (a.gamma - 1.0)), eps = R(a.eps);
+    const int64_t i = C.at(x, y, z), im = C.at(x - ox, y - oy, z - oz);
+    const R dtdx = R(a.dt * a.dxi[c]);
+    // lF = dt/dx (lam'(cell) - lam'(cell - e_c)) for rho, m_c, m_t1, m_t2, E
+    constexpr int vs[5] = {0, 1 + c, 1 + t1, 1 + t2, 4};
+    R lF[5];
+    bool any = false;
+#pragma unroll
+    for (int n = 0; n < 5; ++n) {
+        lF[n] = dtdx * (lnext(a, pt, C, vs[n], x, y, z) - lnext(a, pt, C, vs[n], x - ox, y - oy, z - oz));
+        any |= nonzero_(lF[n]);
+    }
+    if (!any) return;
+    constexpr int ks[7] = {Q_RHO, Q_U + c, Q_U + t1, Q_U + t2, Q_P, Q_BX + t1, Q_BX + t2};
+    R L[7], Rr[7];
+#pragma unroll
+    for (int n = 0; n < 7; ++n) {
+        L[n] = fat(a.F, AF_WH + ks[n], im) + R(0.5) * fat(a.F, AF_DW + 8 * c + ks[n], im);
+        Rr[n] = fat(a.F, AF_WH + ks[n], i) - R(0.5) * fat(a.F, AF_DW + 8 * c + ks[n], i);
+    }
+    const R bn = fat(a.F, AF_BH + c, i);
+    R lL[7] = {0, 0, 0, 0, 0, 0, 0}, lR[7] = {0, 0, 0, 0, 0, 0, 0}, lbn = R(0);
+    if (a.riemann == 1) hll_vjp(L, Rr, bn, gamma, gm1i, lF, lL, lR, lbn);
+    else hlld_vjp(L, Rr, bn, gamma, gm1i, eps, lF, lL, lR, lbn);
+#pragma unroll
+    for (int n = 0; n < 7; ++n) {
+        aadd(&fat(a.G, AF_WH + ks[n], im), lL[n]);
+        aadd(&fat(a.G, AF_DW + 8 * c + ks[n], im), R(0.5) * lL[n]);
+        aadd(&fat(a.G, AF_WH + ks[n], i), lR[n]);
+        aadd(&fat(a.G, AF_DW + 8 * c + ks[n], i), R(-0.5) * lR[n]);
+    }
+    aadd(&fat(a.G, AF_BH + c, i), lbn);
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2) adj_faces(AdjArgs<R> a) {
+    // face direction: one per grid z-slice
     ADJ_FOR_REGION(a, 0, 1, {
-        const int64_t i = C.at(x, y, z);
-        for (int c = blockIdx.z; c < 3; c += gridDim.z) {   // face direction: one per grid z-slice
-            const int t1 = (c + 1) % 3, t2 = (c + 2) % 3;
-            const int v3[3] = {x, y, z};
-            const int lim[3] = {pt.gx + pt.nx, pt.gy + pt.ny, pt.gz + pt.nz};
-            if (v3[t1] >= lim[t1] || v3[t2] >= lim[t2]) continue;
-            int ox, oy, oz;
-            unit(c, ox, oy, oz);
-            const int64_t im = C.at(x - ox, y - oy, z - oz);
-            const R dtdx = R(a.dt * a.dxi[c]);
-            // lF = dt/dx (lam'(cell) - lam'(cell - e_c)) for rho, m_c, m_t1, m_t2, E
-            const int vs[5] = {0, 1 + c, 1 + t1, 1 + t2, 4};
-            R lF[5];
-            bool any = false;
-            for (int n = 0; n < 5; ++n) {
-                lF[n] = dtdx * (lnext(a, pt, C, vs[n], x, y, z) - lnext(a, pt, C, vs[n], x - ox, y - oy, z - oz));
-                any |= lF[n] != R(0);
-            }
-            if (!any) continue;
-            const int ks[7] = {Q_RHO, Q_U + c, Q_U + t1, Q_U + t2, Q_P, Q_BX + t1, Q_BX + t2};
-            R L[7], Rr[7];
-            for (int n = 0; n < 7; ++n) {
-                const int k = ks[n];
-                L[n] = fld(a.F, AF_WH + k, a.ncell)[im] + R(0.5) * fld(a.F, AF_DW + 8 * c + k, a.ncell)[im];
-                Rr[n] = fld(a.F, AF_WH + k, a.ncell)[i] - R(0.5) * fld(a.F, AF_DW + 8 * c + k, a.ncell)[i];
-            }
-            const R bn = fld(a.F, AF_BH + c, a.ncell)[i];
-            R lL[7] = {0, 0, 0, 0, 0, 0, 0}, lR[7] = {0, 0, 0, 0, 0, 0, 0}, lbn = R(0);
-            if (a.riemann == 1) hll_vjp(L, Rr, bn, gamma, gm1i, lF, lL, lR, lbn);
-            else hlld_vjp(L, Rr, bn, gamma, gm1i, eps, lF, lL, lR, lbn);
-            for (int n = 0; n < 7; ++n) {
-                const int k = ks[n];
-                aadd(&fld(a.G, AF_WH + k, a.ncell)[im], lL[n]);
-                aadd(&fld(a.G, AF_DW + 8 * c + k, a.ncell)[im], R(0.5) * lL[n]);
-                aadd(&fld(a.G, AF_WH + k, a.ncell)[i], lR[n]);
-                aadd(&fld(a.G, AF_DW + 8 * c + k, a.ncell)[i], R(-0.5) * lR[n]);
-            }
-            aadd(&fld(a.G, AF_BH + c, a.ncell)[i], lbn);
-        }
+        if (blockIdx.z == 0) adj_face<R, 0>(a, pt, C, x, y, z);
+        else if (blockIdx.z == 1) adj_face<R, 1>(a, pt, C, x, y, z);
+        else adj_face<R, 2>(a, pt, C, x, y, z);
     })
 }
 
-// corner state (sa, sb) of cell X for edge e, with the a-face / b-face fields it uses
-template <typename R>
-__device__ __forceinline__ Corner<R> adj_corner(const AdjArgs<R>& a, const Cell& C, int e, int X0, int Y0, int Z0,
-                                                int sa, int sb, int64_t& fa, int64_t& fb) {
-    const int A = (e + 1) % 3, B = (e + 2) % 3;
-    int ax, ay, az, bx, by, bz;
-    unit(A, ax, ay, az);
-    unit(B, bx, by, bz);
-    const int64_t i = C.at(X0, Y0, Z0);
-    fa = sa > 0 ? C.at(X0 + ax, Y0 + ay, Z0 + az) : i;   // cell whose low a-face it is
-    fb = sb > 0 ? C.at(X0 + bx, Y0 + by, Z0 + bz) : i;
+// corner state (sa, sb) of the cell with index i for edge e, with the a-face / b-face fields of the
+// cells fa / fb whose low faces they are
+template <typename R, int e, int sa, int sb>
+__device__ __forceinline__ Corner<R> adj_corner(const AdjArgs<R>& a, int64_t i, int64_t fa, int64_t fb) {
+    constexpr int A = (e + 1) % 3, B = (e + 2) % 3;
     auto ext = [&](int k) {
-        return fld(a.F, AF_WH + k, a.ncell)[i] +
-               R(0.5) * (R(sa) * fld(a.F, AF_DW + 8 * A + k, a.ncell)[i] + R(sb) * fld(a.F, AF_DW + 8 * B + k, a.ncell)[i]);
+        return fat(a.F, AF_WH + k, i) +
+               R(0.5) * (R(sa) * fat(a.F, AF_DW + 8 * A + k, i) + R(sb) * fat(a.F, AF_DW + 8 * B + k, i));
     };
     Corner<R> s;
     s.rho = ext(Q_RHO);
@@ -319,98 +328,95 @@ __device__ __forceinline__ Corner<R> adj_corner(const AdjArgs<R>& a, const Cell&
     s.ua = ext(Q_U + A);
     s.ub = ext(Q_U + B);
     s.Be = ext(Q_BX + e);
-    s.Ba = fld(a.F, AF_BH + A, a.ncell)[fa] + R(0.5) * R(sb) * fld(a.F, AF_FS + 2 * A + 0, a.ncell)[fa];
-    s.Bb = fld(a.F, AF_BH + B, a.ncell)[fb] + R(0.5) * R(sa) * fld(a.F, AF_FS + 2 * B + 1, a.ncell)[fb];
+    s.Ba = fat(a.F, AF_BH + A, fa) + R(0.5) * R(sb) * fat(a.F, AF_FS + 2 * A + 0, fa);
+    s.Bb = fat(a.F, AF_BH + B, fb) + R(0.5) * R(sa) * fat(a.F, AF_FS + 2 * B + 1, fb);
     return s;
 }
 
-template <typename R>
-__device__ __forceinline__ void adj_corner_scatter(const AdjArgs<R>& a, const Cell& C, int e, int X0, int Y0, int Z0,
-                                                   int sa, int sb, int64_t fa, int64_t fb, const Corner<R>& g) {
-    const int A = (e + 1) % 3, B = (e + 2) % 3;
-    const int64_t i = C.at(X0, Y0, Z0);
-    const int ks[5] = {Q_RHO, Q_P, Q_U + A, Q_U + B, Q_BX + e};
+template <typename R, int e, int sa, int sb>
+__device__ __forceinline__ void adj_corner_scatter(const AdjArgs<R>& a, int64_t i, int64_t fa, int64_t fb,
+                                                   const Corner<R>& g) {
+    constexpr int A = (e + 1) % 3, B = (e + 2) % 3;
+    constexpr int ks[5] = {Q_RHO, Q_P, Q_U + A, Q_U + B, Q_BX + e};
     const R gv[5] = {g.rho, g.p, g.ua, g.ub, g.Be};
+#pragma unroll
     for (int n = 0; n < 5; ++n) {
-        aadd(&fld(a.G, AF_WH + ks[n], a.ncell)[i], gv[n]);
-        aadd(&fld(a.G, AF_DW + 8 * A + ks[n], a.ncell)[i], R(0.5) * R(sa) * gv[n]);
-        aadd(&fld(a.G, AF_DW + 8 * B + ks[n], a.ncell)[i], R(0.5) * R(sb) * gv[n]);
+        aadd(&fat(a.G, AF_WH + ks[n], i), gv[n]);
+        aadd(&fat(a.G, AF_DW + 8 * A + ks[n], i), R(0.5 * sa) * gv[n]);
+        aadd(&fat(a.G, AF_DW + 8 * B + ks[n], i), R(0.5 * sb) * gv[n]);
     }
-    aadd(&fld(a.G, AF_BH + A, a.ncell)[fa], g.Ba);
-    aadd(&fld(a.G, AF_FS + 2 * A + 0, a.ncell)[fa], R(0.5) * R(sb) * g.Ba);
-    aadd(&fld(a.G, AF_BH + B, a.ncell)[fb], g.Bb);
-    aadd(&fld(a.G, AF_FS + 2 * B + 1, a.ncell)[fb], R(0.5) * R(sa) * g.Bb);
+    aadd(&fat(a.G, AF_BH + A, fa), g.Ba);
+    aadd(&fat(a.G, AF_FS + 2 * A + 0, fa), R(0.5 * sb) * g.Ba);
+    aadd(&fat(a.G, AF_BH + B, fb), g.Bb);
+    aadd(&fat(a.G, AF_FS + 2 * B + 1, fb), R(0.5 * sa) * g.Bb);
 }
 
 // edges: the 2D HLL EMF on the edge low in (a, b) of cells with a, b indices in [g, g+n]
 // and the e index in the interior
+template <typename R, int e>
+__device__ __forceinline__ void adj_edge(const AdjArgs<R>& a, const PatchDev& pt, const Cell& C, int x, int y, int z) {
+    constexpr int A = (e + 1) % 3, B = (e + 2) % 3;
+    constexpr int ax = A == 0, ay = A == 1, az = A == 2, bx = B == 0, by = B == 1, bz = B == 2;
+    const int v3[3] = {x, y, z};
+    const int lim[3] = {pt.gx + pt.nx, pt.gy + pt.ny, pt.gz + pt.nz};
+    if (v3[e] >= lim[e]) return;
+    // lE = dt/dx_B (lam_A(cell - e_B) - lam_A(cell)) + dt/dx_A (lam_B(cell) - lam_B(cell - e_A))
+    const R lE = R(a.dt * a.dxi[B]) * (lnext(a, pt, C, 5 + A, x - bx, y - by, z - bz) - lnext(a, pt, C, 5 + A, x, y, z)) +
+                 R(a.dt * a.dxi[A]) * (lnext(a, pt, C, 5 + B, x, y, z) - lnext(a, pt, C, 5 + B, x - ax, y - ay, z - az));
+    if (!nonzero_(lE)) return;
+    // SW = (-a,-b) corner (+,+); SE = (-b) corner (-,+); NW = (-a) corner (+,-); NE = cell (-,-)
+    const int64_t NE = C.at(x, y, z), NW = C.at(x - ax, y - ay, z - az), SE = C.at(x - bx, y - by, z - bz),
+                  SW = C.at(x - ax - bx, y - ay - by, z - az - bz);
+    const Corner<R> s0 = adj_corner<R, e, 1, 1>(a, SW, SE, NW), s1 = adj_corner<R, e, -1, 1>(a, SE, SE, NE),
+                    s2 = adj_corner<R, e, 1, -1>(a, NW, NE, NW), s3 = adj_corner<R, e, -1, -1>(a, NE, NE, NE);
+    Corner<R> g0{0, 0, 0, 0, 0, 0, 0}, g1{0, 0, 0, 0, 0, 0, 0}, g2{0, 0, 0, 0, 0, 0, 0}, g3{0, 0, 0, 0, 0, 0, 0};
+    emf2d_vjp(s0, s1, s2, s3, R(a.gamma), lE, g0, g1, g2, g3);
+    adj_corner_scatter<R, e, 1, 1>(a, SW, SE, NW, g0);
+    adj_corner_scatter<R, e, -1, 1>(a, SE, SE, NE, g1);
+    adj_corner_scatter<R, e, 1, -1>(a, NW, NE, NW, g2);
+    adj_corner_scatter<R, e, -1, -1>(a, NE, NE, NE, g3);
+}
+
 template <typename R>
-__global__ void __launch_bounds__(256, 2) adj_edges(AdjArgs<R> a) {
-    const R gamma = R(a.gamma);
+__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 1 : 2) adj_edges(AdjArgs<R> a) {
+    // edge direction: one per grid z-slice
     ADJ_FOR_REGION(a, 0, 1, {
-        for (int e = blockIdx.z; e < 3; e += gridDim.z) {   // edge direction: one per grid z-slice
-            const int A = (e + 1) % 3, B = (e + 2) % 3;
-            const int v3[3] = {x, y, z};
-            const int lim[3] = {pt.gx + pt.nx, pt.gy + pt.ny, pt.gz + pt.nz};
-            if (v3[e] >= lim[e]) continue;
-            int ax, ay, az, bx, by, bz;
-            unit(A, ax, ay, az);
-            unit(B, bx, by, bz);
-            // lE = dt/dx_B (lam_A(cell - e_B) - lam_A(cell)) + dt/dx_A (lam_B(cell) - lam_B(cell - e_A))
-            const R lE = R(a.dt * a.dxi[B]) * (lnext(a, pt, C, 5 + A, x - bx, y - by, z - bz) -
-                                               lnext(a, pt, C, 5 + A, x, y, z)) +
-                         R(a.dt * a.dxi[A]) * (lnext(a, pt, C, 5 + B, x, y, z) -
-                                               lnext(a, pt, C, 5 + B, x - ax, y - ay, z - az));
-            if (lE == R(0)) continue;
-            // SW = (-a,-b) corner (+,+); SE = (-b) corner (-,+); NW = (-a) corner (+,-); NE = cell (-,-)
-            int64_t fa[4], fb[4];
-            const int cx[4] = {x - ax - bx, x - bx, x - ax, x};
-            const int cy[4] = {y - ay - by, y - by, y - ay, y};
-            const int cz[4] = {z - az - bz, z - bz, z - az, z};
-            const int sa[4] = {1, -1, 1, -1}, sb[4] = {1, 1, -1, -1};
-            Corner<R> s[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) s[k] = adj_corner(a, C, e, cx[k], cy[k], cz[k], sa[k], sb[k], fa[k], fb[k]);
-            Corner<R> g[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) g[k] = Corner<R>{0, 0, 0, 0, 0, 0, 0};
-            emf2d_vjp(s[0], s[1], s[2], s[3], gamma, lE, g[0], g[1], g[2], g[3]);
-#pragma unroll
-            for (int k = 0; k < 4; ++k) adj_corner_scatter(a, C, e, cx[k], cy[k], cz[k], sa[k], sb[k], fa[k], fb[k], g[k]);
-        }
+        if (blockIdx.z == 0) adj_edge<R, 0>(a, pt, C, x, y, z);
+        else if (blockIdx.z == 1) adj_edge<R, 1>(a, pt, C, x, y, z);
+        else adj_edge<R, 2>(a, pt, C, x, y, z);
     })
 }
 
 // predictor: lWH -> lW, lDW (Hancock) and lBH (cell-centred predicted field = face mean)
 template <typename R>
-__global__ void __launch_bounds__(256, 3) adj_pred(AdjArgs<R> a) {
+__global__ void __launch_bounds__(256, sizeof(R) == 8 ? 2 : 3) adj_pred(AdjArgs<R> a) {
     const R hdt = R(0.5 * a.dt), gamma = R(a.gamma);
     ADJ_FOR_REGION(a, -1, 1, {
         const int64_t i = C.at(x, y, z);
         R lo[5], lb[3];
         bool any = false;
         for (int k = 0; k < 5; ++k) {
-            lo[k] = fld(a.G, AF_WH + k, a.ncell)[i];
-            any |= lo[k] != R(0);
+            lo[k] = fat(a.G, AF_WH + k, i);
+            any |= nonzero_(lo[k]);
         }
-        for (int c = 0; c < 3; ++c) lb[c] = fld(a.G, AF_WH + 5 + c, a.ncell)[i];   // before any atomic add
+        for (int c = 0; c < 3; ++c) lb[c] = fat(a.G, AF_WH + 5 + c, i);   // before any atomic add
         if (any) {
             R q[8], D[3][8], lq[8] = {0, 0, 0, 0, 0, 0, 0, 0}, lD[3][8];
             for (int d = 0; d < 3; ++d)
                 for (int k = 0; k < 8; ++k) lD[d][k] = R(0);
             load_q_D(a, i, q, D);
             hancock_vjp(q, D, hdt, gamma, lo, lq, lD);
-            for (int k = 0; k < 8; ++k) aadd(&fld(a.G, AF_W + k, a.ncell)[i], lq[k]);
+            for (int k = 0; k < 8; ++k) aadd(&fat(a.G, AF_W + k, i), lq[k]);
             for (int d = 0; d < 3; ++d)
-                for (int k = 0; k < 8; ++k) aadd(&fld(a.G, AF_DW + 8 * d + k, a.ncell)[i], lD[d][k] * R(a.dxi[d]));
+                for (int k = 0; k < 8; ++k) aadd(&fat(a.G, AF_DW + 8 * d + k, i), lD[d][k] * R(a.dxi[d]));
         }
         for (int c = 0; c < 3; ++c) {
             const R l = lb[c];
-            if (l == R(0)) continue;
+            if (!nonzero_(l)) continue;
             int ox, oy, oz;
             unit(c, ox, oy, oz);
-            aadd(&fld(a.G, AF_BH + c, a.ncell)[i], R(0.5) * l);
-            aadd(&fld(a.G, AF_BH + c, a.ncell)[C.at(x + ox, y + oy, z + oz)], R(0.5) * l);
+            aadd(&fat(a.G, AF_BH + c, i), R(0.5) * l);
+            aadd(&fat(a.G, AF_BH + c, C.at(x + ox, y + oy, z + oz)), R(0.5) * l);
         }
     })
 }
@@ -423,18 +429,18 @@ __global__ void __launch_bounds__(256, 3) adj_bh(AdjArgs<R> a) {
         const int64_t i = C.at(x, y, z);
         for (int c = 0; c < 3; ++c) {
             if (!bh_region(pt, c, x, y, z)) continue;
-            const R l = fld(a.G, AF_BH + c, a.ncell)[i];
-            if (l == R(0)) continue;
+            const R l = fat(a.G, AF_BH + c, i);
+            if (!nonzero_(l)) continue;
             const int A = (c + 1) % 3, B = (c + 2) % 3;
             int ax, ay, az, bx, by, bz;
             unit(A, ax, ay, az);
             unit(B, bx, by, bz);
             aadd(&a.lam[sidx<R>(pt, C, 5 + c, i)], l);
             const R kA = hdt * R(a.dxi[A]) * l, kB = hdt * R(a.dxi[B]) * l;
-            aadd(&fld(a.G, AF_EN + B, a.ncell)[C.at(x + ax, y + ay, z + az)], kA);
-            aadd(&fld(a.G, AF_EN + B, a.ncell)[i], -kA);
-            aadd(&fld(a.G, AF_EN + A, a.ncell)[C.at(x + bx, y + by, z + bz)], -kB);
-            aadd(&fld(a.G, AF_EN + A, a.ncell)[i], kB);
+            aadd(&fat(a.G, AF_EN + B, C.at(x + ax, y + ay, z + az)), kA);
+            aadd(&fat(a.G, AF_EN + B, i), -kA);
+            aadd(&fat(a.G, AF_EN + A, C.at(x + bx, y + by, z + bz)), -kB);
+            aadd(&fat(a.G, AF_EN + A, i), kB);
         }
     })
 }
@@ -445,8 +451,8 @@ __global__ void __launch_bounds__(256, 3) adj_en(AdjArgs<R> a) {
     ADJ_FOR_REGION(a, -1, 2, {
         const int64_t i = C.at(x, y, z);
         for (int e = 0; e < 3; ++e) {
-            const R l = fld(a.G, AF_EN + e, a.ncell)[i];
-            if (l == R(0)) continue;
+            const R l = fat(a.G, AF_EN + e, i);
+            if (!nonzero_(l)) continue;
             const int A = (e + 1) % 3, B = (e + 2) % 3;
             int ax, ay, az, bx, by, bz;
             unit(A, ax, ay, az);
@@ -456,8 +462,8 @@ __global__ void __launch_bounds__(256, 3) adj_en(AdjArgs<R> a) {
             const int64_t cs[4] = {i, C.at(x - ax, y - ay, z - az), C.at(x - bx, y - by, z - bz),
                                    C.at(x - ax - bx, y - ay - by, z - az - bz)};
             for (int k = 0; k < 4; ++k) {
-                aadd(&fld(a.G, AF_W + 1 + A, a.ncell)[cs[k]], R(0.25) * l * Bb);
-                aadd(&fld(a.G, AF_W + 1 + B, a.ncell)[cs[k]], R(-0.25) * l * Ba);
+                aadd(&fat(a.G, AF_W + 1 + A, cs[k]), R(0.25) * l * Bb);
+                aadd(&fat(a.G, AF_W + 1 + B, cs[k]), R(-0.25) * l * Ba);
             }
             aadd(&a.lam[sidx<R>(pt, C, 5 + B, i)], R(0.5) * l * va);
             aadd(&a.lam[sidx<R>(pt, C, 5 + B, cs[1])], R(0.5) * l * va);
@@ -484,21 +490,19 @@ __global__ void __launch_bounds__(256, 2) adj_slopes(AdjArgs<R> a) {
                 R l[8], wm[8], w0[8], wp[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    const R* w = fld(a.F, AF_W + k, a.ncell);
-                    l[k] = fld(a.G, AF_DW + 8 * d + k, a.ncell)[i];
-                    wm[k] = w[im];
-                    w0[k] = w[i];
-                    wp[k] = w[ip];
+                    l[k] = fat(a.G, AF_DW + 8 * d + k, i);
+                    wm[k] = fat(a.F, AF_W + k, im);
+                    w0[k] = fat(a.F, AF_W + k, i);
+                    wp[k] = fat(a.F, AF_W + k, ip);
                 }
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    if (l[k] == R(0)) continue;
+                    if (!nonzero_(l[k])) continue;
                     R lm = 0, l0 = 0, lp = 0;
                     slope_vjp(wm[k], w0[k], wp[k], a.limiter, l[k], lm, l0, lp);
-                    R* gw = fld(a.G, AF_W + k, a.ncell);
-                    aadd(&gw[im], lm);
-                    aadd(&gw[i], l0);
-                    aadd(&gw[ip], lp);
+                    aadd(&fat(a.G, AF_W + k, im), lm);
+                    aadd(&fat(a.G, AF_W + k, i), l0);
+                    aadd(&fat(a.G, AF_W + k, ip), lp);
                 }
             }
         R lf[6], um[6], u0[6], up[6];
@@ -511,14 +515,14 @@ __global__ void __launch_bounds__(256, 2) adj_slopes(AdjArgs<R> a) {
             unit(t, ox, oy, oz);
             fim[f] = C.at(x - ox, y - oy, z - oz);
             fip[f] = C.at(x + ox, y + oy, z + oz);
-            lf[f] = fld(a.G, AF_FS + f, a.ncell)[i];
+            lf[f] = fat(a.G, AF_FS + f, i);
             um[f] = a.U[sidx<R>(pt, C, 5 + c, fim[f])];
             u0[f] = a.U[sidx<R>(pt, C, 5 + c, i)];
             up[f] = a.U[sidx<R>(pt, C, 5 + c, fip[f])];
         }
 #pragma unroll
         for (int f = 0; f < 6; ++f) {
-            if (lf[f] == R(0)) continue;
+            if (!nonzero_(lf[f])) continue;
             const int c = f >> 1;
             R lm = 0, l0 = 0, lp = 0;
             slope_vjp(um[f], u0[f], up[f], a.limiter, lf[f], lm, l0, lp);
@@ -538,8 +542,8 @@ __global__ void __launch_bounds__(256, 3) adj_prim(AdjArgs<R> a) {
         R lq[8];
         bool any = false;
         for (int k = 0; k < 8; ++k) {
-            lq[k] = fld(a.G, AF_W + k, a.ncell)[i];
-            any |= lq[k] != R(0);
+            lq[k] = fat(a.G, AF_W + k, i);
+            any |= nonzero_(lq[k]);
         }
         if (!any) continue;
         const R* u = a.U;
@@ -592,7 +596,7 @@ __global__ void adj_fill_transpose(R* lam, const PatchDev* __restrict__ patches,
 #pragma unroll
             for (int v = 0; v < 8; ++v) {
                 d[v * vol] = R(0);
-                if (g[v] != R(0)) atomicAdd(&s[v * svol], g[v]);
+                if (nonzero_(g[v])) atomicAdd(&s[v * svol], g[v]);
             }
         }
     }
@@ -633,7 +637,7 @@ __global__ void adj_fill_transpose_grid(R* lam, const PatchDev* __restrict__ pat
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
             d[v * vol] = R(0);
-            if (g[v] != R(0)) atomicAdd(&s[v * vol], g[v]);
+            if (nonzero_(g[v])) atomicAdd(&s[v * vol], g[v]);
         }
     }
 }

@@ -2155,7 +2155,7 @@ extern "C" int mhd_bunch_step_adjoint(mhd_bunch* b, double dt, const void* U_n, 
     if (b->ndim != 3) return fail(MHD_EINVAL, "the adjoint is implemented for 3D bunches");
     if (lam == lam_next || lam == U_n) return fail(MHD_EINVAL, "lam must not alias U_n or lam_next");
     const int64_t ncell = (int64_t)(b->state_bytes / b->rb) / 8;
-    const size_t fbytes = (size_t)b->K->adj_fields * (size_t)ncell * b->rb;
+    const size_t fbytes = (size_t)b->K->adj_fields * (size_t)((ncell + 31) / 32 * 32) * b->rb;
     if (!b->d_adjF) {
         // library-owned work arrays, kept for later calls (released by mhd_bunch_destroy)
         cudaError_t e = cudaMalloc(&b->d_adjF, fbytes);

@@ -306,6 +306,25 @@ struct Corner {
     R rho, p, ua, ub, Ba, Bb, Be;
 };
 
+// fast speeds of a corner state along a and b
+template <typename R>
+MHD_HD void corner_speeds(const Corner<R>& s, R gamma, R& cfa, R& cfb) {
+    if constexpr (sizeof(R) == 8) {
+        const R hri = R(0.5) * rcp_(s.rho), gP4 = R(4) * gamma * s.p;
+        const R be2 = s.Be * s.Be;
+        const R ta = fma_(s.Bb, s.Bb, be2), tb = fma_(s.Ba, s.Ba, be2);   // transverse to a, to b
+        const R b2 = fma_(s.Ba, s.Ba, ta);
+        const R sf = fma_(gamma, s.p, b2), df = fma_(gamma, s.p, -b2);
+        const R dd = df * df;
+        cfa = rsqrt_(fast_h(gP4, sf, dd, ta) * hri);
+        cfb = rsqrt_(fast_h(gP4, sf, dd, tb) * hri);
+    } else {   // the rounding of fast_speed (see hlld)
+        const R ri = rcp_(s.rho), gP = gamma * s.p;
+        cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
+        cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
+    }
+}
+
 // Two-dimensional HLL upwind EMF at an edge from the four corner states SW, SE, NW, NE
 // (E/W along a, N/S along b), with E_e = ua*Bb - ub*Ba per state:
 // E = [S_E S_N E_SW - S_E S_S E_NW - S_W S_N E_SE + S_W S_S E_NE] / ((S_E-S_W)(S_N-S_S))
@@ -316,25 +335,11 @@ template <typename R>
 MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, const Corner<R>& NE, R gamma) {
     R ap[4], am[4], bp[4], bm[4];
     const Corner<R>* st[4] = {&SW, &SE, &NW, &NE};
-    const R g4 = R(4) * gamma;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const Corner<R>& s = *st[k];
         R cfa, cfb;
-        if constexpr (sizeof(R) == 8) {
-            const R hri = R(0.5) * rcp_(s.rho), gP4 = g4 * s.p;
-            const R be2 = s.Be * s.Be;
-            const R ta = fma_(s.Bb, s.Bb, be2), tb = fma_(s.Ba, s.Ba, be2);   // transverse to a, to b
-            const R b2 = fma_(s.Ba, s.Ba, ta);
-            const R sf = fma_(gamma, s.p, b2), df = fma_(gamma, s.p, -b2);
-            const R dd = df * df;
-            cfa = rsqrt_(fast_h(gP4, sf, dd, ta) * hri);
-            cfb = rsqrt_(fast_h(gP4, sf, dd, tb) * hri);
-        } else {   // the rounding of fast_speed (see hlld)
-            const R ri = rcp_(s.rho), gP = gamma * s.p;
-            cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
-            cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
-        }
+        corner_speeds(s, gamma, cfa, cfb);
         ap[k] = s.ua + cfa;
         am[k] = s.ua - cfa;
         bp[k] = s.ub + cfb;

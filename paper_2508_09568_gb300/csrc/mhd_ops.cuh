@@ -71,6 +71,45 @@ MHD_HD bool le_mag_(double a, double b) {
     return a <= b;
 #endif
 }
+// x != 0; x > 0 (a NaN passes or fails as its bits say: it stays one in what follows); a > b
+MHD_HD bool nonzero_(float x) { return x != 0.0f; }
+MHD_HD bool positive_(float x) { return x > 0.0f; }
+MHD_HD bool greater_(float a, float b) { return a > b; }
+MHD_HD bool nonzero_(double x) {
+#ifdef __CUDA_ARCH__
+    return (__double_as_longlong(x) << 1) != 0;
+#else
+    return x != 0.0;
+#endif
+}
+MHD_HD bool positive_(double x) {
+#ifdef __CUDA_ARCH__
+    return __double_as_longlong(x) > 0;
+#else
+    return x > 0.0;
+#endif
+}
+#ifdef __CUDA_ARCH__
+// bits of a double ordered as the values (and back)
+__device__ __forceinline__ long long order_(long long i) { return i ^ (long long)((unsigned long long)(i >> 63) >> 1); }
+#endif
+MHD_HD bool greater_(double a, double b) {
+#ifdef __CUDA_ARCH__
+    return order_(__double_as_longlong(a)) > order_(__double_as_longlong(b));
+#else
+    return a > b;
+#endif
+}
+// a and b of the same sign and neither 0 (a b > 0, without the product's underflow in double)
+MHD_HD bool same_sign_(float a, float b) { return a * b > 0.0f; }
+MHD_HD bool same_sign_(double a, double b) {
+#ifdef __CUDA_ARCH__
+    const long long i = __double_as_longlong(a), j = __double_as_longlong(b);
+    return (i ^ j) >= 0 && (i << 1) != 0 && (j << 1) != 0;
+#else
+    return a * b > 0.0;
+#endif
+}
 MHD_HD bool mand(bool a, bool b) { return a && b; }
 MHD_HD bool mor(bool a, bool b) { return a || b; }
 MHD_HD bool mnot(bool a) { return !a; }
@@ -158,10 +197,6 @@ MHD_HD bool finite_(double x) { return isfinite(x); }
 // are checked for finiteness where they are written).
 MHD_HD float fmax_(float a, float b) { return fmaxf(a, b); }
 MHD_HD float fmin_(float a, float b) { return fminf(a, b); }
-#ifdef __CUDA_ARCH__
-// bits of a double ordered as the values (and back)
-__device__ __forceinline__ long long order_(long long i) { return i ^ (long long)((unsigned long long)(i >> 63) >> 1); }
-#endif
 MHD_HD double fmax_(double a, double b) {
 #ifdef __CUDA_ARCH__
     return order_(__double_as_longlong(a)) >= order_(__double_as_longlong(b)) ? a : b;

@@ -17,15 +17,15 @@ namespace mhd {
 // d limited(a, b): lo -> la, lb
 template <typename R>
 MHD_HD void limited_vjp(R a, R b, int limiter, R lo, R& la, R& lb) {
-    if (!(a * b > R(0))) return;
+    if (!same_sign_(a, b)) return;
     if (limiter == 0) {
-        if (rabs(a) <= rabs(b)) la += lo;
+        if (le_mag_(rabs(a), rabs(b))) la += lo;
         else lb += lo;
     } else {
         const R c = R(0.5) * (a + b);
-        const bool pa = rabs(R(2) * a) <= rabs(R(2) * b);
+        const bool pa = le_mag_(rabs(a), rabs(b));
         const R m2 = pa ? R(2) * a : R(2) * b;
-        if (rabs(c) <= rabs(m2)) {
+        if (le_mag_(rabs(c), rabs(m2))) {
             la += R(0.5) * lo;
             lb += R(0.5) * lo;
         } else if (pa) {
@@ -50,7 +50,7 @@ MHD_HD void slope_vjp(R qm, R q0, R qp, int limiter, R lo, R& lqm, R& lq0, R& lq
 template <typename R>
 MHD_HD void fast_speed_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R lcf, R& lrho, R& lP, R& lbn, R& lbt1,
                            R& lbt2) {
-    const R ri = R(1) / rho;
+    const R ri = rcp_(rho);
     const R cs2 = gamma * P * ri;
     const R can2 = bn * bn * ri;
     const R cat2 = (bt1 * bt1 + bt2 * bt2) * ri;
@@ -59,9 +59,8 @@ MHD_HD void fast_speed_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R lcf, R& lr
     const R s = rsqrt_(disc);
     const R h = R(0.5) * (cs2 + can2 + cat2 + s);
     const R cf = rsqrt_(h);
-    const R lh = cf > R(0) ? lcf / (R(2) * cf) : R(0);
-    const R ls = R(0.5) * lh;
-    const R ldisc = disc > R(0) ? ls / (R(2) * s) : R(0);
+    const R lh = positive_(cf) ? R(0.5) * lcf * rcp_(cf) : R(0);
+    const R ldisc = positive_(disc) ? R(0.25) * lh * rcp_(s) : R(0);
     const R lcs2 = R(0.5) * lh + ldisc * (R(2) * d + R(2) * cat2);
     const R lcan2 = R(0.5) * lh + ldisc * (R(-2) * d + R(2) * cat2);
     const R lcat2 = R(0.5) * lh + ldisc * (R(2) * (cs2 + can2) + R(2) * cat2);
@@ -77,7 +76,7 @@ template <typename R>
 MHD_HD void cons_to_prim_vjp(R rho, R mx, R my, R mz, R E, R bxc, R byc, R bzc, R gm1, const R lq[8], R lU[5],
                              R lbc[3]) {
     (void)E;
-    const R ri = R(1) / rho;
+    const R ri = rcp_(rho);
     const R u = mx * ri, v = my * ri, w = mz * ri;
     const R lP = lq[Q_P];
     // P = gm1 (E - rho |u|^2 / 2 - |bc|^2 / 2), u = m / rho
@@ -102,7 +101,7 @@ MHD_HD void hancock_vjp(const R q[8], const R D[3][8], R hdt, R gamma, const R l
     const R u = q[Q_U], v = q[Q_V], w = q[Q_W], rho = q[Q_RHO], P = q[Q_P];
     const R vel[3] = {u, v, w};
     const R divu = D[0][Q_U] + D[1][Q_V] + D[2][Q_W];
-    const R ri = R(1) / rho;
+    const R ri = rcp_(rho);
     R ladv[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) ladv[k] = R(0);
@@ -161,25 +160,25 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const R ptl = pl + R(0.5) * b2l, ptr = pr + R(0.5) * b2r;
     const R el = pl * gm1i + R(0.5) * rl * (ul * ul + vl * vl + wl * wl) + R(0.5) * b2l;
     const R er = pr * gm1i + R(0.5) * rr * (ur * ur + vr * vr + wr * wr) + R(0.5) * b2r;
-    const R cfl = fast_speed(R(1) / rl, gamma * pl, bn, byl, bzl);
-    const R cfr = fast_speed(R(1) / rr, gamma * pr, bn, byr, bzr);
+    const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
+    const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
     const R vbl = ul * bn + vl * byl + wl * bzl, vbr = ur * bn + vr * byr + wr * bzr;
-    const bool cl = cfl >= cfr;            // max picks cf_L
+    const bool cl = !greater_(cfr, cfl);   // max picks cf_L
     const R cmax = cl ? cfl : cfr;
-    const bool ml = ul <= ur;              // min picks u_L
-    const bool Ml = ul >= ur;              // max picks u_L
+    const bool ml = !greater_(ul, ur);     // min picks u_L
+    const bool Ml = !greater_(ur, ul);     // max picks u_L
     const R sl = (ml ? ul : ur) - cmax;
     const R sr = (Ml ? ul : ur) + cmax;
     const R dl = (sl - ul) * rl, dr = (sr - ur) * rr;
     const R den = dr - dl;
-    const R deni = R(1) / den;
+    const R deni = rcp_(den);
     const R smn = dr * ur - dl * ul - ptr + ptl;
     const R ptn = dr * ptl - dl * ptr + dl * dr * (ur - ul);
     const R sm = smn * deni;
     const R pts = ptn * deni;
     // star states, per side
     struct Star {
-        R S, sa, ssm, ssmi, rs, D, nu, nb, vs, ws, bys, bzs, vbs, nes, es;
+        R S, sa, ssm, ssmi, rs, D, Di, nu, nb, vs, ws, bys, bzs, vbs, nes, es;
         bool deg;
     };
     auto star = [&](R S, R r, R u, R v, R w, R by, R bz, R pt, R e, R vb) {
@@ -187,11 +186,12 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         t.S = S;
         t.sa = S - u;
         t.ssm = S - sm;
-        t.ssmi = R(1) / t.ssm;
+        t.ssmi = rcp_(t.ssm);
         t.rs = r * t.sa * t.ssmi;
         t.D = r * t.sa * t.ssm - bn2;
-        t.deg = rabs(t.D) <= eps * bn2;
-        const R Di = t.deg ? R(0) : R(1) / t.D;
+        t.deg = le_mag_(rabs(t.D), eps * bn2);
+        const R Di = t.deg ? R(0) : rcp_(t.D);
+        t.Di = Di;
         t.nu = bn * (sm - u) * Di;
         t.nb = (r * t.sa * t.sa - bn2) * Di;
         t.vs = t.deg ? v : v - by * t.nu;
@@ -207,9 +207,10 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const Star B = star(sr, rr, ur, vr, wr, byr, bzr, ptr, er, vbr);
     const R sql = rsqrt_(A.rs), sqr = rsqrt_(B.rs);
     const R abn = rabs(bn);
-    const R ssl = sm - abn / sql, ssr = sm + abn / sqr;
-    const R sgn = bn > R(0) ? R(1) : (bn < R(0) ? R(-1) : R(0));
-    const R isum = R(1) / (sql + sqr);
+    const R isql = rcp_(sql), isqr = rcp_(sqr);
+    const R ssl = sm - abn * isql, ssr = sm + abn * isqr;
+    const R sgn = nonzero_(bn) ? copysign(R(1), bn) : R(0);
+    const R isum = rcp_(sql + sqr);
     const R nv = sql * A.vs + sqr * B.vs + (B.bys - A.bys) * sgn;
     const R nw = sql * A.ws + sqr * B.ws + (B.bzs - A.bzs) * sgn;
     const R nby = sql * B.bys + sqr * A.bys + sql * sqr * (B.vs - A.vs) * sgn;
@@ -219,11 +220,11 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const R essl = A.es - sql * (A.vbs - vbss) * sgn;
     const R essr = B.es + sqr * (B.vbs - vbss) * sgn;
     int reg = 5;
-    if (sr >= R(0)) reg = 4;
-    if (ssr >= R(0)) reg = 3;
-    if (sm >= R(0)) reg = 2;
-    if (ssl >= R(0)) reg = 1;
-    if (sl >= R(0)) reg = 0;
+    if (nonneg_(sr)) reg = 4;
+    if (nonneg_(ssr)) reg = 3;
+    if (nonneg_(sm)) reg = 2;
+    if (nonneg_(ssl)) reg = 1;
+    if (nonneg_(sl)) reg = 0;
     const bool left = reg <= 2;
 
     // ----- reverse
@@ -251,7 +252,13 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         R g_e0 = lF[4] * u0;
         R g_vb0 = -lF[4] * bn;
         if (reg != 0 && reg != 5) {
-            const Star& T = left ? A : B;
+            // (selected field by field: a reference chosen at run time would put both in memory)
+            Star T;
+            T.S = left ? A.S : B.S;
+            T.rs = left ? A.rs : B.rs;
+            T.vs = left ? A.vs : B.vs;
+            T.ws = left ? A.ws : B.ws;
+            T.es = left ? A.es : B.es;
             const R S = T.S;
             const R us0 = T.rs, us1 = T.rs * sm, us2 = T.rs * T.vs, us3 = T.rs * T.ws, us4 = T.es;
             // f += S (U* - U)
@@ -282,16 +289,16 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
                     gA_vbs -= g_ess * sql * sgn;
                     g_vbss += g_ess * sql * sgn;
                     g_sm += gSs;
-                    g_abn -= gSs / sql;
-                    g_sql += gSs * abn / (sql * sql);
+                    g_abn -= gSs * isql;
+                    g_sql += gSs * abn * (isql * isql);
                 } else {      // essr = esr + sqr (vbsr - vbss) sgn ; ssr = sm + abn / sqr
                     gB_es += g_ess;
                     g_sqr += g_ess * (B.vbs - vbss) * sgn;
                     gB_vbs += g_ess * sqr * sgn;
                     g_vbss -= g_ess * sqr * sgn;
                     g_sm += gSs;
-                    g_abn += gSs / sqr;
-                    g_sqr -= gSs * abn / (sqr * sqr);
+                    g_abn += gSs * isqr;
+                    g_sqr -= gSs * abn * (isqr * isqr);
                 }
                 // vbss = sm bn + vss byss + wss bzss
                 g_sm += g_vbss * bn;
@@ -362,8 +369,8 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         }
     }
     // sql = sqrt(rsl), sqr = sqrt(rsr)
-    gA_rs += g_sql / (R(2) * sql);
-    gB_rs += g_sqr / (R(2) * sqr);
+    gA_rs += R(0.5) * g_sql * isql;
+    gB_rs += R(0.5) * g_sqr * isqr;
     // star states (reverse), side by side
     auto star_rev = [&](const Star& T, R r, R u, R v, R w, R by, R bz, R pt, R e, R vb, R g_rs, R g_vs, R g_ws,
                         R g_bys, R g_bzs, R g_vbs, R g_es, R& g_r, R& g_u, R& g_v, R& g_w, R& g_by, R& g_bz,
@@ -402,7 +409,7 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
             g_nb += g_bys * by;
             g_bz += g_bzs * T.nb;
             g_nb += g_bzs * bz;
-            const R Di = R(1) / T.D;
+            const R Di = T.Di;
             // nu = bn (sm - u) / D
             g_bn += g_nu * (sm - u) * Di;
             g_sm += g_nu * bn * Di;
@@ -506,6 +513,7 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
     const R bn2 = bn * bn;
     const R* st[2] = {L, Rt};
     R U[2][5], F[2][5], cf[2], e[2], pt[2], vb[2];
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
         const R r = st[k][0], u = st[k][1], v = st[k][2], w = st[k][3], p = st[k][4], by = st[k][5], bz = st[k][6];
         const R b2 = bn2 + by * by + bz * bz;
@@ -525,18 +533,18 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
         F[k][4] = (e[k] + pt[k]) * u - bn * vb[k];
     }
     const R ul = L[1], ur = Rt[1];
-    const bool cl = cf[0] >= cf[1];
+    const bool cl = !greater_(cf[1], cf[0]);
     const R cmax = cl ? cf[0] : cf[1];
-    const bool ml = ul <= ur, Ml = ul >= ur;
+    const bool ml = !greater_(ul, ur), Ml = !greater_(ur, ul);
     const R sl = (ml ? ul : ur) - cmax;
     const R sr = (Ml ? ul : ur) + cmax;
     // ----- reverse
     R lU[2][5] = {{0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}}, lFs[2][5] = {{0, 0, 0, 0, 0}, {0, 0, 0, 0, 0}};
     R lsl = R(0), lsr = R(0);
-    if (sl >= R(0)) {
+    if (nonneg_(sl)) {
         for (int c = 0; c < 5; ++c) lFs[0][c] = lF[c];
-    } else if (sr >= R(0)) {
-        const R di = R(1) / (sr - sl);
+    } else if (nonneg_(sr)) {
+        const R di = rcp_(sr - sl);
         for (int c = 0; c < 5; ++c) {
             const R dU = U[1][c] - U[0][c];
             const R fh = (sr * F[0][c] - sl * F[1][c] + sl * sr * dU) * di;
@@ -552,10 +560,11 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
     }
     // wave speeds: sl = min(ul, ur) - cmax, sr = max(ul, ur) + cmax
     R* lst[2] = {lL, lR};
-    lst[ml ? 0 : 1][1] += lsl;
-    lst[Ml ? 0 : 1][1] += lsr;
+    lL[1] += (ml ? lsl : R(0)) + (Ml ? lsr : R(0));
+    lR[1] += (ml ? R(0) : lsl) + (Ml ? R(0) : lsr);
     const R lcmax = lsr - lsl;
     R lcf[2] = {cl ? lcmax : R(0), cl ? R(0) : lcmax};
+#pragma unroll
     for (int k = 0; k < 2; ++k) {
         const R r = st[k][0], u = st[k][1], v = st[k][2], w = st[k][3], p = st[k][4], by = st[k][5], bz = st[k][6];
         R lr = R(0), lu = R(0), lv = R(0), lw = R(0), lp = R(0), lby = R(0), lbz = R(0);
@@ -627,9 +636,8 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const Corner<R>& s = *st[k];
-        const R ri = R(1) / s.rho, gP = gamma * s.p;
-        const R cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
-        const R cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
+        R cfa, cfb;
+        corner_speeds(s, gamma, cfa, cfb);
         ap[k] = s.ua + cfa;
         am[k] = s.ua - cfa;
         bp[k] = s.ub + cfb;
@@ -639,12 +647,13 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
     auto fold_max = [](const R* x, int& k) {
         R m = x[0];
         k = 0;
+#pragma unroll
         for (int j = 1; j < 4; ++j)
-            if (!(m >= x[j])) {
+            if (greater_(x[j], m)) {
                 m = x[j];
                 k = j;
             }
-        if (!(m >= R(0))) {
+        if (!nonneg_(m)) {
             m = R(0);
             k = -1;
         }
@@ -653,12 +662,13 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
     auto fold_min = [](const R* x, int& k) {
         R m = x[0];
         k = 0;
+#pragma unroll
         for (int j = 1; j < 4; ++j)
-            if (!(m <= x[j])) {
+            if (greater_(m, x[j])) {
                 m = x[j];
                 k = j;
             }
-        if (!(m <= R(0))) {
+        if (positive_(m)) {
             m = R(0);
             k = -1;
         }
@@ -671,19 +681,19 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
 #pragma unroll
     for (int k = 0; k < 4; ++k) e[k] = st[k]->ua * st[k]->Bb - st[k]->ub * st[k]->Ba;
     const R num = sE * sN * e[0] - sE * sS * e[2] - sW * sN * e[1] + sW * sS * e[3];
-    const R q = da * db;
-    const R t2 = sE * sW / da, t3 = sN * sS / db;
+    const R ida = rcp_(da), idb = rcp_(db);
+    const R t2 = sE * sW * ida, t3 = sN * sS * idb;
     const R jb = SE.Bb - SW.Bb, ja = NW.Ba - SW.Ba;
-    // E = num / q + t2 jb - t3 ja
-    const R g_num = lE / q;
-    const R g_q = -lE * num / (q * q);
+    // E = num / (da db) + t2 jb - t3 ja
+    const R g_num = lE * ida * idb;
+    const R g_q = -g_num * num * ida * idb;
     R g_da = g_q * db, g_db = g_q * da;
-    const R g_t2 = lE * jb, g_t3 = -lE * ja;
+    const R g_t2 = lE * jb * ida, g_t3 = -lE * ja * idb;   // cotangents of t2 and t3 over da and db
     const R g_jb = lE * t2, g_ja = -lE * t3;
-    R g_sE = g_t2 * sW / da, g_sW = g_t2 * sE / da;
-    g_da -= g_t2 * t2 / da;
-    R g_sN = g_t3 * sS / db, g_sS = g_t3 * sN / db;
-    g_db -= g_t3 * t3 / db;
+    R g_sE = g_t2 * sW, g_sW = g_t2 * sE;
+    g_da -= g_t2 * t2;
+    R g_sN = g_t3 * sS, g_sS = g_t3 * sN;
+    g_db -= g_t3 * t3;
     gSE.Bb += g_jb;
     gSW.Bb -= g_jb;
     gNW.Ba += g_ja;
@@ -704,37 +714,33 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
         gs[k]->ub -= g_e[k] * st[k]->Ba;
         gs[k]->Ba -= g_e[k] * st[k]->ub;
     }
-    // speeds -> corner velocities and fast speeds
-    // (each corner tests whether it was selected, so that every index is a compile-time
-    // constant and the corner cotangents stay in registers)
-    R g_cfa[4] = {0, 0, 0, 0}, g_cfb[4] = {0, 0, 0, 0};
+    // Each of the four speeds comes from one corner: its velocity and fast speed there.  The corner
+    // is selected by value, the result added by testing every corner, so that every index is a
+    // compile-time constant and the corner cotangents stay in registers (four reverse fast speeds
+    // instead of one per corner and direction).
+    auto speed = [&](int k, R g, bool alongb, R sgn) {
+        if (k < 0) return;
+        Corner<R> s = *st[0];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (k == kE) {
-            gs[k]->ua += g_sE;
-            g_cfa[k] += g_sE;
-        }
-        if (k == kW) {
-            gs[k]->ua += g_sW;
-            g_cfa[k] -= g_sW;
-        }
-        if (k == kN) {
-            gs[k]->ub += g_sN;
-            g_cfb[k] += g_sN;
-        }
-        if (k == kS) {
-            gs[k]->ub += g_sS;
-            g_cfb[k] -= g_sS;
-        }
-    }
+        for (int j = 1; j < 4; ++j)
+            if (j == k) s = *st[j];
+        R lrho = R(0), lp = R(0), lbn = R(0), lbt = R(0), lbe = R(0);
+        fast_speed_vjp(s.rho, s.p, alongb ? s.Bb : s.Ba, alongb ? s.Ba : s.Bb, s.Be, gamma, sgn * g, lrho, lp, lbn, lbt, lbe);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const Corner<R>& s = *st[k];
-        fast_speed_vjp(s.rho, s.p, s.Ba, s.Bb, s.Be, gamma, g_cfa[k], gs[k]->rho, gs[k]->p, gs[k]->Ba, gs[k]->Bb,
-                       gs[k]->Be);
-        fast_speed_vjp(s.rho, s.p, s.Bb, s.Ba, s.Be, gamma, g_cfb[k], gs[k]->rho, gs[k]->p, gs[k]->Bb, gs[k]->Ba,
-                       gs[k]->Be);
-    }
+        for (int j = 0; j < 4; ++j) {
+            if (j != k) continue;
+            (alongb ? gs[j]->ub : gs[j]->ua) += g;
+            gs[j]->rho += lrho;
+            gs[j]->p += lp;
+            (alongb ? gs[j]->Bb : gs[j]->Ba) += lbn;
+            (alongb ? gs[j]->Ba : gs[j]->Bb) += lbt;
+            gs[j]->Be += lbe;
+        }
+    };
+    speed(kE, g_sE, false, R(1));
+    speed(kW, g_sW, false, R(-1));
+    speed(kN, g_sN, true, R(1));
+    speed(kS, g_sS, true, R(-1));
 }
 
 }  // namespace mhd
