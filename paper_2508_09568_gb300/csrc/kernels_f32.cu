@@ -13,7 +13,7 @@ static const StepLaunch kStepF32[] = {
     StepInst<float, 3, 24, 8, 512>::entry(4.76f, 4.76f),
     StepInst<float, 2, 16, 16, 256>::entry(4.9f, 11.0f),
     StepInst<float, 2, 32, 8, 256>::entry(4.35f, 9.5f),
-    StepInst<float, 1, 64, 1, 64>::entry(),
+    StepInst<float, 1, 64, 1, 128>::entry(),
 };
 
 const PrecisionKernels& kernels_f32() {

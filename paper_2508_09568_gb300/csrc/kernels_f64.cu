@@ -8,7 +8,7 @@ static const StepLaunch kStepF64[] = {
     StepInst<double, 3, 8, 8, 128>::entry(52.0f, 52.0f),
     StepInst<double, 2, 16, 16, 256>::entry(122.0f, 128.0f),
     StepInst<double, 2, 8, 8, 128>::entry(41.5f, 50.0f),
-    StepInst<double, 1, 64, 1, 64>::entry(),
+    StepInst<double, 1, 64, 1, 128>::entry(),
 };
 
 const PrecisionKernels& kernels_f64() {

@@ -38,6 +38,11 @@ struct Items {
     static constexpr int XTRA = MAP == MAP_ROWS && NI > 32 ? NI - 32 : 0;
     static constexpr int N = MAP == MAP_ROWS ? NJ + (XTRA * NJ + 31) / 32
                                              : ((MAP == MAP_PITCH ? P : NI) * NJ + 31) / 32;   // chunks
+    // one dimension: chunk q holds no item with i <= imax (a tile that reaches past its patch: of the
+    // 64 columns of a tile a 16-cell patch needs one chunk in three, and each costs the FP64 pipe the
+    // same; 1D step of 256 cells 50 -> 24 us).  In 2D and 3D the test costs more than the rows of
+    // ragged tiles that it saves (512^3 +1 %, 21x28x17 patches no change).
+    __device__ static __forceinline__ bool beyond(int q, int imax) { return NJ == 1 && q * 32 > imax; }
     // item (i, j) of lane `lane` of chunk q; false: idle lane
     __device__ static __forceinline__ bool at(int q, int lane, int& i, int& j) {
         if constexpr (MAP == MAP_ROWS) {
@@ -269,7 +274,7 @@ struct Tile {
 template <typename R, typename C>
 __device__ __forceinline__ void convert_chunk(const Tile<R>& T, const R* raw, int m, R* Wslot, int q, R gm1) {
     int li, lj;
-    if (!C::ICV::at(q, threadIdx.x & 31, li, lj)) return;
+    if (C::ICV::beyond(q, T.wx + 2 + C::LOX) || !C::ICV::at(q, threadIdx.x & 31, li, lj)) return;
     const PatchDev& pt = T.pt;
     const int x0 = T.x0, y0 = T.y0;
     const int w = lj * C::LX + li;
@@ -587,10 +592,10 @@ __device__ __forceinline__ void update_chunk(const StepSmem<R, C>& S, const Tile
 
 // The EMF at (i-1/2, j-1/2) of plane c, chunk q of IEZ: i in [0, TX], j in [0, TY]
 template <typename R, typename C>
-__device__ __forceinline__ void flux_ez(const R* P0, R* IB, int q, R gamma) {
+__device__ __forceinline__ void flux_ez(const R* P0, R* IB, int q, int wx, R gamma) {
     R* Ez = IB + 5 * C::FXN + 5 * C::FYN;
     int i, j;
-    if (C::IEZ::at(q, threadIdx.x & 31, i, j)) {
+    if (!C::IEZ::beyond(q, wx) && C::IEZ::at(q, threadIdx.x & 31, i, j)) {
         const int jm = C::AY ? j - 1 : j;
         // cells: SW=(i-1,j-1) RT, SE=(i,j-1) LT, NW=(i-1,j) RB, NE=(i,j) LB
         const int pSW = pidx<C>(i - 1, jm), pSE = pidx<C>(i, jm);
@@ -612,13 +617,13 @@ __device__ __forceinline__ void flux_ez(const R* P0, R* IB, int q, R gamma) {
 
 // In-plane fluxes of plane c (slot P0 into IB), one chunk q of NI.
 template <typename R, typename C>
-__device__ __forceinline__ void flux_inplane(const R* P0, R* IB, int q, R gamma, R gm1i, R eps, int riemann) {
+__device__ __forceinline__ void flux_inplane(const R* P0, R* IB, int q, int wx, R gamma, R gm1i, R eps, int riemann) {
     R* Fx = IB;
     R* Fy = IB + 5 * C::FXN;
     const int lane = threadIdx.x & 31;
     int i, j;
     if (q < C::IFX::N) {   // x-face i-1/2 of cell (i, j): i in [0, TX], j in [0, TY)
-        if (C::IFX::at(q, lane, i, j)) {
+        if (!C::IFX::beyond(q, wx) && C::IFX::at(q, lane, i, j)) {
             R F[5];
             face_flux<R, C>(P0, pidx<C>(i - 1, j), P0, pidx<C>(i, j), 0, gamma, gm1i, eps, riemann, F);
             const int o = j * (C::TX + 1) + i;
@@ -629,7 +634,7 @@ __device__ __forceinline__ void flux_inplane(const R* P0, R* IB, int q, R gamma,
     }
     q -= C::IFX::N;
     if (q < C::IFY::N) {   // y-face j-1/2 of cell (i, j): i in [0, TX), j in [0, TY]
-        if (C::AY && C::IFY::at(q, lane, i, j)) {
+        if (C::AY && !C::IFY::beyond(q, wx) && C::IFY::at(q, lane, i, j)) {
             R F[5];
             face_flux<R, C>(P0, pidx<C>(i, j - 1), P0, pidx<C>(i, j), 1, gamma, gm1i, eps, riemann, F);
             const int o = j * C::TX + i;
@@ -638,20 +643,20 @@ __device__ __forceinline__ void flux_inplane(const R* P0, R* IB, int q, R gamma,
         }
         return;
     }
-    flux_ez<R, C>(P0, IB, q - C::IFY::N, gamma);
+    flux_ez<R, C>(P0, IB, q - C::IFY::N, wx, gamma);
 }
 
 // Fluxes between planes c-1 (slot Pm) and c (slot P0) into ZB, one chunk q of NZ.
 template <typename R, typename C>
-__device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB, int q, R gamma, R gm1i, R eps,
-                                                int riemann) {
+__device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB, int q, int wx, R gamma,
+                                                R gm1i, R eps, int riemann) {
     R* Fz = ZB;
     R* Ex = ZB + 5 * C::FZN;
     R* Ey = Ex + C::EXN;
     const int lane = threadIdx.x & 31;
     int i, j;
     if (q < C::IFZ::N) {   // z-face c-1/2 of cell (i, j): i in [0, TX), j in [0, TY)
-        if (C::AZ && C::IFZ::at(q, lane, i, j)) {
+        if (C::AZ && !C::IFZ::beyond(q, wx) && C::IFZ::at(q, lane, i, j)) {
             const int p = pidx<C>(i, j);
             R F[5];
             face_flux<R, C>(Pm, p, P0, p, 2, gamma, gm1i, eps, riemann, F);
@@ -663,7 +668,7 @@ __device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB,
     }
     q -= C::IFZ::N;
     if (q < C::IEX::N) {   // Ex at (i, j-1/2, c-1/2): a = y, b = z; i in [0, TX), j in [0, TY]
-        if (C::AY && C::IEX::at(q, lane, i, j)) {
+        if (C::AY && !C::IEX::beyond(q, wx) && C::IEX::at(q, lane, i, j)) {
             const int pS = pidx<C>(i, j - 1), pN = pidx<C>(i, j);
             // SW = (j-1, c-1) corner (+y,+z); SE = (j, c-1) (-y,+z);
             // NW = (j-1, c) (+y,-z); NE = (j, c) (-y,-z)
@@ -683,7 +688,7 @@ __device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB,
     }
     q -= C::IEX::N;
     {   // Ey at (i-1/2, j, c-1/2): a = z, b = x; i in [0, TX], j in [0, TY)
-        if (C::IEY::at(q, lane, i, j)) {
+        if (!C::IEY::beyond(q, wx) && C::IEY::at(q, lane, i, j)) {
             const int pW = pidx<C>(i - 1, j), pE = pidx<C>(i, j);
             // SW = (x=i-1, c-1) corner (+z,+x); SE = (i-1, c) (-z,+x);
             // NW = (i, c-1) (+z,-x); NE = (i, c) (-z,-x)
@@ -704,9 +709,9 @@ __device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB,
 
 // prep of one chunk q of a plane
 template <typename R, typename C>
-__device__ __forceinline__ void prep_chunk(const PrepCtx<R, C>& X, R* Ps, int q, int limiter) {
+__device__ __forceinline__ void prep_chunk(const PrepCtx<R, C>& X, R* Ps, int q, int limiter, int wx) {
     int i, j;
-    if (!C::IPR::at(q, threadIdx.x & 31, i, j)) return;
+    if (C::IPR::beyond(q, wx + C::POX) || !C::IPR::at(q, threadIdx.x & 31, i, j)) return;
     i -= C::POX;
     j -= C::POY;
     if (limiter == 0) prep_cell<R, C, 0>(X, i, j, Ps, pidx<C>(i, j));
@@ -873,12 +878,12 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
                 for (int q; (q = list.next()) != 255;) {
                     if (q < C::NI) {
                         if (ci >= z0 && ci < z1) {
-                            if constexpr (B) flux_inplane<R, C>(S.P(ci & 1), S.I(ci & 1), q, a.gamma, a.gm1i, a.eps, a.riemann);
-                            else flux_ez<R, C>(S.P(ci & 1), S.I(ci & 1), q - C::IFX::N - C::IFY::N, a.gamma);
+                            if constexpr (B) flux_inplane<R, C>(S.P(ci & 1), S.I(ci & 1), q, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
+                            else flux_ez<R, C>(S.P(ci & 1), S.I(ci & 1), q - C::IFX::N - C::IFY::N, T.wx, a.gamma);
                         }
                     } else if (q < C::NI + C::NZ) {
                         if (c >= z0)
-                            flux_interplane<R, C>(S.P((c + 1) & 1), S.P(c & 1), S.Z(c & 1), q - C::NI, a.gamma, a.gm1i,
+                            flux_interplane<R, C>(S.P((c + 1) & 1), S.P(c & 1), S.Z(c & 1), q - C::NI, T.wx, a.gamma, a.gm1i,
                                                   a.eps, a.riemann);
                     } else if (q < C::NI + C::NZ + C::IPR::N) {
                         if (c < z1) {
@@ -889,7 +894,7 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
                             X.hdt = T.hdt;
                             X.gamma = a.gamma;
                             for (int d = 0; d < 3; ++d) X.dxi[d] = a.dxir[d];
-                            prep_chunk<R, C>(X, S.P((c + 1) & 1), q - C::NI - C::NZ, a.limiter);
+                            prep_chunk<R, C>(X, S.P((c + 1) & 1), q - C::NI - C::NZ, a.limiter, T.wx);
                         }
                     } else if (q < C::NI + C::NZ + C::IPR::N + C::ICV::N) {
                         if (c < z1) {
@@ -937,11 +942,11 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
             X.hdt = T.hdt;
             X.gamma = a.gamma;
             for (int d = 0; d < 3; ++d) X.dxi[d] = a.dxir[d];
-            for (int q = wid; q < C::IPR::N; q += C::NWARP) prep_chunk<R, C>(X, S.P(0), q, a.limiter);
+            for (int q = wid; q < C::IPR::N; q += C::NWARP) prep_chunk<R, C>(X, S.P(0), q, a.limiter, T.wx);
             __syncthreads();
             for (int q = wid; q < C::NI + C::NZ; q += C::NWARP) {
-                if (q < C::NI) flux_inplane<R, C>(S.P(0), S.I(0), q, a.gamma, a.gm1i, a.eps, a.riemann);
-                else flux_interplane<R, C>(S.P(0), S.P(0), S.Z(0), q - C::NI, a.gamma, a.gm1i, a.eps, a.riemann);
+                if (q < C::NI) flux_inplane<R, C>(S.P(0), S.I(0), q, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
+                else flux_interplane<R, C>(S.P(0), S.P(0), S.Z(0), q - C::NI, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
             }
             if (a.dynamic && threadIdx.x == 0) s_tile = atomicAdd(&a.work[0], 1);
             __syncthreads();

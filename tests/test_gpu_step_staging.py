@@ -48,3 +48,17 @@ def test_step_matches_oracle_in_every_configuration(shape, dtype, limiter):
                 assert_parity(got, ref, dtype, what=shape)
             assert np.array_equal(got, first), (shape, cfg, mode)
     assert b.error()[0] == 0
+
+
+@pytest.mark.parametrize("n", [3, 27, 63, 64, 65, 100])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32], ids=["f64", "f32"])
+def test_1d_tiles_that_reach_past_their_patch(n, dtype):
+    """1D patches from a few cells to more than a tile: the chunks past the patch are left out."""
+    geom, U, meta = W.sod(ncell=4 * n, npatch=4)
+    flat = rounded(W.to_patches(U, geom), dtype)
+    ob = oracle_bunch(geom, meta["gamma"], dtype=dtype)
+    dt = ob.cfl_dt(ob.fill_guards(ob.split(flat)))
+    ref = interior_global(oracle_steps(geom, flat, meta["gamma"], [dt, dt], dtype=dtype), geom)
+    b = gpu_bunch(geom, flat, meta["gamma"], dtype)
+    assert_parity(interior_global(gpu_steps(b, [dt, dt]), geom), ref, dtype)
+    assert b.error()[0] == 0
