@@ -97,22 +97,37 @@ MHD_HD void hancock(const R q[8], const R D[3][8], R hdt, R gamma, R out[5]) {
 
 // The same half step from the undivided slopes dW[d][k] and the inverse cell sizes dxi[d]
 // (D = dW * dxi folded into the products that use it; equal to hancock up to rounding).
-// The step kernel's prep uses this form: one multiply less on each slope's path.
-template <typename R>
+// The step kernel's prep uses this form: one multiply less on each slope's path.  ND: active
+// axes; the slopes of the others are 0, and what they multiply is left out (the compiler keeps
+// products with 0), which leaves the values as they are.
+template <int ND, typename R>
 MHD_HD void hancock_dw(const R q[8], const R dW[3][8], const R dxi[3], R hdt, R gamma, R out[5]) {
     const R u = q[Q_U], v = q[Q_V], w = q[Q_W], rho = q[Q_RHO], P = q[Q_P];
     const R us = u * dxi[0], vs = v * dxi[1], ws = w * dxi[2];
-    const R divu = fma_(dxi[0], dW[0][Q_U], fma_(dxi[1], dW[1][Q_V], dxi[2] * dW[2][Q_W]));
+    // x dW[0][k] + y dW[1][l] + z dW[2][m] over the active axes
+    auto sum = [&](R x, int k, R y, int l, R z, int m) {
+        if constexpr (ND == 3) return fma_(x, dW[0][k], fma_(y, dW[1][l], z * dW[2][m]));
+        else if constexpr (ND == 2) return fma_(x, dW[0][k], y * dW[1][l]);
+        else return x * dW[0][k];
+    };
+    const R divu = sum(dxi[0], Q_U, dxi[1], Q_V, dxi[2], Q_W);
     const R ri = rcp_(rho);
-    auto adv = [&](int k) { return fma_(us, dW[0][k], fma_(vs, dW[1][k], ws * dW[2][k])); };
+    auto adv = [&](int k) { return sum(us, k, vs, k, ws, k); };
+    // d_c B_a - d_a B_c
+    auto twist = [&](int c, int a) {
+        if (c >= ND) return -(dxi[a] * dW[a][Q_BX + c]);
+        if (a >= ND) return dxi[c] * dW[c][Q_BX + a];
+        return fma_(dxi[c], dW[c][Q_BX + a], -(dxi[a] * dW[a][Q_BX + c]));
+    };
     out[0] = rho - hdt * fma_(rho, divu, adv(Q_RHO));
     out[4] = P - hdt * fma_(gamma * P, divu, adv(Q_P));
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const int a = (c + 1) % 3, b = (c + 2) % 3;
-        const R ja = fma_(dxi[c], dW[c][Q_BX + a], -(dxi[a] * dW[a][Q_BX + c]));
-        const R jb = fma_(dxi[c], dW[c][Q_BX + b], -(dxi[b] * dW[b][Q_BX + c]));
-        const R lor = fma_(q[Q_BX + a], ja, fma_(q[Q_BX + b], jb, dxi[c] * dW[c][Q_P]));
+        R lor;
+        if (c < ND) lor = fma_(q[Q_BX + a], twist(c, a), fma_(q[Q_BX + b], twist(c, b), dxi[c] * dW[c][Q_P]));
+        else if (a < ND && b < ND) lor = fma_(q[Q_BX + a], twist(c, a), q[Q_BX + b] * twist(c, b));
+        else lor = a < ND ? q[Q_BX + a] * twist(c, a) : q[Q_BX + b] * twist(c, b);
         out[1 + c] = q[Q_U + c] - hdt * fma_(lor, ri, adv(Q_U + c));
     }
 }
@@ -356,6 +371,33 @@ MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, co
     const R num = fma_(sE, fma_(sN, eSW, -sS * eNW), -sW * fma_(sN, eSE, -sS * eNE));
     const R ida = rcp_(da), idb = rcp_(db);
     return fma_(sE * sW * ida, SE.Bb - SW.Bb, fma_(num * ida, idb, -(sN * sS * idb) * (NW.Ba - SW.Ba)));
+}
+
+// The same where one of the two axes is collapsed (2D: E_x, E_y; 1D: E_y, E_z), from the states s0, s1
+// of the active axis (a if along_a, else b): the four corners are two states twice over.
+// Double precision: the speeds along the collapsed axis cancel, and what stays is the HLL induction
+// flux E = [S_1 e_0 - S_0 e_1 + S_1 S_0 dB] / (S_1 - S_0), S_1 = max(0, max u+cf), S_0 = min(0, min u-cf):
+// 2 fast speeds instead of 8.  Single precision keeps emf2d's rounding; the compiler shares the states
+// that are the same (4 speeds).  512^2 box of 32^2 patches: FP64, 2 steps, 1754 -> 1388 us; FP32, 4 steps,
+// 125.8 -> 118.7 us; 1D, 256 cells, FP64, 8 steps, 98.2 -> 82.5 us.
+template <typename R>
+MHD_HD R emf_line(const Corner<R>& s0, const Corner<R>& s1, bool along_a, R gamma) {
+    if constexpr (sizeof(R) == 4) {
+        return along_a ? emf2d(s0, s1, s0, s1, gamma) : emf2d(s0, s0, s1, s1, gamma);
+    } else {
+        auto speed = [&](const Corner<R>& s) {
+            const R bn = along_a ? s.Ba : s.Bb, bt = along_a ? s.Bb : s.Ba;
+            const R bt2 = fma_(bt, bt, s.Be * s.Be), b2 = fma_(bn, bn, bt2);
+            const R df = fma_(gamma, s.p, -b2);
+            return rsqrt_(fast_h(R(4) * gamma * s.p, fma_(gamma, s.p, b2), df * df, bt2) * (R(0.5) * rcp_(s.rho)));
+        };
+        const R c0 = speed(s0), c1 = speed(s1);
+        const R u0 = along_a ? s0.ua : s0.ub, u1 = along_a ? s1.ua : s1.ub;
+        const R S1 = fmax_(fmax_(u0 + c0, u1 + c1), R(0)), S0 = fmin_(fmin_(u0 - c0, u1 - c1), R(0));
+        const R e0 = fma_(s0.ua, s0.Bb, -s0.ub * s0.Ba), e1 = fma_(s1.ua, s1.Bb, -s1.ub * s1.Ba);
+        const R dB = along_a ? s1.Bb - s0.Bb : s0.Ba - s1.Ba;
+        return fma_(S1 * S0, dB, fma_(S1, e0, -S0 * e1)) * rcp_(S1 - S0);
+    }
 }
 
 }  // namespace mhd

@@ -430,7 +430,7 @@ __device__ __forceinline__ void prep_cell(const PrepCtx<R, C>& X, int i, int j, 
 
     // a5: Hancock predictor
     R hq[5];
-    hancock_dw(q, dW, X.dxi, X.hdt, X.gamma, hq);
+    hancock_dw<C::NDIM>(q, dW, X.dxi, X.hdt, X.gamma, hq);
 
 #pragma unroll
     for (int k = 0; k < 5; ++k) Pslot[PV_WH(k) * C::PSZ + pid] = hq[k];
@@ -503,6 +503,30 @@ __device__ __forceinline__ Corner<R> corner(const R* P, int pid, int e, R sa, R 
     s.Ba = ba_face + R(0.5) * sb * ba_slope;
     s.Bb = bb_face + R(0.5) * sa * bb_slope;
     return s;
+}
+
+// The EMF on an edge along e whose transverse axis o is collapsed, between the cells pid0 and pid1 along
+// the other, d (the face between them is the low face of pid1): each cell's state at that face.
+template <typename R, typename C>
+__device__ __forceinline__ R line_emf(const R* P, int pid0, int pid1, int e, int d, R gamma) {
+    const int o = 3 - e - d, k = d == (o + 1) % 3 ? 0 : 1;   // PV_FS(o, k): slope along d of the o-face field
+    const bool along_a = d == (e + 1) % 3;
+    const R bd = pv<R, C>(P, PV_BH(d), pid1);
+    auto state = [&](int pid, R s) {
+        auto ext = [&](int v) { return pv<R, C>(P, PV_WH(v), pid) + R(0.5) * (s * pv<R, C>(P, PV_DW(d, v), pid)); };
+        const R ud = ext(Q_U + d), uo = ext(Q_U + o);
+        const R bo = pv<R, C>(P, PV_BH(o), pid) + R(0.5) * s * pv<R, C>(P, PV_FS(o, k), pid);
+        Corner<R> c;
+        c.rho = ext(Q_RHO);
+        c.p = ext(Q_P);
+        c.ua = along_a ? ud : uo;
+        c.ub = along_a ? uo : ud;
+        c.Be = ext(Q_BX + e);
+        c.Ba = along_a ? bd : bo;
+        c.Bb = along_a ? bo : bd;
+        return c;
+    };
+    return emf_line(state(pid0, R(1)), state(pid1, R(-1)), along_a, gamma);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -596,7 +620,11 @@ __device__ __forceinline__ void flux_ez(const R* P0, R* IB, int q, int wx, R gam
     R* Ez = IB + 5 * C::FXN + 5 * C::FYN;
     int i, j;
     if (!C::IEZ::beyond(q, wx) && C::IEZ::at(q, threadIdx.x & 31, i, j)) {
-        const int jm = C::AY ? j - 1 : j;
+        if constexpr (!C::AY) {
+            Ez[i] = line_emf<R, C>(P0, pidx<C>(i - 1, j), pidx<C>(i, j), 2, 0, gamma);
+            return;
+        }
+        const int jm = j - 1;
         // cells: SW=(i-1,j-1) RT, SE=(i,j-1) LT, NW=(i-1,j) RB, NE=(i,j) LB
         const int pSW = pidx<C>(i - 1, jm), pSE = pidx<C>(i, jm);
         const int pNW = pidx<C>(i - 1, j), pNE = pidx<C>(i, j);
@@ -670,6 +698,10 @@ __device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB,
     if (q < C::IEX::N) {   // Ex at (i, j-1/2, c-1/2): a = y, b = z; i in [0, TX), j in [0, TY]
         if (C::AY && !C::IEX::beyond(q, wx) && C::IEX::at(q, lane, i, j)) {
             const int pS = pidx<C>(i, j - 1), pN = pidx<C>(i, j);
+            if constexpr (!C::AZ) {
+                Ex[j * C::TX + i] = line_emf<R, C>(P0, pS, pN, 0, 1, gamma);
+                return;
+            }
             // SW = (j-1, c-1) corner (+y,+z); SE = (j, c-1) (-y,+z);
             // NW = (j-1, c) (+y,-z); NE = (j, c) (-y,-z)
             // Ba = By face at side sy: the low y-face of row j (both planes)
@@ -690,6 +722,10 @@ __device__ __forceinline__ void flux_interplane(const R* Pm, const R* P0, R* ZB,
     {   // Ey at (i-1/2, j, c-1/2): a = z, b = x; i in [0, TX], j in [0, TY)
         if (!C::IEY::beyond(q, wx) && C::IEY::at(q, lane, i, j)) {
             const int pW = pidx<C>(i - 1, j), pE = pidx<C>(i, j);
+            if constexpr (!C::AZ) {
+                Ey[j * (C::TX + 1) + i] = line_emf<R, C>(P0, pW, pE, 1, 0, gamma);
+                return;
+            }
             // SW = (x=i-1, c-1) corner (+z,+x); SE = (i-1, c) (-z,+x);
             // NW = (i, c-1) (+z,-x); NE = (i, c) (-z,-x)
             // Ba = Bz face at side sz: low face of plane c (shared); slope along x

@@ -62,3 +62,31 @@ def test_1d_tiles_that_reach_past_their_patch(n, dtype):
     b = gpu_bunch(geom, flat, meta["gamma"], dtype)
     assert_parity(interior_global(gpu_steps(b, [dt, dt]), geom), ref, dtype)
     assert b.error()[0] == 0
+
+
+# 1D and 2D boxes with all field components: edges along and across the collapsed axes
+COLLAPSED = {
+    "1d": ((37, 1, 1), (37, 1, 1)),
+    "1d_patches": ((72, 1, 1), (24, 1, 1)),
+    "2d_odd": ((33, 17, 1), (33, 17, 1)),
+    "2d_patches": ((40, 24, 1), (20, 12, 1)),
+    "2d_smallest": ((6, 6, 1), (3, 3, 1)),
+}
+
+
+@pytest.mark.parametrize("shape", list(COLLAPSED))
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32], ids=["f64", "f32"])
+@pytest.mark.parametrize("riemann,limiter", [(0, 0), (1, 1)], ids=["hlld_minmod", "hll_mc"])
+def test_edges_of_collapsed_axes(shape, dtype, riemann, limiter):
+    ncell, patch = COLLAPSED[shape]
+    geom, U, meta = W.small_box(ncell=ncell, patch=patch, seed=47)
+    flat = rounded(W.to_patches(U, geom), dtype)
+    ob = oracle_bunch(geom, meta["gamma"], limiter=limiter, dtype=dtype, riemann=riemann)
+    dt = ob.cfl_dt(ob.fill_guards(ob.split(flat)))
+    ref = oracle_steps(geom, flat, meta["gamma"], [dt], limiter=limiter, dtype=dtype, riemann=riemann)
+    b = gpu_bunch(geom, flat, meta["gamma"], dtype, limiter=limiter, riemann=riemann)
+    for cfg in range(-1, b.num_configs()):
+        b.set_mode(capi.MHD_MODE_PERSISTENT, cfg)
+        b.upload(flat)
+        assert_parity(interior_global(gpu_steps(b, [dt]), geom), interior_global(ref, geom), dtype, what=shape, b_vector=True)
+    assert b.error()[0] == 0
