@@ -120,7 +120,8 @@ struct StepInst {
     static cudaError_t launch(const void* args, int grid, cudaStream_t s) {
         const StepArgs<R> a = to_args<R>(*static_cast<const StepHostArgs*>(args));
         static const StepPlan plan = NDIM == 3 ? make_plan<C>() : StepPlan{};
-        (a.slice ? async : a.nzb > 1 ? split : whole)<<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
+        if (a.slice) launch_pdl(async, grid, NT, C::SMEM_BYTES, s, a, plan);
+        else (a.nzb > 1 ? split : whole)<<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
         return cudaGetLastError();
     }
     static StepLaunch entry(float plane_us = 1, float alone_us = 1) {
@@ -175,13 +176,13 @@ static cudaError_t launch_fill_interp(void* U0, void* U1, const PatchDev* patche
     if (nlist <= 0) return cudaSuccess;
     const int gy = std::min(std::min(nlist, grid_y > 0 ? grid_y : nlist), 65535);
     if (nboff) {
-        fill_interp_grid_kernel<R><<<dim3(Zp, gy), 128, 0, s>>>(static_cast<R*>(U0), static_cast<R*>(U1), patches,
-                                                                 nboff, list, nlist, nlist_dev, pstride, slice, t_old,
-                                                                 t_cur);
+        const unsigned grid = (unsigned)std::min<int64_t>((int64_t)nlist * Zp, (int64_t)8 * gy);
+        launch_pdl(fill_interp_grid_kernel<R>, grid, 128, 0, s, static_cast<R*>(U0), static_cast<R*>(U1), patches, nboff,
+                   list, nlist, nlist_dev, pstride, Zp, slice, t_old, t_cur);
         return cudaGetLastError();
     }
     dim3 grid(32, gy);
-    fill_interp_kernel<R><<<grid, 256, 0, s>>>(static_cast<R*>(U0), static_cast<R*>(U1), patches, npatch, list, nlist,
+    launch_pdl(fill_interp_kernel<R>, grid, 256, 0, s, static_cast<R*>(U0), static_cast<R*>(U1), patches, npatch, list, nlist,
                                                nlist_dev, slice, t_old, t_cur, fg, err);
     return cudaGetLastError();
 }
@@ -192,9 +193,8 @@ static cudaError_t launch_cfl_patch(const void* U0, const void* U1, const PatchD
                                    const double dxi[3], const int act[3], unsigned long long* rate_max,
                                    unsigned* err, cudaStream_t s) {
     if (nlist <= 0) return cudaSuccess;
-    const int gy = std::min(std::min(nlist, grid_y > 0 ? grid_y : nlist), 65535);
-    dim3 grid(16, gy);
-    cfl_patch_kernel<R><<<grid, 256, 0, s>>>(static_cast<const R*>(U0), static_cast<const R*>(U1), patches, list,
+    const unsigned grid = (unsigned)std::min<int64_t>((int64_t)16 * nlist, (int64_t)8 * (grid_y > 0 ? grid_y : nlist));
+    launch_pdl(cfl_patch_kernel<R>, grid, 256, 0, s, static_cast<const R*>(U0), static_cast<const R*>(U1), patches, list,
                                              nlist, nlist_dev, slice, gamma, dxi[0], dxi[1], dxi[2], act[1], act[2],
                                              rate_max, err);
     return cudaGetLastError();

@@ -713,10 +713,11 @@ __global__ void __launch_bounds__(256, 4) fill_cfl_staged_kernel(R* __restrict__
 // between the owner's two slices, w = (t_cur[p] - t_old[q]) / (t_cur[q] - t_old[q]); w >= 1
 // (or equal slice times) takes the current slice exactly, w <= 0 the previous one.
 template <typename R>
-__global__ void fill_interp_kernel(R* __restrict__ U0, R* __restrict__ U1, const PatchDev* __restrict__ patches,
-                                   int npatch, const int* __restrict__ list, int nlist, const int* nlist_dev,
-                                   const int* __restrict__ slice, const double* __restrict__ t_old,
-                                   const double* __restrict__ t_cur, FillGeom fg, unsigned* err) {
+__global__ void fill_interp_kernel(R* U0, R* U1, const PatchDev* __restrict__ patches,
+                                   int npatch, const int* list, int nlist, const int* nlist_dev,
+                                   const int* slice, const double* t_old,
+                                   const double* t_cur, FillGeom fg, unsigned* err) {
+    pdl_begin();
     const int nl = nlist_dev ? min(*nlist_dev, nlist) : nlist;
     for (int L = blockIdx.y; L < nl; L += gridDim.y) {
         const int p = list[L];
@@ -792,33 +793,33 @@ __global__ void fill_interp_kernel(R* __restrict__ U0, R* __restrict__ U1, const
 // The same for equal patches on a regular grid: sources from the neighbour table (as
 // fill_grid_kernel; the patch owning a source is its state offset over pstride, the state
 // stride of one patch, the patches being stored back to back), one CTA per padded z-plane of
-// a listed patch (blockIdx.x = plane), four ghost cells per thread and pass with both slices
-// of their sources loaded before the stores; the same values as fill_interp_kernel.
+// a listed patch at a time, four ghost cells per thread and pass with the slices of their sources
+// loaded before the stores; the same values as fill_interp_kernel.  The weight depends on the source
+// patch only: once per direction and plane, with what it says of the slices needed (1: the current
+// one, -1: the previous one, 0: both), so that a cell's loop has no FP64 and a slice that does not
+// count is not read.
 template <typename R>
-__global__ void __launch_bounds__(128) fill_interp_grid_kernel(R* __restrict__ U0, R* __restrict__ U1,
-                                                              const PatchDev* __restrict__ patches,
-                                                              const int64_t* __restrict__ nboff,
-                                                              const int* __restrict__ list, int nlist,
-                                                              const int* nlist_dev, int64_t pstride,
-                                                              const int* __restrict__ slice,
-                                                              const double* __restrict__ t_old,
-                                                              const double* __restrict__ t_cur) {
-    __shared__ double s_w[27];   // time weight of the slices of the patch in each direction
-    __shared__ int s_sq[27];     // its current slice
+__global__ void __launch_bounds__(128) fill_interp_grid_kernel(R* U0, R* U1, const PatchDev* __restrict__ patches,
+                                                              const int64_t* __restrict__ nboff, const int* list,
+                                                              int nlist, const int* nlist_dev, int64_t pstride, int Zp,
+                                                              const int* slice, const double* t_old,
+                                                              const double* t_cur) {
+    pdl_begin();
+    __shared__ R s_w[27];            // time weight of the slices of the patch in each direction
+    __shared__ int s_sq[27], s_m[27];   // its current slice, the slices needed
     const int nl = nlist_dev ? min(*nlist_dev, nlist) : nlist;
-    const int z = blockIdx.x;
-    for (int L = blockIdx.y; L < nl; L += gridDim.y) {
+    for (int64_t item = blockIdx.x; item < (int64_t)nl * Zp; item += gridDim.x) {
+        const int L = (int)(item / Zp), z = (int)(item - (int64_t)L * Zp);
         const int p = list[L];
         const PatchDev pt = patches[p];
-        if (z >= pt.Z) continue;
         const int64_t* nb = nboff + (int64_t)p * 27;
-        // the weight depends on the source patch only: once per direction, not per ghost cell
-        // (an FP64 division per cell kept the small FP64 pipe busy)
         __syncthreads();
         if (threadIdx.x < 27) {
             const int q = (int)(nb[threadIdx.x] / pstride);
-            const double den = t_cur[q] - t_old[q];
-            s_w[threadIdx.x] = den > 0.0 ? (t_cur[p] - t_old[q]) / den : 1.0;
+            const double t0 = t_old[q], den = t_cur[q] - t0;
+            const double w = den > 0.0 ? (t_cur[p] - t0) / den : 1.0;
+            s_w[threadIdx.x] = R(w);
+            s_m[threadIdx.x] = w >= 1.0 ? 1 : (w <= 0.0 ? -1 : 0);
             s_sq[threadIdx.x] = slice[q];
         }
         __syncthreads();
@@ -832,9 +833,7 @@ __global__ void __launch_bounds__(128) fill_interp_grid_kernel(R* __restrict__ U
         constexpr int NC = 4;
         for (int k0 = threadIdx.x; k0 < ncnt; k0 += NC * blockDim.x) {
             int64_t so[NC];
-            int64_t dof[NC];
-            double w[NC];
-            int sq[NC];
+            int dof[NC], dir[NC];
             bool on[NC];
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
@@ -853,32 +852,31 @@ __global__ void __launch_bounds__(128) fill_interp_grid_kernel(R* __restrict__ U
                         x = cc < gx ? cc : pt.nx + cc;
                     }
                 }
-                int dir;
-                so[c] = neighbour_source_dir(pt, nb, on[c] ? x - gx : 0, on[c] ? y - gy : 0, on[c] ? iz : 0, dir);
-                sq[c] = s_sq[dir];
-                w[c] = s_w[dir];
-                dof[c] = (int64_t)y * X + x;
+                so[c] = neighbour_source_dir(pt, nb, on[c] ? x - gx : 0, on[c] ? y - gy : 0, on[c] ? iz : 0, dir[c]);
+                dof[c] = y * X + x;
             }
             R vc[NC][8], vo[NC][8];
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
-                const R* cur = (sq[c] ? U1 : U0) + so[c];
-                const R* old = (sq[c] ? U0 : U1) + so[c];
+                const int sq = s_sq[dir[c]], m = s_m[dir[c]];
+                const R* cur = (sq ? U1 : U0) + so[c];
+                const R* old = (sq ? U0 : U1) + so[c];
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
-                    vc[c][v] = on[c] ? cur[v * vol] : R(0);
-                    vo[c][v] = on[c] ? old[v * vol] : R(0);
+                    vc[c][v] = on[c] && m >= 0 ? cur[v * vol] : R(0);
+                    vo[c][v] = on[c] && m <= 0 ? old[v * vol] : R(0);
                 }
             }
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 if (!on[c]) continue;
-                const R wr = R(w[c]);
+                const R wr = s_w[dir[c]];
+                const int m = s_m[dir[c]];
                 R* d = plane + dof[c];
 #pragma unroll
                 for (int v = 0; v < 8; ++v) {
                     const R o = vo[c][v];
-                    d[v * vol] = w[c] >= 1.0 ? vc[c][v] : (w[c] <= 0.0 ? o : o + wr * (vc[c][v] - o));
+                    d[v * vol] = m > 0 ? vc[c][v] : (m < 0 ? o : o + wr * (vc[c][v] - o));
                 }
             }
         }
@@ -887,21 +885,25 @@ __global__ void __launch_bounds__(128) fill_interp_grid_kernel(R* __restrict__ U
 
 // a2 per listed patch: the maximum CFL rate over the patch's interior cells of its current
 // slice, as the bit pattern of a non-negative double in rate_max[p] (zeroed beforehand;
-// blocks along x share a patch and combine with an integer atomic max, which orders
+// the blocks of the grid share the listed patches out, several to a patch where there are few,
+// and combine with an integer atomic max, which orders
 // non-negative doubles as their values, so the result is exact and order independent).
 // The dt, courant / max rate, is taken by the asynchronous scheduler.  Non-finite rates
 // set ERR_PHYS and are left out of the maximum.
 template <typename R>
-__global__ void cfl_patch_kernel(const R* __restrict__ U0, const R* __restrict__ U1,
-                                 const PatchDev* __restrict__ patches, const int* __restrict__ list, int nlist,
-                                 const int* nlist_dev, const int* __restrict__ slice, double gamma_d, double dxi0_d,
+__global__ void cfl_patch_kernel(const R* U0, const R* U1,
+                                 const PatchDev* __restrict__ patches, const int* list, int nlist,
+                                 const int* nlist_dev, const int* slice, double gamma_d, double dxi0_d,
                                  double dxi1_d, double dxi2_d, int act1, int act2, unsigned long long* rate_max,
                                  unsigned* err) {
+    pdl_begin();
     __shared__ R red[32];
     const int nl = nlist_dev ? min(*nlist_dev, nlist) : nlist;
     const R gamma = R(gamma_d), gm1 = R(gamma_d - 1.0);
     const R dxi0 = R(dxi0_d), dxi1 = R(dxi1_d), dxi2 = R(dxi2_d);
-    for (int L = blockIdx.y; L < nl; L += gridDim.y) {
+    const int parts = max(1, min((int)gridDim.x / max(nl, 1), 128));
+    for (int64_t item = blockIdx.x; item < (int64_t)nl * parts; item += gridDim.x) {
+        const int L = (int)(item / parts), part = (int)(item - (int64_t)L * parts);
         const int p = list[L];
         const PatchDev pt = patches[p];
         const int n = pt.nx * pt.ny * pt.nz;
@@ -909,7 +911,8 @@ __global__ void cfl_patch_kernel(const R* __restrict__ U0, const R* __restrict__
         const R* base = (slice[p] ? U1 : U0) + pt.off;
         R vmax = R(0);
         bool bad = false;
-        for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
+#pragma unroll 2
+        for (int k = part * blockDim.x + threadIdx.x; k < n; k += parts * blockDim.x) {
             const int x = k % pt.nx + pt.gx, y = (k / pt.nx) % pt.ny + pt.gy, z = k / (pt.nx * pt.ny) + pt.gz;
             const R* c = base + ((int64_t)z * pt.Y + y) * pt.X + x;
             const R rate = cell_rate(c, vol, pt.X, pt.X * pt.Y, act1 != 0, act2 != 0, gamma, gm1, dxi0, dxi1, dxi2);

@@ -126,7 +126,6 @@ struct mhd_bunch {
     int* d_tcount = nullptr;
     int* d_rows_list = nullptr;
     double* d_rows_dt = nullptr;
-    unsigned char* d_rows_last = nullptr;
     int* d_rows_n = nullptr;
     int* d_ntiles = nullptr;
     unsigned* d_abort = nullptr;
@@ -408,7 +407,7 @@ int build_tiles(mhd_bunch* b) {
         CK(cudaMemcpy(T.d_lpt, lpt.data(), sizeof(int4) * T.n, cudaMemcpyHostToDevice));
     }
     // z-blocks of each configuration's launch over the whole bunch, and the configuration used when
-    // none is set: the shortest by step_time (the first one in 1D and 2D)
+    // none is set: the shortest by step_time
     double least = 0;
     for (size_t k = 0; k < b->cfg_index.size(); ++k) {
         const StepLaunch& L = step_cfg(b, (int)k);
@@ -842,7 +841,6 @@ int ensure_async(mhd_bunch* b) {
         CK(cudaMalloc(&b->d_tcount, sizeof(int) * P));
         CK(cudaMalloc(&b->d_rows_list, sizeof(int) * P * kAsyncRows));
         CK(cudaMalloc(&b->d_rows_dt, sizeof(double) * P * kAsyncRows));
-        CK(cudaMalloc(&b->d_rows_last, P * kAsyncRows));
         CK(cudaMalloc(&b->d_rows_n, sizeof(int) * kAsyncRows));
         CK(cudaMalloc(&b->d_ntiles, sizeof(int)));
         CK(cudaMalloc(&b->d_abort, sizeof(unsigned)));
@@ -1972,15 +1970,6 @@ int mhd_bunch_advance_async(mhd_bunch* b, double t_span, int max_rounds, int* ro
     b->log_patches.clear();
     b->log_dts.clear();
 
-    // the previous round's commit (prev < 0: none)
-    auto commit = [&](int prev) -> cudaError_t {
-        if (prev < 0) return cudaSuccess;
-        async_commit_kernel<<<std::max(1, b->nsm), 256, 0, st>>>(
-            b->d_rows_list + (size_t)prev * P, b->d_rows_n + prev, b->d_rows_dt + (size_t)prev * P,
-            b->d_rows_last + (size_t)prev * P, t_span, b->d_told, b->d_tcur, b->d_slice);
-        ++b->launches;
-        return cudaGetLastError();
-    };
     StepHostArgs a = step_args(b, nullptr, 0.0);
     a.U = b->buf[A];
     a.Unew = b->buf[1 - A];
@@ -2009,20 +1998,19 @@ int mhd_bunch_advance_async(mhd_bunch* b, double t_span, int max_rounds, int* ro
         for (int i = 0; i < kb; ++i) {
             int* row = b->d_rows_list + (size_t)i * P;
             int* nrow = b->d_rows_n + i;
-            CK(commit(prev));
-            async_ready_kernel<<<(P + 255) / 256, 256, 0, st>>>(P, b->d_nb_off, b->d_nb_idx, b->d_tcur, t_span,
-                                                                 b->d_abort, b->d_ready);
-            async_list_kernel<<<1, kSchedThreads, 0, st>>>(P, b->d_ready, b->d_tfirst, b->d_tcount, T.d_nat, row,
-                                                           nrow, b->d_atiles, b->d_ntiles, b->d_rmax);
+            launch_pdl(async_ready_kernel, (P + 7) / 8, 256, 0, st, P, b->d_nb_off, b->d_nb_idx, b->d_tcur, t_span,
+                       b->d_abort, b->d_ready);
+            launch_pdl(async_list_kernel, 1, kSchedThreads, 0, st, P, b->d_ready, b->d_tfirst, b->d_tcount, T.d_nat, row,
+                       nrow, b->d_atiles, b->d_ntiles, b->d_rmax, b->d_rows_list + (size_t)std::max(prev, 0) * P,
+                       prev < 0 ? nullptr : b->d_rows_n + prev, b->d_slice);
             CK(cudaGetLastError());
             // guard zones at each patch's own time, then its own CFL dt, clipped
             CK(b->K->fill_interp(b->buf[A], b->buf[1 - A], b->d_patches, P, row, P, nrow, list_blocks, b->d_slice,
                                  b->d_told, b->d_tcur, b->fg, b->d_nboff, b->hp[0].Z, pstride, b->d_err, st));
             CK(b->K->cfl_patch(b->buf[A], b->buf[1 - A], b->d_patches, row, P, nrow, list_blocks, b->d_slice,
                                b->gamma, dxi, act, b->d_rmax, b->d_err, st));
-            async_clamp_kernel<<<std::max(1, (P + 255) / 256), 256, 0, st>>>(
-                row, nrow, b->d_rmax, b->courant, b->d_tcur, t_span, b->d_dtp, b->d_rows_dt + (size_t)i * P,
-                b->d_rows_last + (size_t)i * P, b->d_abort, b->d_err);
+            launch_pdl(async_clamp_kernel, std::max(1, (P + 255) / 256), 256, 0, st, row, nrow, b->d_rmax, b->courant,
+                       b->d_told, b->d_tcur, t_span, b->d_dtp, b->d_rows_dt + (size_t)i * P, b->d_abort, b->d_err);
             CK(cudaGetLastError());
             // the update of the listed tiles, current slice -> the other, each by its own dt
             CK(L.launch(&a, step_grid, st));
@@ -2050,11 +2038,14 @@ int mhd_bunch_advance_async(mhd_bunch* b, double t_span, int max_rounds, int* ro
         r += m;
         if (m < kb) done = true;
     }
-    // commit the last round, then gather every patch's final slice into the current buffer
-    CK(commit(prev));
-    async_gather_kernel<<<dim3(16, std::min(P, 65535)), 256, 0, st>>>(
-        static_cast<unsigned*>(b->buf[A]), static_cast<const unsigned*>(b->buf[1 - A]), b->d_patches, P,
-        b->d_slice, b->rb / 4);
+    // the last round's slices flipped, then every patch's final slice into the current buffer
+    if (prev >= 0) {
+        launch_pdl(async_flip_kernel, (P + 255) / 256, 256, 0, st, b->d_rows_list + (size_t)prev * P, b->d_rows_n + prev,
+                   b->d_slice);
+        ++b->launches;
+    }
+    launch_pdl(async_gather_kernel, dim3(16, std::min(P, 65535)), 256, 0, st, static_cast<unsigned*>(b->buf[A]),
+               static_cast<const unsigned*>(b->buf[1 - A]), b->d_patches, P, b->d_slice, b->rb / 4);
     CK(cudaGetLastError());
     ++b->launches;
     std::vector<double> t_cur(P);
@@ -2116,7 +2107,6 @@ void mhd_bunch_destroy(mhd_bunch* b) {
     cudaFree(b->d_tcount);
     cudaFree(b->d_rows_list);
     cudaFree(b->d_rows_dt);
-    cudaFree(b->d_rows_last);
     cudaFree(b->d_rows_n);
     cudaFree(b->d_ntiles);
     cudaFree(b->d_abort);

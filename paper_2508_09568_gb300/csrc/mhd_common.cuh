@@ -66,6 +66,36 @@ struct FillGeom {
     const int* owner;     // [M2][M1][M0]
 };
 
+// The launches of an asynchronous round, six short kernels, are chained by programmatic dependent
+// launch: a kernel's CTAs become resident, and its launch latency passes, while the last CTAs of the
+// kernel before it still run.  pdl_begin() comes before everything that reads global memory in every
+// kernel launched by launch_pdl: it waits until the kernel before has finished and its writes are
+// visible (and, as that one waited too, all before it), then lets the next one come in.  What another
+// kernel of the chain writes is not read through a const __restrict__ pointer (such loads may be moved
+// across it).  Asynchronous 256^3 box of 512 patches, 64 rounds: 11.6 -> 10.8 ms.  The synchronous
+// kernels are launched plainly: of theirs the ones that wait take up SMs early and gain nothing
+// (512^3 box 21.35 -> 21.43 ms, 512^2 box, 4 steps, 118.7 -> 121.1 us when chained).
+__device__ __forceinline__ void pdl_begin() {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
+// k<<<grid, block, smem, s>>>(args...), chained to the kernel before it on the stream
+template <typename... P, typename... A>
+static inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);
+}
+
 // Device error word bits.
 enum : unsigned { ERR_PHYS = 1u, ERR_BOUNDS = 2u, ERR_TIMEOUT = 4u };
 

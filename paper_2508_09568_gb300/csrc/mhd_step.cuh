@@ -228,6 +228,8 @@ __device__ __forceinline__ void stage_plane(const R* __restrict__ U, const Patch
         const int wid = threadIdx.x >> 5;
         for (int v = (wid + C::NWARP - w0 % C::NWARP) % C::NWARP; v < 9; v += C::NWARP) {
             if ((threadIdx.x & 31) == 0) {
+                // what the CTA's threads did here before the barrier comes before the copy
+                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
                 const int64_t e0 = pt.off + (v == 8 ? 7 * vol + XY : v * vol) + (int64_t)z * XY + g.r0;
                 const int64_t e = e0 & ~(int64_t)(C::EQ - 1);
                 const unsigned bytes = (unsigned)(((int)(e0 - e) + g.rows * pt.X + C::EQ - 1) / C::EQ * 16);
@@ -534,15 +536,15 @@ __device__ __forceinline__ R line_emf(const R* P, int pid0, int pid1, int e, int
 // ---------------------------------------------------------------------------------------
 template <typename R>
 struct StepArgs {
-    const R* __restrict__ U;
-    R* __restrict__ Unew;
+    const R* U;
+    R* Unew;
     // asynchronous stepping (both null otherwise): patch p reads its current time slice
     // from buffer slice[p] (U when 0, Unew when 1) and writes the new one into the other
     // buffer, advancing by its own dt_patch[p]
-    const int* __restrict__ slice;
-    const double* __restrict__ dt_patch;
+    const int* slice;
+    const double* dt_patch;
     const PatchDev* __restrict__ patches;
-    const int4* __restrict__ tiles;
+    const int4* tiles;
     int ntiles;
     int nzb;              // 3D: z-blocks of a tile, each a work item (ASYNC: chosen from the tile count)
     const int* ntiles_dev;  // ASYNC: tile count written by the device scheduler (null: ntiles)
@@ -812,7 +814,6 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
     const int wid = threadIdx.x >> 5;
 
     if (threadIdx.x == 0) {
-        s_tile = a.dynamic ? atomicAdd(&a.work[0], 1) : (int)blockIdx.x;
         s_fail = 0;
         if constexpr (C::STAGED) {
             mbar_init(&s_bar[0], 27);
@@ -820,6 +821,8 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
             asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         }
     }
+    if constexpr (ASYNC) pdl_begin();
+    if (threadIdx.x == 0) s_tile = a.dynamic ? atomicAdd(&a.work[0], 1) : (int)blockIdx.x;
     __syncthreads();
     int t = s_tile;
     int ntiles = a.ntiles, nzb = ZB ? a.nzb : 1;

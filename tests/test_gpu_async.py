@@ -95,6 +95,27 @@ def test_async_many_rounds_and_max_rounds_cut():
         assert np.array_equal(d1, d2)
 
 
+@pytest.mark.parametrize("ncell,patch", [((36, 36, 36), (3, 3, 3)), ((40, 36, 48), (8, 6, 8)), ((17, 9, 33), (17, 9, 33))],
+                         ids=["1728_patches", "180_patches", "one_patch"])
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32], ids=["f64", "f32"])
+def test_async_round_of_the_whole_box_is_a_synchronous_step(ncell, patch, dtype):
+    """A span below every patch's own dt is one round of all patches with dt = span: bitwise the synchronous
+    step, from more listed planes and patches than the fill's and CFL pass's grids to a single one."""
+    from paper_2508_09568_gb300.bunch import MHDBunch
+    geom, U, meta = W.small_box(ncell=ncell, patch=patch, seed=35)
+    flat = W.to_patches(U, geom)
+    b = MHDBunch(geom, dtype=dtype, gamma=meta["gamma"])
+    b.upload(flat)
+    b.fill_guards()
+    span = 0.9 * b.cfl_dt()
+    b.step(span)
+    ref = interior_global(b.download(), geom)
+    b.upload(flat)
+    rounds, updates = b.advance_async(span)
+    assert (rounds, updates) == (1, geom.npatch)
+    assert np.array_equal(interior_global(b.download(), geom), ref)
+
+
 def test_async_nonphysical_state_is_reported():
     """Failure detection without a GPU fault: a patch whose every density is negative has no
     finite CFL rate, so its dt is not finite; the device scheduler sets that dt to 0 and
