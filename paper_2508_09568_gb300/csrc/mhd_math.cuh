@@ -137,10 +137,16 @@ MHD_HD void hancock_dw(const R q[8], const R dW[3][8], const R dxi[3], R hdt, R 
 // B^2): the value of fast_speed with the density divided out once at the end and both terms of
 // disc non-negative, so that nothing cancels when gamma P ~ Bn^2 and B is along n.  disc's
 // first term and s do not depend on the direction: a corner's two speeds share them.
-// Returns 2 rho c_f^2.
+// Returns 2 rho c_f^2; root: sqrt(disc).
+template <typename R>
+MHD_HD R fast_h(R gP4, R s, R dd, R bt2, R& root) {
+    root = rsqrt_(fma_(gP4, bt2, dd));
+    return s + root;
+}
 template <typename R>
 MHD_HD R fast_h(R gP4, R s, R dd, R bt2) {
-    return s + rsqrt_(fma_(gP4, bt2, dd));
+    R root;
+    return fast_h(gP4, s, dd, bt2, root);
 }
 
 // HLLD flux (Sec. 2.1.2; Miyoshi & Kusano 2005) through a face with normal field bn.
@@ -321,9 +327,9 @@ struct Corner {
     R rho, p, ua, ub, Ba, Bb, Be;
 };
 
-// fast speeds of a corner state along a and b
+// fast speeds of a corner state along a and b (double precision: and their inner square roots)
 template <typename R>
-MHD_HD void corner_speeds(const Corner<R>& s, R gamma, R& cfa, R& cfb) {
+MHD_HD void corner_speeds(const Corner<R>& s, R gamma, R& cfa, R& cfb, R& ra, R& rb) {
     if constexpr (sizeof(R) == 8) {
         const R hri = R(0.5) * rcp_(s.rho), gP4 = R(4) * gamma * s.p;
         const R be2 = s.Be * s.Be;
@@ -331,9 +337,10 @@ MHD_HD void corner_speeds(const Corner<R>& s, R gamma, R& cfa, R& cfb) {
         const R b2 = fma_(s.Ba, s.Ba, ta);
         const R sf = fma_(gamma, s.p, b2), df = fma_(gamma, s.p, -b2);
         const R dd = df * df;
-        cfa = rsqrt_(fast_h(gP4, sf, dd, ta) * hri);
-        cfb = rsqrt_(fast_h(gP4, sf, dd, tb) * hri);
+        cfa = rsqrt_(fast_h(gP4, sf, dd, ta, ra) * hri);
+        cfb = rsqrt_(fast_h(gP4, sf, dd, tb, rb) * hri);
     } else {   // the rounding of fast_speed (see hlld)
+        ra = rb = R(0);
         const R ri = rcp_(s.rho), gP = gamma * s.p;
         cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
         cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
@@ -353,8 +360,8 @@ MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, co
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const Corner<R>& s = *st[k];
-        R cfa, cfb;
-        corner_speeds(s, gamma, cfa, cfb);
+        R cfa, cfb, ra, rb;
+        corner_speeds(s, gamma, cfa, cfb, ra, rb);
         ap[k] = s.ua + cfa;
         am[k] = s.ua - cfa;
         bp[k] = s.ub + cfb;

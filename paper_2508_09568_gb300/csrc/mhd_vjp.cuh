@@ -71,6 +71,26 @@ MHD_HD void fast_speed_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R lcf, R& lr
     lrho -= (lcs2 * cs2 + lcan2 * can2 + lcat2 * cat2) * ri;
 }
 
+// The same for the form the double-precision solvers take, c_f = sqrt((s + root) / (2 rho)), root =
+// sqrt(disc) (fast_h), from the speed and the root that the forward code found: no square root and
+// half the operations.
+template <typename R>
+MHD_HD void fast_h_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R cf, R root, R lcf, R& lrho, R& lP, R& lbn, R& lbt1,
+                       R& lbt2) {
+    const R hri = R(0.5) * rcp_(rho), gP = gamma * P;
+    const R t = fma_(bt1, bt1, bt2 * bt2), d = gP - fma_(bn, bn, t);
+    const R lx = lcf * hri;
+    const R lh = positive_(cf) ? R(0.5) * lx * rcp_(cf) : R(0);      // of s + root
+    const R ld = positive_(root) ? lh * rcp_(root) : R(0);           // of disc, twice
+    const R lb = fma_(-ld, d, lh);                                   // of B^2
+    const R l2 = R(2) * lb, lt = fma_(R(4) * gP, ld, l2);
+    lP += gamma * fma_(ld, fma_(R(2), t, d), lh);
+    lbn += l2 * bn;
+    lbt1 += lt * bt1;
+    lbt2 += lt * bt2;
+    lrho -= lx * cf;
+}
+
 // d cons_to_prim: lq[8] -> lU (rho, mx, my, mz, E) and lbc[3] (cell-centred field)
 template <typename R>
 MHD_HD void cons_to_prim_vjp(R rho, R mx, R my, R mz, R E, R bxc, R byc, R bzc, R gm1, const R lq[8], R lU[5],
@@ -156,15 +176,28 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const R bn2 = bn * bn;
     const R rl = L[0], ul = L[1], vl = L[2], wl = L[3], pl = L[4], byl = L[5], bzl = L[6];
     const R rr = Rt[0], ur = Rt[1], vr = Rt[2], wr = Rt[3], pr = Rt[4], byr = Rt[5], bzr = Rt[6];
-    const R b2l = bn2 + byl * byl + bzl * bzl, b2r = bn2 + byr * byr + bzr * bzr;
+    const R btl = byl * byl + bzl * bzl, btr = byr * byr + bzr * bzr;
+    const R b2l = bn2 + btl, b2r = bn2 + btr;
     const R ptl = pl + R(0.5) * b2l, ptr = pr + R(0.5) * b2r;
     const R el = pl * gm1i + R(0.5) * rl * (ul * ul + vl * vl + wl * wl) + R(0.5) * b2l;
     const R er = pr * gm1i + R(0.5) * rr * (ur * ur + vr * vr + wr * wr) + R(0.5) * b2r;
-    const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
-    const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
     const R vbl = ul * bn + vl * byl + wl * bzl, vbr = ur * bn + vr * byr + wr * bzr;
-    const bool cl = !greater_(cfr, cfl);   // max picks cf_L
-    const R cmax = cl ? cfl : cfr;
+    bool cl;   // max picks cf_L
+    R cmax, croot = 0;
+    if constexpr (sizeof(R) == 8) {
+        const R g4 = R(4) * gamma, gpl = gamma * pl, gpr = gamma * pr;
+        R rootl, rootr;
+        const R hl = fast_h(g4 * pl, gpl + b2l, (gpl - b2l) * (gpl - b2l), btl, rootl) * rcp_(rl);
+        const R hr = fast_h(g4 * pr, gpr + b2r, (gpr - b2r) * (gpr - b2r), btr, rootr) * rcp_(rr);
+        cl = !greater_(hr, hl);
+        cmax = rsqrt_(R(0.5) * (cl ? hl : hr));
+        croot = cl ? rootl : rootr;
+    } else {
+        const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
+        const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
+        cl = !greater_(cfr, cfl);
+        cmax = cl ? cfl : cfr;
+    }
     const bool ml = !greater_(ul, ur);     // min picks u_L
     const bool Ml = !greater_(ur, ul);     // max picks u_L
     const R sl = (ml ? ul : ur) - cmax;
@@ -181,13 +214,16 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         R S, sa, ssm, ssmi, rs, D, Di, nu, nb, vs, ws, bys, bzs, vbs, nes, es;
         bool deg;
     };
-    auto star = [&](R S, R r, R u, R v, R w, R by, R bz, R pt, R e, R vb) {
-        Star t;
+    auto star = [&](R S, R r, R u) {
+        Star t{};
         t.S = S;
         t.sa = S - u;
         t.ssm = S - sm;
         t.ssmi = rcp_(t.ssm);
         t.rs = r * t.sa * t.ssmi;
+        return t;
+    };
+    auto star_rest = [&](Star& t, R r, R u, R v, R w, R by, R bz, R pt, R e, R vb) {
         t.D = r * t.sa * t.ssm - bn2;
         t.deg = le_mag_(rabs(t.D), eps * bn2);
         const R Di = t.deg ? R(0) : rcp_(t.D);
@@ -201,24 +237,13 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         t.vbs = sm * bn + t.vs * t.bys + t.ws * t.bzs;
         t.nes = t.sa * e - pt * u + pts * sm + bn * (vb - t.vbs);
         t.es = t.nes * t.ssmi;
-        return t;
     };
-    const Star A = star(sl, rl, ul, vl, wl, byl, bzl, ptl, el, vbl);
-    const Star B = star(sr, rr, ur, vr, wr, byr, bzr, ptr, er, vbr);
+    Star A = star(sl, rl, ul), B = star(sr, rr, ur);
     const R sql = rsqrt_(A.rs), sqr = rsqrt_(B.rs);
     const R abn = rabs(bn);
     const R isql = rcp_(sql), isqr = rcp_(sqr);
     const R ssl = sm - abn * isql, ssr = sm + abn * isqr;
     const R sgn = nonzero_(bn) ? copysign(R(1), bn) : R(0);
-    const R isum = rcp_(sql + sqr);
-    const R nv = sql * A.vs + sqr * B.vs + (B.bys - A.bys) * sgn;
-    const R nw = sql * A.ws + sqr * B.ws + (B.bzs - A.bzs) * sgn;
-    const R nby = sql * B.bys + sqr * A.bys + sql * sqr * (B.vs - A.vs) * sgn;
-    const R nbz = sql * B.bzs + sqr * A.bzs + sql * sqr * (B.ws - A.ws) * sgn;
-    const R vss = nv * isum, wss = nw * isum, byss = nby * isum, bzss = nbz * isum;
-    const R vbss = sm * bn + vss * byss + wss * bzss;
-    const R essl = A.es - sql * (A.vbs - vbss) * sgn;
-    const R essr = B.es + sqr * (B.vbs - vbss) * sgn;
     int reg = 5;
     if (nonneg_(sr)) reg = 4;
     if (nonneg_(ssr)) reg = 3;
@@ -226,6 +251,12 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     if (nonneg_(ssl)) reg = 1;
     if (nonneg_(sl)) reg = 0;
     const bool left = reg <= 2;
+    // What only some regions use is formed, and reversed, there alone: the rest of a side's star state
+    // beside its own star and the double star, a side's energy and v.B where its state or star counts
+    // (neighbouring faces, and so a warp's lanes, are mostly of one region).
+    const bool dstar = reg == 2 || reg == 3, starA = reg >= 1 && reg <= 3, starB = reg >= 2 && reg <= 4;
+    if (starA) star_rest(A, rl, ul, vl, wl, byl, bzl, ptl, el, vbl);
+    if (starB) star_rest(B, rr, ur, vr, wr, byr, bzr, ptr, er, vbr);
 
     // ----- reverse
     R g_rl = 0, g_ul = 0, g_vl = 0, g_wl = 0, g_pl = 0, g_byl = 0, g_bzl = 0;
@@ -271,10 +302,17 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
             g_e0 -= S * lF[4];
             R gUs0 = S * lF[0], gUs1 = S * lF[1], gUs2 = S * lF[2], gUs3 = S * lF[3], gUs4 = S * lF[4];
             R g_rs = 0, g_vs = 0, g_ws = 0, g_es = 0;
-            if (reg == 2 || reg == 3) {
+            if (dstar) {
+                const R isum = rcp_(sql + sqr);
+                const R nv = sql * A.vs + sqr * B.vs + (B.bys - A.bys) * sgn;
+                const R nw = sql * A.ws + sqr * B.ws + (B.bzs - A.bzs) * sgn;
+                const R nby = sql * B.bys + sqr * A.bys + sql * sqr * (B.vs - A.vs) * sgn;
+                const R nbz = sql * B.bzs + sqr * A.bzs + sql * sqr * (B.ws - A.ws) * sgn;
+                const R vss = nv * isum, wss = nw * isum, byss = nby * isum, bzss = nbz * isum;
+                const R vbss = sm * bn + vss * byss + wss * bzss;
                 // f += S* (U** - U*), U** - U* = (0, 0, rs (vss - vs), rs (wss - ws), ess - es)
                 const R Ss = left ? ssl : ssr;
-                const R ess = left ? essl : essr;
+                const R ess = left ? A.es - sql * (A.vbs - vbss) * sgn : B.es + sqr * (B.vbs - vbss) * sgn;
                 const R gSs = lF[2] * T.rs * (vss - T.vs) + lF[3] * T.rs * (wss - T.ws) + lF[4] * (ess - T.es);
                 g_rs += Ss * (lF[2] * (vss - T.vs) + lF[3] * (wss - T.ws));
                 const R g_vss = Ss * lF[2] * T.rs, g_wss = Ss * lF[3] * T.rs;
@@ -440,9 +478,9 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         g_sm -= g_ssm;
         g_u -= g_sa;
     };
-    star_rev(B, rr, ur, vr, wr, byr, bzr, ptr, er, vbr, gB_rs, gB_vs, gB_ws, gB_bys, gB_bzs, gB_vbs, gB_es, g_rr, g_ur,
+    if (starB) star_rev(B, rr, ur, vr, wr, byr, bzr, ptr, er, vbr, gB_rs, gB_vs, gB_ws, gB_bys, gB_bzs, gB_vbs, gB_es, g_rr, g_ur,
              g_vr, g_wr, g_byr, g_bzr, g_ptr, g_er, g_vbr, g_sr);
-    star_rev(A, rl, ul, vl, wl, byl, bzl, ptl, el, vbl, gA_rs, gA_vs, gA_ws, gA_bys, gA_bzs, gA_vbs, gA_es, g_rl, g_ul,
+    if (starA) star_rev(A, rl, ul, vl, wl, byl, bzl, ptl, el, vbl, gA_rs, gA_vs, gA_ws, gA_bys, gA_bzs, gA_vbs, gA_es, g_rl, g_ul,
              g_vl, g_wl, g_byl, g_bzl, g_ptl, g_el, g_vbl, g_sl);
     // sm = smn / den ; pts = ptn / den
     const R g_smn = g_sm * deni, g_ptn = g_pts * deni;
@@ -477,23 +515,39 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     else g_ur += g_sl;
     if (Ml) g_ul += g_sr;
     else g_ur += g_sr;
-    R g_cfl = cl ? g_cmax : R(0), g_cfr = cl ? R(0) : g_cmax;
-    // vb = u bn + v by + w bz
-    g_ul += g_vbl * bn; g_bn += g_vbl * ul; g_vl += g_vbl * byl; g_byl += g_vbl * vl; g_wl += g_vbl * bzl;
-    g_bzl += g_vbl * wl;
-    g_ur += g_vbr * bn; g_bn += g_vbr * ur; g_vr += g_vbr * byr; g_byr += g_vbr * vr; g_wr += g_vbr * bzr;
-    g_bzr += g_vbr * wr;
-    // fast speeds
-    fast_speed_vjp(rl, pl, bn, byl, bzl, gamma, g_cfl, g_rl, g_pl, g_bn, g_byl, g_bzl);
-    fast_speed_vjp(rr, pr, bn, byr, bzr, gamma, g_cfr, g_rr, g_pr, g_bn, g_byr, g_bzr);
-    // e = p gm1i + rho |u|^2 / 2 + b2 / 2 ; pt = p + b2 / 2
-    R g_b2l = R(0.5) * g_el + R(0.5) * g_ptl, g_b2r = R(0.5) * g_er + R(0.5) * g_ptr;
-    g_pl += g_el * gm1i + g_ptl;
-    g_pr += g_er * gm1i + g_ptr;
-    g_rl += g_el * R(0.5) * (ul * ul + vl * vl + wl * wl);
-    g_rr += g_er * R(0.5) * (ur * ur + vr * vr + wr * wr);
-    g_ul += g_el * rl * ul; g_vl += g_el * rl * vl; g_wl += g_el * rl * wl;
-    g_ur += g_er * rr * ur; g_vr += g_er * rr * vr; g_wr += g_er * rr * wr;
+    // the fast speed of the side that the max picked
+    {
+        R h_r = 0, h_p = 0, h_by = 0, h_bz = 0;
+        const R r0 = cl ? rl : rr, p0 = cl ? pl : pr, by0 = cl ? byl : byr, bz0 = cl ? bzl : bzr;
+        if constexpr (sizeof(R) == 8)
+            fast_h_vjp(r0, p0, bn, by0, bz0, gamma, cmax, croot, g_cmax, h_r, h_p, g_bn, h_by, h_bz);
+        else
+            fast_speed_vjp(r0, p0, bn, by0, bz0, gamma, g_cmax, h_r, h_p, g_bn, h_by, h_bz);
+        if (cl) {
+            g_rl += h_r; g_pl += h_p; g_byl += h_by; g_bzl += h_bz;
+        } else {
+            g_rr += h_r; g_pr += h_p; g_byr += h_by; g_bzr += h_bz;
+        }
+    }
+    // vb = u bn + v by + w bz ; e = p gm1i + rho |u|^2 / 2 + b2 / 2
+    if (reg <= 3) {
+        g_ul += g_vbl * bn; g_bn += g_vbl * ul; g_vl += g_vbl * byl; g_byl += g_vbl * vl; g_wl += g_vbl * bzl;
+        g_bzl += g_vbl * wl;
+        g_pl += g_el * gm1i;
+        g_rl += g_el * R(0.5) * (ul * ul + vl * vl + wl * wl);
+        g_ul += g_el * rl * ul; g_vl += g_el * rl * vl; g_wl += g_el * rl * wl;
+    }
+    if (reg >= 2) {
+        g_ur += g_vbr * bn; g_bn += g_vbr * ur; g_vr += g_vbr * byr; g_byr += g_vbr * vr; g_wr += g_vbr * bzr;
+        g_bzr += g_vbr * wr;
+        g_pr += g_er * gm1i;
+        g_rr += g_er * R(0.5) * (ur * ur + vr * vr + wr * wr);
+        g_ur += g_er * rr * ur; g_vr += g_er * rr * vr; g_wr += g_er * rr * wr;
+    }
+    // pt = p + b2 / 2 (and the b2 / 2 of e)
+    const R g_b2l = R(0.5) * g_el + R(0.5) * g_ptl, g_b2r = R(0.5) * g_er + R(0.5) * g_ptr;
+    g_pl += g_ptl;
+    g_pr += g_ptr;
     // b2 = bn2 + by^2 + bz^2
     g_bn2 += g_b2l + g_b2r;
     g_byl += R(2) * byl * g_b2l; g_bzl += R(2) * bzl * g_b2l;
@@ -632,50 +686,54 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
                       R lE, Corner<R>& gSW, Corner<R>& gSE, Corner<R>& gNW, Corner<R>& gNE) {
     const Corner<R>* st[4] = {&SW, &SE, &NW, &NE};
     Corner<R>* gs[4] = {&gSW, &gSE, &gNW, &gNE};
-    R ap[4], am[4], bp[4], bm[4];
+    R ap[4], am[4], bp[4], bm[4], ca[4], cb[4], ra[4], rb[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const Corner<R>& s = *st[k];
-        R cfa, cfb;
-        corner_speeds(s, gamma, cfa, cfb);
-        ap[k] = s.ua + cfa;
-        am[k] = s.ua - cfa;
-        bp[k] = s.ub + cfb;
-        bm[k] = s.ub - cfb;
+        corner_speeds(s, gamma, ca[k], cb[k], ra[k], rb[k]);
+        ap[k] = s.ua + ca[k];
+        am[k] = s.ua - ca[k];
+        bp[k] = s.ub + cb[k];
+        bm[k] = s.ub - cb[k];
     }
-    // folds with the selected index (-1: the clip at zero won)
-    auto fold_max = [](const R* x, int& k) {
+    // folds with the selected index (-1: the clip at zero won) and what the selected speed came from
+    struct Pick {
+        int k;
+        R c, root;
+    };
+    auto fold_max = [](const R* x, const R* c, const R* r, Pick& p) {
         R m = x[0];
-        k = 0;
+        p = {0, c[0], r[0]};
 #pragma unroll
         for (int j = 1; j < 4; ++j)
             if (greater_(x[j], m)) {
                 m = x[j];
-                k = j;
+                p = {j, c[j], r[j]};
             }
         if (!nonneg_(m)) {
             m = R(0);
-            k = -1;
+            p.k = -1;
         }
         return m;
     };
-    auto fold_min = [](const R* x, int& k) {
+    auto fold_min = [](const R* x, const R* c, const R* r, Pick& p) {
         R m = x[0];
-        k = 0;
+        p = {0, c[0], r[0]};
 #pragma unroll
         for (int j = 1; j < 4; ++j)
             if (greater_(m, x[j])) {
                 m = x[j];
-                k = j;
+                p = {j, c[j], r[j]};
             }
         if (positive_(m)) {
             m = R(0);
-            k = -1;
+            p.k = -1;
         }
         return m;
     };
-    int kE, kW, kN, kS;
-    const R sE = fold_max(ap, kE), sW = fold_min(am, kW), sN = fold_max(bp, kN), sS = fold_min(bm, kS);
+    Pick kE, kW, kN, kS;
+    const R sE = fold_max(ap, ca, ra, kE), sW = fold_min(am, ca, ra, kW), sN = fold_max(bp, cb, rb, kN),
+            sS = fold_min(bm, cb, rb, kS);
     const R da = sE - sW, db = sN - sS;
     R e[4];
 #pragma unroll
@@ -718,14 +776,19 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
     // is selected by value, the result added by testing every corner, so that every index is a
     // compile-time constant and the corner cotangents stay in registers (four reverse fast speeds
     // instead of one per corner and direction).
-    auto speed = [&](int k, R g, bool alongb, R sgn) {
+    auto speed = [&](const Pick& pick, R g, bool alongb, R sgn) {
+        const int k = pick.k;
         if (k < 0) return;
         Corner<R> s = *st[0];
 #pragma unroll
         for (int j = 1; j < 4; ++j)
             if (j == k) s = *st[j];
         R lrho = R(0), lp = R(0), lbn = R(0), lbt = R(0), lbe = R(0);
-        fast_speed_vjp(s.rho, s.p, alongb ? s.Bb : s.Ba, alongb ? s.Ba : s.Bb, s.Be, gamma, sgn * g, lrho, lp, lbn, lbt, lbe);
+        const R bn = alongb ? s.Bb : s.Ba, bt = alongb ? s.Ba : s.Bb;
+        if constexpr (sizeof(R) == 8)
+            fast_h_vjp(s.rho, s.p, bn, bt, s.Be, gamma, pick.c, pick.root, sgn * g, lrho, lp, lbn, lbt, lbe);
+        else
+            fast_speed_vjp(s.rho, s.p, bn, bt, s.Be, gamma, sgn * g, lrho, lp, lbn, lbt, lbe);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if (j != k) continue;
