@@ -341,9 +341,10 @@ __device__ __forceinline__ void adj_corner_scatter(const AdjArgs<R>& a, int64_t 
     const R gv[5] = {g.rho, g.p, g.ua, g.ub, g.Be};
 #pragma unroll
     for (int n = 0; n < 5; ++n) {
+        const R h = R(0.5) * gv[n];
         aadd(&fat(a.G, AF_WH + ks[n], i), gv[n]);
-        aadd(&fat(a.G, AF_DW + 8 * A + ks[n], i), R(0.5 * sa) * gv[n]);
-        aadd(&fat(a.G, AF_DW + 8 * B + ks[n], i), R(0.5 * sb) * gv[n]);
+        aadd(&fat(a.G, AF_DW + 8 * A + ks[n], i), sa > 0 ? h : -h);
+        aadd(&fat(a.G, AF_DW + 8 * B + ks[n], i), sb > 0 ? h : -h);
     }
     aadd(&fat(a.G, AF_BH + A, fa), g.Ba);
     aadd(&fat(a.G, AF_FS + 2 * A + 0, fa), R(0.5 * sb) * g.Ba);

@@ -179,9 +179,6 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const R btl = byl * byl + bzl * bzl, btr = byr * byr + bzr * bzr;
     const R b2l = bn2 + btl, b2r = bn2 + btr;
     const R ptl = pl + R(0.5) * b2l, ptr = pr + R(0.5) * b2r;
-    const R el = pl * gm1i + R(0.5) * rl * (ul * ul + vl * vl + wl * wl) + R(0.5) * b2l;
-    const R er = pr * gm1i + R(0.5) * rr * (ur * ur + vr * vr + wr * wr) + R(0.5) * b2r;
-    const R vbl = ul * bn + vl * byl + wl * bzl, vbr = ur * bn + vr * byr + wr * bzr;
     bool cl;   // max picks cf_L
     R cmax, croot = 0;
     if constexpr (sizeof(R) == 8) {
@@ -209,279 +206,237 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const R ptn = dr * ptl - dl * ptr + dl * dr * (ur - ul);
     const R sm = smn * deni;
     const R pts = ptn * deni;
-    // star states, per side
-    struct Star {
-        R S, sa, ssm, ssmi, rs, D, Di, nu, nb, vs, ws, bys, bzs, vbs, nes, es;
-        bool deg;
+    // density of the star states, Alfven speeds, and the region at x/t = 0
+    struct Side {   // a side's state and what all regions need of its star state
+        R r, u, v, w, p, by, bz, b2, pt, S, sa, ssm, ssmi, rs, sq, isq;
     };
-    auto star = [&](R S, R r, R u) {
-        Star t{};
-        t.S = S;
-        t.sa = S - u;
+    auto side = [&](const R* W, R b2, R pt, R S) {
+        Side t{W[0], W[1], W[2], W[3], W[4], W[5], W[6], b2, pt, S};
+        t.sa = S - t.u;
         t.ssm = S - sm;
         t.ssmi = rcp_(t.ssm);
-        t.rs = r * t.sa * t.ssmi;
+        t.rs = t.r * t.sa * t.ssmi;
+        t.sq = rsqrt_(t.rs);
+        t.isq = rcp_(t.sq);
         return t;
     };
-    auto star_rest = [&](Star& t, R r, R u, R v, R w, R by, R bz, R pt, R e, R vb) {
-        t.D = r * t.sa * t.ssm - bn2;
-        t.deg = le_mag_(rabs(t.D), eps * bn2);
-        const R Di = t.deg ? R(0) : rcp_(t.D);
-        t.Di = Di;
-        t.nu = bn * (sm - u) * Di;
-        t.nb = (r * t.sa * t.sa - bn2) * Di;
-        t.vs = t.deg ? v : v - by * t.nu;
-        t.ws = t.deg ? w : w - bz * t.nu;
-        t.bys = t.deg ? by : by * t.nb;
-        t.bzs = t.deg ? bz : bz * t.nb;
-        t.vbs = sm * bn + t.vs * t.bys + t.ws * t.bzs;
-        t.nes = t.sa * e - pt * u + pts * sm + bn * (vb - t.vbs);
-        t.es = t.nes * t.ssmi;
-    };
-    Star A = star(sl, rl, ul), B = star(sr, rr, ur);
-    const R sql = rsqrt_(A.rs), sqr = rsqrt_(B.rs);
+    const Side A = side(L, b2l, ptl, sl), B = side(Rt, b2r, ptr, sr);
     const R abn = rabs(bn);
-    const R isql = rcp_(sql), isqr = rcp_(sqr);
-    const R ssl = sm - abn * isql, ssr = sm + abn * isqr;
     const R sgn = nonzero_(bn) ? copysign(R(1), bn) : R(0);
     int reg = 5;
     if (nonneg_(sr)) reg = 4;
-    if (nonneg_(ssr)) reg = 3;
+    if (nonneg_(sm + abn * B.isq)) reg = 3;
     if (nonneg_(sm)) reg = 2;
-    if (nonneg_(ssl)) reg = 1;
+    if (nonneg_(sm - abn * A.isq)) reg = 1;
     if (nonneg_(sl)) reg = 0;
-    const bool left = reg <= 2;
-    // What only some regions use is formed, and reversed, there alone: the rest of a side's star state
-    // beside its own star and the double star, a side's energy and v.B where its state or star counts
-    // (neighbouring faces, and so a warp's lanes, are mostly of one region).
-    const bool dstar = reg == 2 || reg == 3, starA = reg >= 1 && reg <= 3, starB = reg >= 2 && reg <= 4;
-    if (starA) star_rest(A, rl, ul, vl, wl, byl, bzl, ptl, el, vbl);
-    if (starB) star_rest(B, rr, ur, vr, wr, byr, bzr, ptr, er, vbr);
+    const bool left = reg <= 2, dstar = reg == 2 || reg == 3;
 
-    // ----- reverse
-    R g_rl = 0, g_ul = 0, g_vl = 0, g_wl = 0, g_pl = 0, g_byl = 0, g_bzl = 0;
-    R g_rr = 0, g_ur = 0, g_vr = 0, g_wr = 0, g_pr = 0, g_byr = 0, g_bzr = 0;
-    R g_bn = 0, g_bn2 = 0, g_ptl = 0, g_ptr = 0, g_el = 0, g_er = 0, g_vbl = 0, g_vbr = 0;
-    R g_sl = 0, g_sr = 0, g_sm = 0, g_pts = 0;
-    // per-side star adjoints
-    R gA_rs = 0, gA_vs = 0, gA_ws = 0, gA_bys = 0, gA_bzs = 0, gA_vbs = 0, gA_es = 0;
-    R gB_rs = 0, gB_vs = 0, gB_ws = 0, gB_bys = 0, gB_bzs = 0, gB_vbs = 0, gB_es = 0;
-    R g_sql = 0, g_sqr = 0, g_abn = 0;
+    // ----- reverse, in terms of the near side (that of x/t = 0: field by field, so that lanes of either
+    // side take one path) and the far side, whose star state only the double star uses; with sg =
+    // sgn on the left, -sgn on the right, and tau = 1, -1 the formulas of the two sides are one.
+    auto pick = [&](bool l) {
+        Side t;
+        t.r = sel(l, A.r, B.r); t.u = sel(l, A.u, B.u); t.v = sel(l, A.v, B.v); t.w = sel(l, A.w, B.w);
+        t.p = sel(l, A.p, B.p); t.by = sel(l, A.by, B.by); t.bz = sel(l, A.bz, B.bz); t.b2 = sel(l, A.b2, B.b2);
+        t.pt = sel(l, A.pt, B.pt); t.S = sel(l, A.S, B.S); t.sa = sel(l, A.sa, B.sa); t.ssm = sel(l, A.ssm, B.ssm);
+        t.ssmi = sel(l, A.ssmi, B.ssmi); t.rs = sel(l, A.rs, B.rs); t.sq = sel(l, A.sq, B.sq); t.isq = sel(l, A.isq, B.isq);
+        return t;
+    };
+    const Side N = pick(left), O = pick(!left);
+    const R sg = left ? sgn : -sgn, tabn = left ? abn : -abn;
+    struct SideGrad {   // cotangents of a side's state (pt, e and v.B as they come), its wave speed
+        R r = 0, u = 0, v = 0, w = 0, p = 0, by = 0, bz = 0, pt = 0, e = 0, vb = 0, S = 0;
+    } gn, go;
+    R g_bn = 0, g_bn2 = 0, g_sm = 0, g_pts = 0, g_tabn = 0;
+    struct Energy {
+        R kin, e, vb;
+    };
+    auto energy = [&](const Side& T) {   // u^2 / 2, e = p gm1i + r u^2 / 2 + b2 / 2, v.B
+        const R kin = R(0.5) * (T.u * T.u + T.v * T.v + T.w * T.w);
+        return Energy{kin, T.p * gm1i + T.r * kin + R(0.5) * T.b2, T.u * bn + T.v * T.by + T.w * T.bz};
+    };
+    auto energy_rev = [&](const Side& T, const Energy& E, SideGrad& g) {   // (b2 / 2 comes with pt's)
+        g.u += g.vb * bn; g_bn += g.vb * T.u; g.v += g.vb * T.by; g.by += g.vb * T.v; g.w += g.vb * T.bz; g.bz += g.vb * T.w;
+        g.p += g.e * gm1i;
+        g.r += g.e * E.kin;
+        const R er = g.e * T.r;
+        g.u += er * T.u; g.v += er * T.v; g.w += er * T.w;
+    };
+    struct Star {
+        R Di, nu, nb, vs, ws, bys, bzs, vbs, es;
+        bool deg;
+    };
+    auto star = [&](const Side& T, const Energy& E) {
+        Star t;
+        const R D = T.r * T.sa * T.ssm - bn2;
+        t.deg = le_mag_(rabs(D), eps * bn2);
+        t.Di = t.deg ? R(0) : rcp_(D);
+        t.nu = bn * (sm - T.u) * t.Di;
+        t.nb = (T.r * T.sa * T.sa - bn2) * t.Di;
+        t.vs = t.deg ? T.v : T.v - T.by * t.nu;
+        t.ws = t.deg ? T.w : T.w - T.bz * t.nu;
+        t.bys = t.deg ? T.by : T.by * t.nb;
+        t.bzs = t.deg ? T.bz : T.bz * t.nb;
+        t.vbs = sm * bn + t.vs * t.bys + t.ws * t.bzs;
+        t.es = (T.sa * E.e - T.pt * T.u + pts * sm + bn * (E.vb - t.vbs)) * T.ssmi;
+        return t;
+    };
+    struct StarGrad {
+        R rs = 0, vs = 0, ws = 0, bys = 0, bzs = 0, vbs = 0, es = 0, sq = 0;
+    };
+    auto star_rev = [&](const Side& T, const Energy& E, const Star& t, StarGrad h, SideGrad& g) {
+        // sq = sqrt(rs)
+        h.rs += R(0.5) * h.sq * T.isq;
+        // es = nes * ssmi
+        const R g_nes = h.es * T.ssmi;
+        R g_ssm = -g_nes * t.es;
+        // nes = sa e - pt u + pts sm + bn (vb - vbs)
+        R g_sa = g_nes * E.e;
+        g.e += g_nes * T.sa;
+        g.pt -= g_nes * T.u;
+        g.u -= g_nes * T.pt;
+        g_pts += g_nes * sm;
+        g_sm += g_nes * pts;
+        g_bn += g_nes * (E.vb - t.vbs);
+        g.vb += g_nes * bn;
+        h.vbs -= g_nes * bn;
+        // vbs = sm bn + vs bys + ws bzs
+        g_sm += h.vbs * bn;
+        g_bn += h.vbs * sm;
+        h.vs += h.vbs * t.bys;
+        h.bys += h.vbs * t.vs;
+        h.ws += h.vbs * t.bzs;
+        h.bzs += h.vbs * t.ws;
+        g.v += h.vs;
+        g.w += h.ws;
+        if (!t.deg) {
+            g.by += h.bys * t.nb - h.vs * t.nu;
+            g.bz += h.bzs * t.nb - h.ws * t.nu;
+            // nu = bn (sm - u) / D, nb = (r sa^2 - bn2) / D
+            const R g_nu = -(h.vs * T.by + h.ws * T.bz) * t.Di, g_nb = (h.bys * T.by + h.bzs * T.bz) * t.Di;
+            g_bn += g_nu * (sm - T.u);
+            g_sm += g_nu * bn;
+            g.u -= g_nu * bn;
+            const R g_D = -(g_nu * t.nu + g_nb * t.nb);
+            const R bsa = g_nb * T.sa;
+            g.r += bsa * T.sa;
+            g_sa += R(2) * bsa * T.r;
+            g_bn2 -= g_nb + g_D;
+            // D = r sa ssm - bn2
+            const R dss = g_D * T.ssm, dr_ = g_D * T.r;
+            g.r += dss * T.sa;
+            g_sa += dss * T.r;
+            g_ssm += dr_ * T.sa;
+        } else {
+            g.by += h.bys;
+            g.bz += h.bzs;
+        }
+        // rs = r sa ssmi
+        const R rsi = h.rs * T.ssmi;
+        g.r += rsi * T.sa;
+        g_sa += rsi * T.r;
+        g_ssm -= rsi * T.rs;
+        // ssm = S - sm ; sa = S - u
+        g.S += g_ssm + g_sa;
+        g_sm -= g_ssm;
+        g.u -= g_sa;
+    };
 
-    // outer flux of the chosen side
+    // the near side's flux
+    const Energy En = energy(N);
     {
-        const R r0 = left ? rl : rr, u0 = left ? ul : ur, v0 = left ? vl : vr, w0 = left ? wl : wr;
-        const R by0 = left ? byl : byr, bz0 = left ? bzl : bzr, pt0 = left ? ptl : ptr;
-        const R e0 = left ? el : er, vb0 = left ? vbl : vbr;
-        R g_r0 = lF[0] * u0 + lF[1] * u0 * u0 + lF[2] * v0 * u0 + lF[3] * w0 * u0;
-        R g_u0 = lF[0] * r0 + lF[1] * R(2) * r0 * u0 + lF[2] * r0 * v0 + lF[3] * r0 * w0 + lF[4] * (e0 + pt0);
-        R g_v0 = lF[2] * r0 * u0, g_w0 = lF[3] * r0 * u0;
-        R g_pt0 = lF[1] + lF[4] * u0;
+        const R lv = lF[1] * N.u + lF[2] * N.v + lF[3] * N.w;
+        const R ru = N.r * N.u;
+        gn.r = (lF[0] + lv) * N.u;
+        gn.u = N.r * (lF[0] + lv) + lF[1] * ru + lF[4] * (En.e + N.pt);
+        gn.v = lF[2] * ru;
+        gn.w = lF[3] * ru;
+        gn.pt = lF[1] + lF[4] * N.u;
         g_bn2 -= lF[1];
-        R g_by0 = -lF[2] * bn, g_bz0 = -lF[3] * bn;
-        g_bn -= lF[2] * by0 + lF[3] * bz0 + lF[4] * vb0;
-        R g_e0 = lF[4] * u0;
-        R g_vb0 = -lF[4] * bn;
+        gn.by = -lF[2] * bn;
+        gn.bz = -lF[3] * bn;
+        g_bn -= lF[2] * N.by + lF[3] * N.bz + lF[4] * En.vb;
+        gn.e = lF[4] * N.u;
+        gn.vb = -lF[4] * bn;
         if (reg != 0 && reg != 5) {
-            // (selected field by field: a reference chosen at run time would put both in memory)
-            Star T;
-            T.S = left ? A.S : B.S;
-            T.rs = left ? A.rs : B.rs;
-            T.vs = left ? A.vs : B.vs;
-            T.ws = left ? A.ws : B.ws;
-            T.es = left ? A.es : B.es;
-            const R S = T.S;
-            const R us0 = T.rs, us1 = T.rs * sm, us2 = T.rs * T.vs, us3 = T.rs * T.ws, us4 = T.es;
-            // f += S (U* - U)
-            R gS = lF[0] * (us0 - r0) + lF[1] * (us1 - r0 * u0) + lF[2] * (us2 - r0 * v0) +
-                   lF[3] * (us3 - r0 * w0) + lF[4] * (us4 - e0);
-            g_r0 -= S * (lF[0] + lF[1] * u0 + lF[2] * v0 + lF[3] * w0);
-            g_u0 -= S * lF[1] * r0;
-            g_v0 -= S * lF[2] * r0;
-            g_w0 -= S * lF[3] * r0;
-            g_e0 -= S * lF[4];
-            R gUs0 = S * lF[0], gUs1 = S * lF[1], gUs2 = S * lF[2], gUs3 = S * lF[3], gUs4 = S * lF[4];
-            R g_rs = 0, g_vs = 0, g_ws = 0, g_es = 0;
+            const Star T = star(N, En);
+            // f += S (U* - U), U* = (rs, rs sm, rs vs, rs ws, es)
+            const R ls = lF[0] + lF[1] * sm + lF[2] * T.vs + lF[3] * T.ws;
+            gn.S += N.rs * ls - N.r * (lF[0] + lv) + lF[4] * (T.es - En.e);
+            const R Sr = N.S * N.r, Srs = N.S * N.rs;
+            gn.r -= N.S * (lF[0] + lv);
+            gn.u -= Sr * lF[1];
+            gn.v -= Sr * lF[2];
+            gn.w -= Sr * lF[3];
+            gn.e -= N.S * lF[4];
+            StarGrad h;
+            h.rs = N.S * ls;
+            g_sm += Srs * lF[1];
+            h.vs = Srs * lF[2];
+            h.ws = Srs * lF[3];
+            h.es = N.S * lF[4];
             if (dstar) {
-                const R isum = rcp_(sql + sqr);
-                const R nv = sql * A.vs + sqr * B.vs + (B.bys - A.bys) * sgn;
-                const R nw = sql * A.ws + sqr * B.ws + (B.bzs - A.bzs) * sgn;
-                const R nby = sql * B.bys + sqr * A.bys + sql * sqr * (B.vs - A.vs) * sgn;
-                const R nbz = sql * B.bzs + sqr * A.bzs + sql * sqr * (B.ws - A.ws) * sgn;
-                const R vss = nv * isum, wss = nw * isum, byss = nby * isum, bzss = nbz * isum;
+                const Energy Eo = energy(O);
+                const Star F = star(O, Eo);
+                StarGrad k;
+                const R isum = rcp_(N.sq + O.sq), sq2 = N.sq * O.sq * sg;
+                const R dvs = (F.vs - T.vs) * sg, dws = (F.ws - T.ws) * sg;
+                const R vss = (N.sq * T.vs + O.sq * F.vs + (F.bys - T.bys) * sg) * isum;
+                const R wss = (N.sq * T.ws + O.sq * F.ws + (F.bzs - T.bzs) * sg) * isum;
+                const R byss = (N.sq * F.bys + O.sq * T.bys + sq2 * (F.vs - T.vs)) * isum;
+                const R bzss = (N.sq * F.bzs + O.sq * T.bzs + sq2 * (F.ws - T.ws)) * isum;
                 const R vbss = sm * bn + vss * byss + wss * bzss;
-                // f += S* (U** - U*), U** - U* = (0, 0, rs (vss - vs), rs (wss - ws), ess - es)
-                const R Ss = left ? ssl : ssr;
-                const R ess = left ? A.es - sql * (A.vbs - vbss) * sgn : B.es + sqr * (B.vbs - vbss) * sgn;
-                const R gSs = lF[2] * T.rs * (vss - T.vs) + lF[3] * T.rs * (wss - T.ws) + lF[4] * (ess - T.es);
-                g_rs += Ss * (lF[2] * (vss - T.vs) + lF[3] * (wss - T.ws));
-                const R g_vss = Ss * lF[2] * T.rs, g_wss = Ss * lF[3] * T.rs;
-                g_vs -= Ss * lF[2] * T.rs;
-                g_ws -= Ss * lF[3] * T.rs;
+                // f += S* (U** - U*), S* = sm - tau abn / sq,
+                // U** - U* = (0, 0, rs (vss - vs), rs (wss - ws), -sq (vbs - vbss) sg)
+                const R Ss = sm - tabn * N.isq, dvb = (T.vbs - vbss) * sg;
+                const R ld = lF[2] * (vss - T.vs) + lF[3] * (wss - T.ws);
+                const R gSs = N.rs * ld - lF[4] * N.sq * dvb;
+                h.rs += Ss * ld;
+                const R Ssrs = Ss * N.rs;
+                const R g_vss = Ssrs * lF[2], g_wss = Ssrs * lF[3];
+                h.vs -= g_vss;
+                h.ws -= g_wss;
                 const R g_ess = Ss * lF[4];
-                g_es -= Ss * lF[4];
-                R g_vbss = 0;
-                if (left) {   // essl = esl - sql (vbsl - vbss) sgn ; ssl = sm - abn / sql
-                    gA_es += g_ess;
-                    g_sql -= g_ess * (A.vbs - vbss) * sgn;
-                    gA_vbs -= g_ess * sql * sgn;
-                    g_vbss += g_ess * sql * sgn;
-                    g_sm += gSs;
-                    g_abn -= gSs * isql;
-                    g_sql += gSs * abn * (isql * isql);
-                } else {      // essr = esr + sqr (vbsr - vbss) sgn ; ssr = sm + abn / sqr
-                    gB_es += g_ess;
-                    g_sqr += g_ess * (B.vbs - vbss) * sgn;
-                    gB_vbs += g_ess * sqr * sgn;
-                    g_vbss -= g_ess * sqr * sgn;
-                    g_sm += gSs;
-                    g_abn += gSs * isqr;
-                    g_sqr -= gSs * abn * (isqr * isqr);
-                }
+                h.sq -= g_ess * dvb;
+                const R g_vbss = g_ess * N.sq * sg;
+                h.vbs -= g_vbss;
+                const R gsi = gSs * N.isq;
+                g_sm += gSs;
+                g_tabn -= gsi;
+                h.sq += gsi * N.isq * tabn;
                 // vbss = sm bn + vss byss + wss bzss
                 g_sm += g_vbss * bn;
                 g_bn += g_vbss * sm;
-                const R g_vss2 = g_vss + g_vbss * byss, g_wss2 = g_wss + g_vbss * bzss;
-                const R g_byss = g_vbss * vss, g_bzss = g_vbss * wss;
                 // x = n * isum
-                const R g_nv = g_vss2 * isum, g_nw = g_wss2 * isum, g_nby = g_byss * isum, g_nbz = g_bzss * isum;
-                const R g_isum = g_vss2 * nv + g_wss2 * nw + g_byss * nby + g_bzss * nbz;
-                // nv = sql vsl + sqr vsr + (bysr - bysl) sgn
-                g_sql += g_nv * A.vs;
-                gA_vs += g_nv * sql;
-                g_sqr += g_nv * B.vs;
-                gB_vs += g_nv * sqr;
-                gB_bys += g_nv * sgn;
-                gA_bys -= g_nv * sgn;
-                // nw
-                g_sql += g_nw * A.ws;
-                gA_ws += g_nw * sql;
-                g_sqr += g_nw * B.ws;
-                gB_ws += g_nw * sqr;
-                gB_bzs += g_nw * sgn;
-                gA_bzs -= g_nw * sgn;
-                // nby = sql bysr + sqr bysl + sql sqr (vsr - vsl) sgn
-                g_sql += g_nby * (B.bys + sqr * (B.vs - A.vs) * sgn);
-                g_sqr += g_nby * (A.bys + sql * (B.vs - A.vs) * sgn);
-                gB_bys += g_nby * sql;
-                gA_bys += g_nby * sqr;
-                gB_vs += g_nby * sql * sqr * sgn;
-                gA_vs -= g_nby * sql * sqr * sgn;
-                // nbz
-                g_sql += g_nbz * (B.bzs + sqr * (B.ws - A.ws) * sgn);
-                g_sqr += g_nbz * (A.bzs + sql * (B.ws - A.ws) * sgn);
-                gB_bzs += g_nbz * sql;
-                gA_bzs += g_nbz * sqr;
-                gB_ws += g_nbz * sql * sqr * sgn;
-                gA_ws -= g_nbz * sql * sqr * sgn;
-                // isum = 1 / (sql + sqr)
-                g_sql -= g_isum * isum * isum;
-                g_sqr -= g_isum * isum * isum;
+                const R g_nv = (g_vss + g_vbss * byss) * isum, g_nw = (g_wss + g_vbss * bzss) * isum;
+                const R g_nby = g_vbss * vss * isum, g_nbz = g_vbss * wss * isum;
+                const R g_sum = g_nv * vss + g_nw * wss + g_nby * byss + g_nbz * bzss;   // isum = 1 / (sq + sq_o)
+                // nv = sq vs + sq_o vs_o + (bys_o - bys) sg, nw alike;
+                // nby = sq bys_o + sq_o bys + sq sq_o (vs_o - vs) sg, nbz alike
+                h.sq += g_nv * T.vs + g_nw * T.ws + g_nby * (F.bys + O.sq * dvs) + g_nbz * (F.bzs + O.sq * dws) - g_sum;
+                k.sq = g_nv * F.vs + g_nw * F.ws + g_nby * (T.bys + N.sq * dvs) + g_nbz * (T.bzs + N.sq * dws) - g_sum;
+                h.vs += g_nv * N.sq - g_nby * sq2;
+                k.vs = g_nv * O.sq + g_nby * sq2;
+                h.ws += g_nw * N.sq - g_nbz * sq2;
+                k.ws = g_nw * O.sq + g_nbz * sq2;
+                h.bys = g_nby * O.sq - g_nv * sg;
+                k.bys = g_nby * N.sq + g_nv * sg;
+                h.bzs = g_nbz * O.sq - g_nw * sg;
+                k.bzs = g_nbz * N.sq + g_nw * sg;
+                star_rev(O, Eo, F, k, go);
+                energy_rev(O, Eo, go);
             }
-            // U* = (rs, rs sm, rs vs, rs ws, es)
-            g_rs += gUs0 + gUs1 * sm + gUs2 * T.vs + gUs3 * T.ws;
-            g_sm += gUs1 * T.rs;
-            g_vs += gUs2 * T.rs;
-            g_ws += gUs3 * T.rs;
-            g_es += gUs4;
-            if (left) {
-                gA_rs += g_rs;
-                gA_vs += g_vs;
-                gA_ws += g_ws;
-                gA_es += g_es;
-                g_sl += gS;
-            } else {
-                gB_rs += g_rs;
-                gB_vs += g_vs;
-                gB_ws += g_ws;
-                gB_es += g_es;
-                g_sr += gS;
-            }
-        }
-        if (left) {
-            g_rl += g_r0; g_ul += g_u0; g_vl += g_v0; g_wl += g_w0; g_ptl += g_pt0;
-            g_byl += g_by0; g_bzl += g_bz0; g_el += g_e0; g_vbl += g_vb0;
-        } else {
-            g_rr += g_r0; g_ur += g_u0; g_vr += g_v0; g_wr += g_w0; g_ptr += g_pt0;
-            g_byr += g_by0; g_bzr += g_bz0; g_er += g_e0; g_vbr += g_vb0;
+            star_rev(N, En, T, h, gn);
         }
     }
-    // sql = sqrt(rsl), sqr = sqrt(rsr)
-    gA_rs += R(0.5) * g_sql * isql;
-    gB_rs += R(0.5) * g_sqr * isqr;
-    // star states (reverse), side by side
-    auto star_rev = [&](const Star& T, R r, R u, R v, R w, R by, R bz, R pt, R e, R vb, R g_rs, R g_vs, R g_ws,
-                        R g_bys, R g_bzs, R g_vbs, R g_es, R& g_r, R& g_u, R& g_v, R& g_w, R& g_by, R& g_bz,
-                        R& g_pt, R& g_e, R& g_vb, R& g_S) {
-        (void)v;
-        (void)w;
-        // es = nes * ssmi
-        const R g_nes = g_es * T.ssmi;
-        R g_ssm = -g_es * T.es * T.ssmi;
-        // nes = sa e - pt u + pts sm + bn (vb - vbs)
-        R g_sa = g_nes * e;
-        g_e += g_nes * T.sa;
-        g_pt -= g_nes * u;
-        g_u -= g_nes * pt;
-        g_pts += g_nes * sm;
-        g_sm += g_nes * pts;
-        g_bn += g_nes * (vb - T.vbs);
-        g_vb += g_nes * bn;
-        g_vbs -= g_nes * bn;
-        // vbs = sm bn + vs bys + ws bzs
-        g_sm += g_vbs * bn;
-        g_bn += g_vbs * sm;
-        g_vs += g_vbs * T.bys;
-        g_bys += g_vbs * T.vs;
-        g_ws += g_vbs * T.bzs;
-        g_bzs += g_vbs * T.ws;
-        if (!T.deg) {
-            R g_nu = 0, g_nb = 0;
-            g_v += g_vs;
-            g_by -= g_vs * T.nu;
-            g_nu -= g_vs * by;
-            g_w += g_ws;
-            g_bz -= g_ws * T.nu;
-            g_nu -= g_ws * bz;
-            g_by += g_bys * T.nb;
-            g_nb += g_bys * by;
-            g_bz += g_bzs * T.nb;
-            g_nb += g_bzs * bz;
-            const R Di = T.Di;
-            // nu = bn (sm - u) / D
-            g_bn += g_nu * (sm - u) * Di;
-            g_sm += g_nu * bn * Di;
-            g_u -= g_nu * bn * Di;
-            R g_D = -g_nu * T.nu * Di;
-            // nb = (r sa^2 - bn2) / D
-            g_r += g_nb * T.sa * T.sa * Di;
-            g_sa += g_nb * R(2) * r * T.sa * Di;
-            g_bn2 -= g_nb * Di;
-            g_D -= g_nb * T.nb * Di;
-            // D = r sa ssm - bn2
-            g_r += g_D * T.sa * T.ssm;
-            g_sa += g_D * r * T.ssm;
-            g_ssm += g_D * r * T.sa;
-            g_bn2 -= g_D;
-        } else {
-            g_v += g_vs;
-            g_w += g_ws;
-            g_by += g_bys;
-            g_bz += g_bzs;
-        }
-        // rs = r sa ssmi
-        g_r += g_rs * T.sa * T.ssmi;
-        g_sa += g_rs * r * T.ssmi;
-        g_ssm -= g_rs * T.rs * T.ssmi;
-        // ssm = S - sm ; sa = S - u
-        g_S += g_ssm + g_sa;
-        g_sm -= g_ssm;
-        g_u -= g_sa;
-    };
-    if (starB) star_rev(B, rr, ur, vr, wr, byr, bzr, ptr, er, vbr, gB_rs, gB_vs, gB_ws, gB_bys, gB_bzs, gB_vbs, gB_es, g_rr, g_ur,
-             g_vr, g_wr, g_byr, g_bzr, g_ptr, g_er, g_vbr, g_sr);
-    if (starA) star_rev(A, rl, ul, vl, wl, byl, bzl, ptl, el, vbl, gA_rs, gA_vs, gA_ws, gA_bys, gA_bzs, gA_vbs, gA_es, g_rl, g_ul,
-             g_vl, g_wl, g_byl, g_bzl, g_ptl, g_el, g_vbl, g_sl);
+    energy_rev(N, En, gn);
+    const R g_abn = left ? g_tabn : -g_tabn;
+    R g_rl = sel(left, gn.r, go.r), g_rr = sel(left, go.r, gn.r), g_ul = sel(left, gn.u, go.u), g_ur = sel(left, go.u, gn.u);
+    const R g_vl = sel(left, gn.v, go.v), g_vr = sel(left, go.v, gn.v), g_wl = sel(left, gn.w, go.w), g_wr = sel(left, go.w, gn.w);
+    R g_pl = sel(left, gn.p, go.p), g_pr = sel(left, go.p, gn.p), g_byl = sel(left, gn.by, go.by), g_byr = sel(left, go.by, gn.by);
+    R g_bzl = sel(left, gn.bz, go.bz), g_bzr = sel(left, go.bz, gn.bz), g_ptl = sel(left, gn.pt, go.pt), g_ptr = sel(left, go.pt, gn.pt);
+    const R g_el = sel(left, gn.e, go.e), g_er = sel(left, go.e, gn.e);
+    R g_sl = sel(left, gn.S, go.S), g_sr = sel(left, go.S, gn.S);
     // sm = smn / den ; pts = ptn / den
     const R g_smn = g_sm * deni, g_ptn = g_pts * deni;
     R g_den = -(g_sm * sm + g_pts * pts) * deni;
@@ -528,21 +483,6 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         } else {
             g_rr += h_r; g_pr += h_p; g_byr += h_by; g_bzr += h_bz;
         }
-    }
-    // vb = u bn + v by + w bz ; e = p gm1i + rho |u|^2 / 2 + b2 / 2
-    if (reg <= 3) {
-        g_ul += g_vbl * bn; g_bn += g_vbl * ul; g_vl += g_vbl * byl; g_byl += g_vbl * vl; g_wl += g_vbl * bzl;
-        g_bzl += g_vbl * wl;
-        g_pl += g_el * gm1i;
-        g_rl += g_el * R(0.5) * (ul * ul + vl * vl + wl * wl);
-        g_ul += g_el * rl * ul; g_vl += g_el * rl * vl; g_wl += g_el * rl * wl;
-    }
-    if (reg >= 2) {
-        g_ur += g_vbr * bn; g_bn += g_vbr * ur; g_vr += g_vbr * byr; g_byr += g_vbr * vr; g_wr += g_vbr * bzr;
-        g_bzr += g_vbr * wr;
-        g_pr += g_er * gm1i;
-        g_rr += g_er * R(0.5) * (ur * ur + vr * vr + wr * wr);
-        g_ur += g_er * rr * ur; g_vr += g_er * rr * vr; g_wr += g_er * rr * wr;
     }
     // pt = p + b2 / 2 (and the b2 / 2 of e)
     const R g_b2l = R(0.5) * g_el + R(0.5) * g_ptl, g_b2r = R(0.5) * g_er + R(0.5) * g_ptr;
