@@ -42,58 +42,45 @@ static StepArgs<R> to_args(const StepHostArgs& h) {
     return a;
 }
 
-// The chunks of a 3D plane shared out to the warps (StepPlan), longest first to the least loaded
-// warp, for every number of in-plane flux chunks moved to phase A; the split with the shortest
-// two phases is taken.  Costs: cycles of a chunk with four
-// warps per scheduler running, measured (FP32, 32x8); FP64 operations (FP64, bound by that pipe).
+// The chunks of a 3D plane shared out to the warps (StepPlan), longest first to the least loaded warp:
+// in phase A the edges, the z-faces and the conversion, in phase B the prep, the other faces and the
+// update.  Costs: cycles of a chunk with four warps per scheduler running, measured (FP32, 32x8); FP64
+// operations (FP64, bound by that pipe).  False: a list is too long.
 template <typename C>
-static StepPlan make_plan() {
+static bool make_plan(StepPlan& plan) {
     constexpr bool F64 = C::EQ == 2;
     constexpr int PREP = F64 ? 330 : 2480, FACE = F64 ? 220 : 1450, EDGE = F64 ? 260 : 1400, CONV = F64 ? 40 : 620,
                   UPD = F64 ? 45 : 700;
-    auto share = [](std::vector<std::pair<int, int>> tasks, StepPlan& P, int phase) {
+    using Tasks = std::vector<std::pair<int, int>>;   // (cost, chunk)
+    auto share = [&](Tasks tasks, int phase) {
         std::stable_sort(tasks.begin(), tasks.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
-        int load[StepPlan::MAXW] = {}, top = 0;
-        std::vector<std::pair<int, int>> list[StepPlan::MAXW];
+        int load[C::NWARP] = {};
+        Tasks list[C::NWARP];
         for (const auto& t : tasks) {
             const int w = (int)(std::min_element(load, load + C::NWARP) - load);
             list[w].push_back(t);
             load[w] += t.first;
-            top = std::max(top, load[w]);
         }
-        for (int w = 0; w < StepPlan::MAXW; ++w) {
+        for (int w = 0; w < C::NWARP; ++w) {
             // the short, latency-bound chunks at another place in the list of each warp of a
             // scheduler (warps w, w + 4, ...), so that the others have work meanwhile
             auto& L = list[w];
             if (L.size() > 1) std::rotate(L.begin(), L.end() - (w / 4) % (int)L.size(), L.end());
-            if ((int)L.size() > 8 * C::NQ - (C::NQ > 1)) return 1 << 30;
-            P.t[phase][w][0] = P.t[phase][w][1] = ~0ull;
+            if ((int)L.size() > 8 * C::NQ - (C::NQ > 1)) return false;
+            plan.t[phase][w][0] = plan.t[phase][w][1] = ~0ull;
             for (size_t k = 0; k < L.size(); ++k)
-                P.t[phase][w][k / 8] ^= (255ull ^ (unsigned long long)L[k].second) << (8 * (k % 8));
+                plan.t[phase][w][k / 8] ^= (255ull ^ (unsigned long long)L[k].second) << (8 * (k % 8));
         }
-        return top;
+        return true;
     };
-    StepPlan best{};
-    int least = 1 << 30;
-    for (int x = 0; x <= C::IEZ::N; ++x) {
-        std::vector<std::pair<int, int>> A, B;
-        for (int q = 0; q < C::NZ; ++q) A.emplace_back(q < C::IFZ::N ? FACE : EDGE, C::NI + q);
-        for (int q = 0; q < C::IPR::N; ++q) B.emplace_back(PREP, C::NI + C::NZ + q);
-        for (int q = 0; q < C::NI; ++q) {
-            const int cost = q < C::IFX::N + C::IFY::N ? FACE : EDGE;
-            if (q >= C::NI - x) A.emplace_back(cost, q);
-            else B.emplace_back(cost, q);
-        }
-        for (int q = 0; q < C::ICV::N; ++q) A.emplace_back(CONV, C::NI + C::NZ + C::IPR::N + q);
-        for (int q = 0; q < C::IUP::N; ++q) B.emplace_back(UPD, C::NI + C::NZ + C::IPR::N + C::ICV::N + q);
-        StepPlan P{};
-        const int a = share(A, P, 0), b = share(B, P, 1);
-        if (a < (1 << 30) && b < (1 << 30) && a + b < least) {
-            least = a + b;
-            best = P;
-        }
-    }
-    return best;
+    Tasks A, B;
+    for (int q = 0; q < C::NZ; ++q) A.emplace_back(q < C::IFZ::N ? FACE : EDGE, C::NI + q);
+    for (int q = 0; q < C::IEZ::N; ++q) A.emplace_back(EDGE, C::IFX::N + C::IFY::N + q);
+    for (int q = 0; q < C::ICV::N; ++q) A.emplace_back(CONV, C::NI + C::NZ + C::IPR::N + q);
+    for (int q = 0; q < C::IPR::N; ++q) B.emplace_back(PREP, C::NI + C::NZ + q);
+    for (int q = 0; q < C::IFX::N + C::IFY::N; ++q) B.emplace_back(FACE, q);
+    for (int q = 0; q < C::IUP::N; ++q) B.emplace_back(UPD, C::NI + C::NZ + C::IPR::N + C::ICV::N + q);
+    return share(A, 0) && share(B, 1);
 }
 
 template <typename R, int NDIM, int TX, int TY, int NT, int MINB = 1>
@@ -107,7 +94,13 @@ struct StepInst {
     static constexpr auto whole = &step_kernel<R, NDIM, TX, TY, NT, MINB, false, false>;
     static constexpr auto split = &step_kernel<R, NDIM, TX, TY, NT, MINB, NDIM == 3, false>;
     static constexpr auto async = &step_kernel<R, NDIM, TX, TY, NT, MINB, NDIM == 3, true>;
+    static const StepPlan* plan() {   // null: none
+        static StepPlan p{};
+        static const bool ok = NDIM != 3 || make_plan<C>(p);
+        return ok ? &p : nullptr;
+    }
     static cudaError_t prepare() {
+        if (!plan()) return cudaErrorInvalidConfiguration;
         for (auto k : {whole, split, async}) {
             const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM_BYTES);
             if (e != cudaSuccess) return e;
@@ -119,7 +112,7 @@ struct StepInst {
     }
     static cudaError_t launch(const void* args, int grid, cudaStream_t s) {
         const StepArgs<R> a = to_args<R>(*static_cast<const StepHostArgs*>(args));
-        static const StepPlan plan = NDIM == 3 ? make_plan<C>() : StepPlan{};
+        const StepPlan& plan = *StepInst::plan();
         if (a.slice) launch_pdl(async, grid, NT, C::SMEM_BYTES, s, a, plan);
         else (a.nzb > 1 ? split : whole)<<<grid, NT, C::SMEM_BYTES, s>>>(a, plan);
         return cudaGetLastError();

@@ -645,9 +645,9 @@ __device__ __forceinline__ void flux_ez(const R* P0, R* IB, int q, int wx, R gam
     }
 }
 
-// In-plane fluxes of plane c (slot P0 into IB), one chunk q of NI.
+// The x- and y-faces of plane c (slot P0 into IB), one chunk q of IFX::N + IFY::N.
 template <typename R, typename C>
-__device__ __forceinline__ void flux_inplane(const R* P0, R* IB, int q, int wx, R gamma, R gm1i, R eps, int riemann) {
+__device__ __forceinline__ void flux_faces(const R* P0, R* IB, int q, int wx, R gamma, R gm1i, R eps, int riemann) {
     R* Fx = IB;
     R* Fy = IB + 5 * C::FXN;
     const int lane = threadIdx.x & 31;
@@ -671,9 +671,7 @@ __device__ __forceinline__ void flux_inplane(const R* P0, R* IB, int q, int wx, 
 #pragma unroll
             for (int v = 0; v < 5; ++v) Fy[v * C::FYN + o] = F[v];
         }
-        return;
     }
-    flux_ez<R, C>(P0, IB, q - C::IFY::N, wx, gamma);
 }
 
 // Fluxes between planes c-1 (slot Pm) and c (slot P0) into ZB, one chunk q of NZ.
@@ -778,18 +776,24 @@ struct ChunkList {
 //   B: the prep of plane c+1 into the slot of plane c-1, which phase A was the last to read,
 //      beside the fluxes inside plane c, which read slot c only, and the update of plane c-1,
 //      whose last fluxes came in phase A.
-// The EMFs inside plane c may as well run in phase A of plane c+1 (slot c is still there), so
-// the plan moves as many of them there as makes the two phases even, and gives every warp a fixed
-// list of chunks in each phase.  The tile is copied to registers and the lists come from the
-// parameter bank: with the lists decoded chunk by chunk from memory, or shared out through a
-// counter, the step took 24.7 and 25.7 ms.
+// The EMFs inside plane c run in phase A of plane c+1 (slot c is still there): the two phases are even
+// then, and the edge solvers' code is in A alone, that of the prep and of the x- and y-faces in B.
+// Every warp has a fixed list of chunks in each phase.  The tile is copied to registers and the
+// lists come from the parameter bank: with the lists decoded chunk by chunk from memory, or shared out
+// through a counter, the step took 24.7 and 25.7 ms.
 //
-// What bounds it (FP32): the issue slots (66 % busy; 16 warps, the registers allow no more) and
-// the shared-memory pipe (49 %) together, and the ends of the phases; neither HBM (8 %) nor the
-// FP32 pipes (33 %).  512^3 box, 32x8: 18.6 ms per step against 21.0 for the form with three
-// phases (load + update + conversion / prep / fluxes) over the whole CTA, whose flux phase ended
-// on a half-filled pass and whose prep left four of sixteen warps idle.  FP64 is bound by the FP64
-// pipe (see mhd_math.cuh).
+// What bounds it (FP32): the issue slots (61-66 % busy; 16 warps, the registers allow no more), left
+// empty mostly by waits for instructions (of 5.4 warps waiting per issued instruction 1.4: the code of a
+// phase's solvers and prep is more than the instruction cache holds) and at the ends of the phases (1.0);
+// neither HBM (8 %) nor the FP32 pipes (33 %).  Measured on the 512^3 box, 32x8, step and fill: part of
+// the EMFs inside the plane in either phase, a little more even but with their solver in both, 21.36
+// ms; as it is 20.66; one solver per phase behind the state loads of all directions 21.12 (24^3
+// patches -1 %), one with offsets chosen at run time 23.5 (a third more instructions); one chunk list
+// per warp and plane with two mbarrier points instead of the barriers, no waits at the ends (1.02 ->
+// 0.04) but all code at once (instruction stalls 2.7), 30.4.  The form before this one, three phases
+// (load + update + conversion / prep / fluxes) whose flux phase ended on a half-filled pass and whose
+// prep left four of sixteen warps idle, took 21.0 ms for the step alone, this one 17.9.  FP64 is bound
+// by the FP64 pipe (see mhd_math.cuh).
 //
 // ZB: work items are z-blocks of tiles (a launch of fewer tiles than SMs: the 64^3 box of 32^3
 // patches, 32 tiles, took 172 us and takes 58); an instantiation of its own, whose block bounds cost
@@ -917,7 +921,7 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
                 for (int q; (q = list.next()) != 255;) {
                     if (q < C::NI) {
                         if (ci >= z0 && ci < z1) {
-                            if constexpr (B) flux_inplane<R, C>(S.P(ci & 1), S.I(ci & 1), q, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
+                            if constexpr (B) flux_faces<R, C>(S.P(ci & 1), S.I(ci & 1), q, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
                             else flux_ez<R, C>(S.P(ci & 1), S.I(ci & 1), q - C::IFX::N - C::IFY::N, T.wx, a.gamma);
                         }
                     } else if (q < C::NI + C::NZ) {
@@ -984,7 +988,9 @@ __global__ void __launch_bounds__(NT, MINB) step_kernel(StepArgs<R> a, StepPlan 
             for (int q = wid; q < C::IPR::N; q += C::NWARP) prep_chunk<R, C>(X, S.P(0), q, a.limiter, T.wx);
             __syncthreads();
             for (int q = wid; q < C::NI + C::NZ; q += C::NWARP) {
-                if (q < C::NI) flux_inplane<R, C>(S.P(0), S.I(0), q, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
+                constexpr int NF = C::IFX::N + C::IFY::N;
+                if (q < NF) flux_faces<R, C>(S.P(0), S.I(0), q, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
+                else if (q < C::NI) flux_ez<R, C>(S.P(0), S.I(0), q - NF, T.wx, a.gamma);
                 else flux_interplane<R, C>(S.P(0), S.P(0), S.Z(0), q - C::NI, T.wx, a.gamma, a.gm1i, a.eps, a.riemann);
             }
             if (a.dynamic && threadIdx.x == 0) s_tile = atomicAdd(&a.work[0], 1);
