@@ -100,14 +100,15 @@ MHD_HD bool greater_(double a, double b) {
     return a > b;
 #endif
 }
-// a and b of the same sign and neither 0 (a b > 0, without the product's underflow in double)
-MHD_HD bool same_sign_(float a, float b) { return a * b > 0.0f; }
+// a and b of the same sign and neither 0, without the product a b, which underflows where both are
+// small (in single precision at 1e-19): the condition under which minmod_ below is not 0
+MHD_HD bool same_sign_(float a, float b) { return (a > 0.0f && b > 0.0f) || (a < 0.0f && b < 0.0f); }
 MHD_HD bool same_sign_(double a, double b) {
 #ifdef __CUDA_ARCH__
     const long long i = __double_as_longlong(a), j = __double_as_longlong(b);
     return (i ^ j) >= 0 && (i << 1) != 0 && (j << 1) != 0;
 #else
-    return a * b > 0.0;
+    return (a > 0.0 && b > 0.0) || (a < 0.0 && b < 0.0);
 #endif
 }
 MHD_HD bool mand(bool a, bool b) { return a && b; }
@@ -272,7 +273,7 @@ MHD_HD double minmod_(double a, double b) {
     const long long pick = (ia & m) <= (ib & m) ? ia : ib;
     return __longlong_as_double((ia ^ ib) < 0 ? 0ll : pick);
 #else
-    return a * b > 0.0 ? (fabs(a) <= fabs(b) ? a : b) : 0.0;
+    return same_sign_(a, b) ? (fabs(a) <= fabs(b) ? a : b) : 0.0;
 #endif
 }
 

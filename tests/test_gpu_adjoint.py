@@ -135,6 +135,28 @@ def test_adjoint_fp32_against_fp64_reference():
     assert err <= 1e-4, err
 
 
+@pytest.mark.parametrize("limiter", [0, 1], ids=["minmod", "mc"])
+def test_adjoint_fp32_of_a_field_whose_slopes_are_tiny(limiter):
+    """A seed field 2^-70 times the usual one: products of two of its differences underflow in single
+    precision, the slopes the step takes of it do not.  Its gradient (that of the field after the step,
+    the only cotangents) against the FP64 oracle's, with the bound of the FP32 test above."""
+    geom, U, meta = W.small_box(ncell=(16, 16, 16), patch=(8, 8, 8), seed=51)
+    U = U.copy()
+    U[5:] *= 2.0 ** -70
+    flat = W.to_patches(U, geom).astype(np.float32).astype(np.float64)
+    mask = interior_mask(geom)
+    face = np.zeros((geom.npatch, 8, geom.state_elems() // (8 * geom.npatch)), dtype=bool)
+    face[:, 5:] = True
+    face = mask & face.reshape(-1)
+    ob = O.Bunch(geom, meta["gamma"])
+    dt = ob.cfl_dt(ob.fill_guards(ob.split(flat)))
+    w = np.where(face, np.random.default_rng(151).normal(size=flat.size), 0.0)
+    ref = oracle_grad(geom, flat, dt, meta["gamma"], w, limiter, eps=O.HLLD_EPS[4])
+    got, _ = gpu_adjoint(geom, flat, dt, meta["gamma"], w, torch.float32, limiter)
+    err = np.max(np.abs(got[face] - ref[face])) / np.max(np.abs(ref[face]))
+    assert err <= 1e-4, err
+
+
 def jitter(flat, mask, seed, amp=1e-2):
     """Seeded relative plus absolute noise on every interior entry: a generic state with no
     exactly tied or exactly zero one-sided differences (a field that is identically zero, like
