@@ -77,15 +77,10 @@ def p(a, d):
     return torch.roll(a, shifts=-1, dims=AXIS[d])
 
 
-def same_sign(a, b):
-    """a * b > 0, without the product (which underflows where both are small)."""
-    return ((a > 0) & (b > 0)) | ((a < 0) & (b < 0))
-
-
 def minmod(a, b):
     """minmod(a, b) = 0 if a*b <= 0 else the argument of smaller magnitude (ties: a)."""
     pick = torch.where(a.abs() <= b.abs(), a, b)
-    return torch.where(same_sign(a, b), pick, torch.zeros_like(a))
+    return torch.where(a * b > 0, pick, torch.zeros_like(a))
 
 
 def mc(a, b):
@@ -93,7 +88,7 @@ def mc(a, b):
     c = 0.5 * (a + b)
     m2 = torch.where((2 * a).abs() <= (2 * b).abs(), 2 * a, 2 * b)
     pick = torch.where(c.abs() <= m2.abs(), c, m2)
-    return torch.where(same_sign(a, b), pick, torch.zeros_like(a))
+    return torch.where(a * b > 0, pick, torch.zeros_like(a))
 
 
 def limited(q, d, limiter):
