@@ -90,12 +90,13 @@ MHD_HD bool positive_(double x) {
 #endif
 }
 #ifdef __CUDA_ARCH__
-// bits of a double ordered as the values (and back)
+// bits of a double ordered as the values (and back); order0_: and the two zeros equal
 __device__ __forceinline__ long long order_(long long i) { return i ^ (long long)((unsigned long long)(i >> 63) >> 1); }
+__device__ __forceinline__ long long order0_(long long i) { return i < 0 ? (long long)0x8000000000000000ull - i : i; }
 #endif
 MHD_HD bool greater_(double a, double b) {
 #ifdef __CUDA_ARCH__
-    return order_(__double_as_longlong(a)) > order_(__double_as_longlong(b));
+    return order0_(__double_as_longlong(a)) > order0_(__double_as_longlong(b));
 #else
     return a > b;
 #endif

@@ -1,0 +1,67 @@
+"""The element operations of the scheme (mhd_ops.cuh, mhd_math.cuh, mhd_vjp.cuh) as the device
+evaluates them, one operation per argument row, in both precisions and with the compiler flags of the
+kernels."""
+import ctypes as ct
+import os
+import subprocess
+
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+OPS = ["greater", "hlld_vjp"]
+DTYPES = [torch.float64, torch.float32]
+both = pytest.mark.parametrize("dtype", DTYPES, ids=["f64", "f32"])
+
+
+@pytest.fixture(scope="module")
+def ops(tmp_path_factory):
+    """ops(name, rows, nout, dtype): rows (n, nin) through an operation, (n, nout) back."""
+    from paper_2508_09568_gb300 import build as B
+    tmp = tmp_path_factory.mktemp("device_ops")
+    libs = {}
+    for dtype, real, unit in ((torch.float64, "double", "kernels_f64.cu"), (torch.float32, "float", "kernels_f32.cu")):
+        so = str(tmp / f"ops_{real}.so")
+        flags = [f for f in B.UNITS[unit] if f.startswith("-prec") or f.startswith("-ftz")]
+        subprocess.run([B._nvcc()] + B.ARCH + B.COMMON + flags + [f"-DREAL={real}", "-shared", "-o", so,
+                                                                   os.path.join(HERE, "device_ops.cu")], check=True)
+        libs[dtype] = ct.CDLL(so)
+        libs[dtype].run_rows.argtypes = [ct.c_int, ct.c_int, ct.c_int, ct.c_void_p, ct.c_void_p, ct.c_int]
+
+    def run(name, rows, nout, dtype):
+        x = torch.as_tensor(np.ascontiguousarray(rows), dtype=dtype).cuda()
+        y = torch.full((x.shape[0], nout), float("nan"), dtype=dtype, device="cuda")
+        torch.cuda.synchronize()
+        assert libs[dtype].run_rows(OPS.index(name), x.shape[1], nout, x.data_ptr(), y.data_ptr(), x.shape[0]) == 0
+        return y.cpu().numpy()
+    return run
+
+
+def pairs(values):
+    a, b = np.meshgrid(values, values, indexing="ij")
+    return np.stack([a.ravel(), b.ravel()], axis=1)
+
+
+@both
+def test_greater_takes_the_two_zeros_as_equal(ops, dtype):
+    x = pairs([0.0, -0.0, 1e-30, -1e-30, 1.0, -1.0, 1.5, -1.5, np.inf, -np.inf])
+    assert np.array_equal(ops("greater", x, 1, dtype)[:, 0], (x[:, 0] > x[:, 1]).astype(float))
+
+
+@both
+def test_hlld_reverse_at_rest_does_not_depend_on_the_sign_of_zero(ops, dtype):
+    """Gas at rest on both sides of a face, a velocity of +0 or -0: a tie of the two velocities, whose
+    cotangent goes to the first in every case."""
+    rng = np.random.default_rng(5)
+    rows = []
+    for ul in (0.0, -0.0):
+        for ur in (0.0, -0.0):
+            rows.append([1.0, ul, 0.1, -0.2, 0.9, 0.3, 0.2, 0.8, ur, 0.3, 0.1, 1.1, -0.1, 0.4, 0.5])
+    rows = np.concatenate([np.array(rows), np.tile(rng.normal(size=5), (4, 1))], axis=1)
+    y = ops("hlld_vjp", rows, 15, dtype)
+    assert np.all(np.isfinite(y)) and np.any(y[:, [1, 8]] != 0)
+    for k in range(1, 4):
+        assert np.array_equal(y[k], y[0]), k
