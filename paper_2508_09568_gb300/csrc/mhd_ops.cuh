@@ -6,7 +6,7 @@
 // Helpers used by the scheme code for R = float, double:
 //   fma_(a, b, c) = a * b + c rounded once      sel(m, a, b) = m ? a : b
 //   mul_(a, b) = a * b, never fused
-//   nonneg_, le_mag_ -> mask                    mand / mor / mnot on masks
+//   nonneg_, le_mag_, greater_ ... -> mask       mand / mor / mnot on masks
 //   rabs, rdiv (quotient), rsqrt_ (square root), fmax_ / fmin_ (larger / smaller value)
 #pragma once
 
@@ -51,14 +51,31 @@ MHD_HD double mul_(double a, double b) {
 #endif
 }
 
-// x >= 0, and a <= b for two magnitudes.  Double precision on the device: on the bits (doubles of
-// one sign order as integers), off the FP64 pipe, whose 2 lanes per clock and SM bound every FP64
-// kernel and on which a comparison costs as much as a product; the integer pipe has 64 and is idle.
+// Comparisons.  Double precision on the device: on the bits (doubles of one sign order as integers),
+// off the FP64 pipe, whose 2 lanes per clock and SM bound every FP64 kernel and on which a comparison
+// costs as much as a product; the integer pipe has 64 and is idle.  They give what the comparison of
+// the values gives: the two zeros are equal, and a NaN compares false.
+#ifdef __CUDA_ARCH__
+constexpr long long kInfBits = 0x7ff0000000000000ll, kMagBits = 0x7fffffffffffffffll;
+// bits of a double ordered as the values (and back); order0_: and the two zeros equal
+__device__ __forceinline__ long long order_(long long i) { return i ^ (long long)((unsigned long long)(i >> 63) >> 1); }
+__device__ __forceinline__ long long order0_(long long i) { return i < 0 ? (long long)0x8000000000000000ull - i : i; }
+#endif
+// x is a number
+MHD_HD bool number_(float x) { return x == x; }
+MHD_HD bool number_(double x) {
+#ifdef __CUDA_ARCH__
+    return (__double_as_longlong(x) & kMagBits) <= kInfBits;
+#else
+    return x == x;
+#endif
+}
+// x >= 0; a <= b for two magnitudes (a not NaN, or b a number)
 MHD_HD bool nonneg_(float x) { return x >= 0.0f; }
 MHD_HD bool nonneg_(double x) {
 #ifdef __CUDA_ARCH__
     const long long i = __double_as_longlong(x);
-    return i >= 0 || (i << 1) == 0;   // (-0 is not below 0)
+    return (unsigned long long)i <= (unsigned long long)kInfBits || (i << 1) == 0;   // (-0 is not below 0)
 #else
     return x >= 0.0;
 #endif
@@ -71,7 +88,7 @@ MHD_HD bool le_mag_(double a, double b) {
     return a <= b;
 #endif
 }
-// x != 0; x > 0 (a NaN passes or fails as its bits say: it stays one in what follows); a > b
+// x != 0; x > 0; a > b
 MHD_HD bool nonzero_(float x) { return x != 0.0f; }
 MHD_HD bool positive_(float x) { return x > 0.0f; }
 MHD_HD bool greater_(float a, float b) { return a > b; }
@@ -84,19 +101,15 @@ MHD_HD bool nonzero_(double x) {
 }
 MHD_HD bool positive_(double x) {
 #ifdef __CUDA_ARCH__
-    return __double_as_longlong(x) > 0;
+    return (unsigned long long)(__double_as_longlong(x) - 1) < (unsigned long long)kInfBits;
 #else
     return x > 0.0;
 #endif
 }
-#ifdef __CUDA_ARCH__
-// bits of a double ordered as the values (and back); order0_: and the two zeros equal
-__device__ __forceinline__ long long order_(long long i) { return i ^ (long long)((unsigned long long)(i >> 63) >> 1); }
-__device__ __forceinline__ long long order0_(long long i) { return i < 0 ? (long long)0x8000000000000000ull - i : i; }
-#endif
 MHD_HD bool greater_(double a, double b) {
 #ifdef __CUDA_ARCH__
-    return order0_(__double_as_longlong(a)) > order0_(__double_as_longlong(b));
+    const long long i = order0_(__double_as_longlong(a)), j = order0_(__double_as_longlong(b));
+    return i > j && i <= kInfBits && j >= -kInfBits;
 #else
     return a > b;
 #endif
@@ -107,7 +120,8 @@ MHD_HD bool same_sign_(float a, float b) { return (a > 0.0f && b > 0.0f) || (a <
 MHD_HD bool same_sign_(double a, double b) {
 #ifdef __CUDA_ARCH__
     const long long i = __double_as_longlong(a), j = __double_as_longlong(b);
-    return (i ^ j) >= 0 && (i << 1) != 0 && (j << 1) != 0;
+    return (i ^ j) >= 0 && (unsigned long long)((i & kMagBits) - 1) < (unsigned long long)kInfBits &&
+           (unsigned long long)((j & kMagBits) - 1) < (unsigned long long)kInfBits;
 #else
     return (a > 0.0 && b > 0.0) || (a < 0.0 && b < 0.0);
 #endif
@@ -195,29 +209,39 @@ MHD_HD double rcp_(double x) {
 MHD_HD bool finite_(float x) { return isfinite(x); }
 MHD_HD bool finite_(double x) { return isfinite(x); }
 
-// Larger / smaller of two values (NaN operands are not propagated; the scheme's results
-// are checked for finiteness where they are written).
+// Larger / smaller of two values; a NaN is passed over, as in fmaxf and fminf (a corner's speeds are
+// NaN where its extrapolated density is negative: the others' decide then).
 MHD_HD float fmax_(float a, float b) { return fmaxf(a, b); }
 MHD_HD float fmin_(float a, float b) { return fminf(a, b); }
 MHD_HD double fmax_(double a, double b) {
 #ifdef __CUDA_ARCH__
-    return order_(__double_as_longlong(a)) >= order_(__double_as_longlong(b)) ? a : b;
+    const bool p = order_(__double_as_longlong(a)) >= order_(__double_as_longlong(b));
+    const double m = p ? a : b;
+    return number_(m) ? m : (p ? b : a);
 #else
     return fmax(a, b);
 #endif
 }
 MHD_HD double fmin_(double a, double b) {
 #ifdef __CUDA_ARCH__
-    return order_(__double_as_longlong(a)) <= order_(__double_as_longlong(b)) ? a : b;
+    const bool p = order_(__double_as_longlong(a)) <= order_(__double_as_longlong(b));
+    const double m = p ? a : b;
+    return number_(m) ? m : (p ? b : a);
 #else
     return fmin(a, b);
 #endif
 }
 
-// max(a, b, c, d, 0) and min(a, b, c, d, 0).  Single precision: two three-input instructions
-// (sm_100 and later); double precision: on the bits, as above (of values among which 0 is, the
-// largest signed integer is the largest value; the smallest value is the largest with its sign
-// turned).
+// max(a, b, c, d, 0) and min(a, b, c, d, 0), NaN passed over.  Single precision: two three-input
+// instructions (sm_100 and later); double precision: on the bits, as above (of values among which 0 is,
+// the largest signed integer is the largest value; the smallest value is the largest with its sign
+// turned; a NaN whose sign makes it the largest counts as 0).
+#ifdef __CUDA_ARCH__
+__device__ __forceinline__ long long max0_bits_(long long a, long long b, long long c, long long d) {
+    auto num = [](long long i) { return i > kInfBits ? 0ll : i; };
+    return max(max(max(num(a), num(b)), max(num(c), num(d))), 0ll);
+}
+#endif
 MHD_HD float max0_(float a, float b, float c, float d) {
 #ifdef __CUDA_ARCH__
     float r;
@@ -242,9 +266,8 @@ MHD_HD float min0_(float a, float b, float c, float d) {
 }
 MHD_HD double max0_(double a, double b, double c, double d) {
 #ifdef __CUDA_ARCH__
-    const long long m = max(max(__double_as_longlong(a), __double_as_longlong(b)),
-                            max(__double_as_longlong(c), __double_as_longlong(d)));
-    return __longlong_as_double(max(m, 0ll));
+    return __longlong_as_double(max0_bits_(__double_as_longlong(a), __double_as_longlong(b), __double_as_longlong(c),
+                                           __double_as_longlong(d)));
 #else
     return fmax(fmax(fmax(a, b), fmax(c, d)), 0.0);
 #endif
@@ -252,27 +275,24 @@ MHD_HD double max0_(double a, double b, double c, double d) {
 MHD_HD double min0_(double a, double b, double c, double d) {
 #ifdef __CUDA_ARCH__
     const long long s = (long long)0x8000000000000000ull;
-    const long long m = max(max(__double_as_longlong(a) ^ s, __double_as_longlong(b) ^ s),
-                            max(__double_as_longlong(c) ^ s, __double_as_longlong(d) ^ s));
-    return __longlong_as_double(max(m, 0ll) ^ s);
+    return __longlong_as_double(max0_bits_(__double_as_longlong(a) ^ s, __double_as_longlong(b) ^ s,
+                                           __double_as_longlong(c) ^ s, __double_as_longlong(d) ^ s) ^ s);
 #else
     return fmin(fmin(fmin(a, b), fmin(c, d)), 0.0);
 #endif
 }
 
 // minmod(a, b): the argument of smaller magnitude when both have the same sign, else 0, i.e.
-// the median of a, b and 0.
+// the median of a, b and 0 (double precision: 0 beside a NaN).
 MHD_HD float minmod_(float a, float b) {
     return fminf(fmaxf(a, fminf(b, 0.0f)), fmaxf(b, 0.0f));
 }
 MHD_HD double minmod_(double a, double b) {
 #ifdef __CUDA_ARCH__
-    // on the integer pipe (doubles of one sign order as their bits): the FP64 pipe, where a
-    // comparison costs as much as a product, is what bounds the FP64 kernels
     const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-    const long long m = 0x7fffffffffffffffll;
-    const long long pick = (ia & m) <= (ib & m) ? ia : ib;
-    return __longlong_as_double((ia ^ ib) < 0 ? 0ll : pick);
+    const long long ma = ia & kMagBits, mb = ib & kMagBits;
+    const long long pick = ma <= mb ? ia : ib;
+    return __longlong_as_double((ia ^ ib) < 0 || max(ma, mb) > kInfBits ? 0ll : pick);
 #else
     return same_sign_(a, b) ? (fabs(a) <= fabs(b) ? a : b) : 0.0;
 #endif

@@ -186,13 +186,13 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         R rootl, rootr;
         const R hl = fast_h(g4 * pl, gpl + b2l, (gpl - b2l) * (gpl - b2l), btl, rootl) * rcp_(rl);
         const R hr = fast_h(g4 * pr, gpr + b2r, (gpr - b2r) * (gpr - b2r), btr, rootr) * rcp_(rr);
-        cl = !greater_(hr, hl);
+        cl = number_(hl) && !greater_(hr, hl);
         cmax = rsqrt_(R(0.5) * (cl ? hl : hr));
         croot = cl ? rootl : rootr;
     } else {
         const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
         const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
-        cl = !greater_(cfr, cfl);
+        cl = number_(cfl) && !greater_(cfr, cfl);
         cmax = cl ? cfl : cfr;
     }
     const bool ml = !greater_(ul, ur);     // min picks u_L
@@ -527,7 +527,7 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
         F[k][4] = (e[k] + pt[k]) * u - bn * vb[k];
     }
     const R ul = L[1], ur = Rt[1];
-    const bool cl = !greater_(cf[1], cf[0]);
+    const bool cl = number_(cf[0]) && !greater_(cf[1], cf[0]);
     const R cmax = cl ? cf[0] : cf[1];
     const bool ml = !greater_(ul, ur), Ml = !greater_(ur, ul);
     const R sl = (ml ? ul : ur) - cmax;
@@ -636,7 +636,8 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
         bp[k] = s.ub + cb[k];
         bm[k] = s.ub - cb[k];
     }
-    // folds with the selected index (-1: the clip at zero won) and what the selected speed came from
+    // folds with the selected index (-1: the clip at zero won) and what the selected speed came from; a
+    // NaN is passed over, as in max0_ and min0_
     struct Pick {
         int k;
         R c, root;
@@ -646,7 +647,7 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
         p = {0, c[0], r[0]};
 #pragma unroll
         for (int j = 1; j < 4; ++j)
-            if (greater_(x[j], m)) {
+            if (greater_(x[j], m) || !number_(m)) {
                 m = x[j];
                 p = {j, c[j], r[j]};
             }
@@ -661,7 +662,7 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
         p = {0, c[0], r[0]};
 #pragma unroll
         for (int j = 1; j < 4; ++j)
-            if (greater_(m, x[j])) {
+            if (greater_(m, x[j]) || !number_(m)) {
                 m = x[j];
                 p = {j, c[j], r[j]};
             }

@@ -12,7 +12,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-OPS = ["greater", "hlld_vjp"]
+OPS = ["greater", "hlld_vjp", "compare", "max0", "emf2d", "emf2d_vjp"]
 DTYPES = [torch.float64, torch.float32]
 both = pytest.mark.parametrize("dtype", DTYPES, ids=["f64", "f32"])
 
@@ -65,3 +65,60 @@ def test_hlld_reverse_at_rest_does_not_depend_on_the_sign_of_zero(ops, dtype):
     assert np.all(np.isfinite(y)) and np.any(y[:, [1, 8]] != 0)
     for k in range(1, 4):
         assert np.array_equal(y[k], y[0]), k
+
+
+def special(dtype):
+    """Values whose bits order in every way: zeros, normal numbers, infinities, NaN of both signs
+    (double precision: subnormal numbers too)."""
+    v = [0.0, -0.0, 1.0, -1.0, 1.5, -1.5, 1e-30, -1e-30, 3e30, -3e30, np.inf, -np.inf, np.nan, np.copysign(np.nan, -1.0)]
+    return np.array(v + ([5e-324, -5e-324, 1e-310] if dtype == torch.float64 else []))
+
+
+def same(got, ref):
+    return np.all((got == ref) | (np.isnan(got) & np.isnan(ref)))
+
+
+@both
+def test_comparisons_are_those_of_the_values(ops, dtype):
+    x = pairs(special(dtype))
+    a, b = (x.astype(np.float32) if dtype == torch.float32 else x).T
+    y = ops("compare", x, 8, dtype).T
+    with np.errstate(invalid="ignore"):
+        for k, ref in enumerate((a >= 0, a > 0, a != 0, a > b, ((a > 0) & (b > 0)) | ((a < 0) & (b < 0)))):
+            assert same(y[k], ref.astype(float)), k
+        assert same(y[5], np.fmax(a, b)) and same(y[6], np.fmin(a, b))
+        both_ = ((a > 0) & (b > 0)) | ((a < 0) & (b < 0))
+        ref = np.where(both_, np.where(np.abs(a) <= np.abs(b), a, b), 0)
+        ok = slice(None) if dtype == torch.float64 else ~(np.isnan(a) | np.isnan(b))
+        assert same(y[7][ok], ref[ok])
+
+
+@both
+def test_largest_and_smallest_of_four_pass_over_nan(ops, dtype):
+    v = special(dtype)
+    x = v[np.random.default_rng(3).integers(0, len(v), size=(4096, 4))]
+    x = np.concatenate([x, [[s] * 4 for s in v]])
+    y = ops("max0", x, 2, dtype)
+    x = x.astype(y.dtype)
+    assert same(y[:, 0], np.fmax(np.fmax.reduce(x, axis=1), 0)) and same(y[:, 1], np.fmin(np.fmin.reduce(x, axis=1), 0))
+
+
+@both
+@pytest.mark.parametrize("bad", range(4))
+def test_edge_emf_beside_a_corner_without_speeds(ops, dtype, bad):
+    """A corner whose extrapolated density is negative has no fast speed; the speeds of the other three
+    decide, in the EMF and in its reverse: both equal, bit for bit, those with a corner so dense that its
+    speeds are never the largest."""
+    rng = np.random.default_rng(60 + bad)
+    n = 256
+    c = np.empty((n, 4, 7))
+    c[:, :, 0] = rng.uniform(0.8, 1.2, (n, 4))
+    c[:, :, 1] = rng.uniform(0.8, 1.2, (n, 4))
+    c[:, :, 2:] = rng.uniform(-0.1, 0.1, (n, 4, 5))
+    neg, dense = c.copy(), c.copy()
+    neg[:, bad, 0], dense[:, bad, 0] = -0.3, 1e8
+    l = rng.normal(size=(n, 1))
+    e = [ops("emf2d", r.reshape(n, 28), 1, dtype) for r in (neg, dense)]
+    assert np.all(np.isfinite(e[1])) and np.array_equal(e[0], e[1])
+    g = [ops("emf2d_vjp", np.concatenate([r.reshape(n, 28), l], axis=1), 28, dtype) for r in (neg, dense)]
+    assert np.all(np.isfinite(g[1])) and np.array_equal(g[0], g[1])
