@@ -40,7 +40,8 @@ MHD_HD R limited(R a, R b, int limiter) {
 // Fast magnetosonic speed along a normal with field component bn (transverse bt1, bt2).
 // cf^2 = 1/2 (cs^2 + ca^2 + sqrt(disc)), disc = (cs^2 + ca^2)^2 - 4 cs^2 can^2 evaluated
 // as (cs^2 - can^2)^2 + cat^2 (2 (cs^2 + can^2) + cat^2) (identical, no cancellation).
-template <typename R>
+// EXACT: correctly rounded square roots (the CFL rates), else near ones (the solvers).
+template <bool EXACT, typename R>
 MHD_HD R fast_speed(R rho_inv, R gP, R bn, R bt1, R bt2) {
     // (products that feed sums are unfusable: every kernel rounds the speed the same way)
     const R cs2 = mul_(gP, rho_inv);
@@ -50,7 +51,8 @@ MHD_HD R fast_speed(R rho_inv, R gP, R bn, R bt1, R bt2) {
     const R disc = fma_(d, d, cat2 * fma_(R(2), cs2 + can2, cat2));
     // 1/2 (s + sqrt(disc)) as one fused step after the square root (halving is exact, so
     // this rounds as 1/2 * (s + sqrt(disc)) does)
-    return rsqrt_(fma_(R(0.5), rsqrt_(disc), R(0.5) * (cs2 + can2 + cat2)));
+    auto root = [](R x) { return EXACT ? rsqrt_(x) : rsqrt_near_(x); };
+    return root(fma_(R(0.5), root(disc), R(0.5) * (cs2 + can2 + cat2)));
 }
 
 // Primitive state from the conserved one; the cell-centred field is the mean of the two
@@ -140,7 +142,7 @@ MHD_HD void hancock_dw(const R q[8], const R dW[3][8], const R dxi[3], R hdt, R 
 // Returns 2 rho c_f^2; root: sqrt(disc).
 template <typename R>
 MHD_HD R fast_h(R gP4, R s, R dd, R bt2, R& root) {
-    root = rsqrt_(fma_(gP4, bt2, dd));
+    root = rsqrt_near_(fma_(gP4, bt2, dd));
     return s + root;
 }
 template <typename R>
@@ -180,28 +182,28 @@ MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[
         const R dfl = fma_(gamma, pl, -b2l), dfr = fma_(gamma, pr, -b2r);
         const R hl = fast_h(g4 * pl, fma_(gamma, pl, b2l), dfl * dfl, btl);
         const R hr = fast_h(g4 * pr, fma_(gamma, pr, b2r), dfr * dfr, btr);
-        cmax = rsqrt_(half * fmax_(hl * rcp_(rl), hr * rcp_(rr)));
+        cmax = rsqrt_near_(half * fmax_(hl * rcp_near_(rl), hr * rcp_near_(rr)));
     } else {
         b2l = fma_(byl, byl, fma_(bzl, bzl, bn2));
         b2r = fma_(byr, byr, fma_(bzr, bzr, bn2));
-        cmax = fmax_(fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl), fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr));
+        cmax = fmax_(fast_speed<false>(rcp_near_(rl), gamma * pl, bn, byl, bzl), fast_speed<false>(rcp_near_(rr), gamma * pr, bn, byr, bzr));
     }
     const R ptl = fma_(half, b2l, pl), ptr = fma_(half, b2r, pr);
     const R sl = fmin_(ul, ur) - cmax;
     const R sr = fmax_(ul, ur) + cmax;
     const R sul = sl - ul, sur = sr - ur;
     const R dl = sul * rl, dr = sur * rr;
-    const R deni = rcp_(dr - dl);
+    const R deni = rcp_near_(dr - dl);
     const R sm = (fma_(dr, ur, -dl * ul) - ptr + ptl) * deni;
 
     // star states (transverse velocity and field)
     const R sml = sl - sm, smr = sr - sm;
-    const R sli = rcp_(sml), sri = rcp_(smr);
+    const R sli = rcp_near_(sml), sri = rcp_near_(smr);
     const R rsl = dl * sli, rsr = dr * sri;
     const R Dl = fma_(dl, sml, -bn2), Dr = fma_(dr, smr, -bn2);
     const R epb = eps * bn2;
     const auto degl = le_mag_(rabs(Dl), epb), degr = le_mag_(rabs(Dr), epb);
-    const R Dli = sel(degl, zero, rcp_(Dl)), Dri = sel(degr, zero, rcp_(Dr));
+    const R Dli = sel(degl, zero, rcp_near_(Dl)), Dri = sel(degr, zero, rcp_near_(Dr));
     const R nul = bn * (sm - ul) * Dli, nur = bn * (sm - ur) * Dri;   // 0 when degenerate
     const R nbl = sel(degl, R(1), fma_(dl, sul, -bn2) * Dli), nbr = sel(degr, R(1), fma_(dr, sur, -bn2) * Dri);
     const R vsl = fma_(-byl, nul, vl), wsl = fma_(-bzl, nul, wl);
@@ -211,9 +213,9 @@ MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[
 
     // double-star states (sign of bn: at bn = 0 their region has zero width and is never the
     // one selected, so the value there does not matter)
-    const R sql = rsqrt_(rsl), sqr = rsqrt_(rsr);
+    const R sql = rsqrt_near_(rsl), sqr = rsqrt_near_(rsr);
     const R sgn = copysign(R(1), bn);
-    const R isum = rcp_(sql + sqr);
+    const R isum = rcp_near_(sql + sqr);
     const R vss = fma_(sql, vsl, fma_(sqr, vsr, (bysr - bysl) * sgn)) * isum;
     const R wss = fma_(sql, wsl, fma_(sqr, wsr, (bzsr - bzsl) * sgn)) * isum;
     const R sq2 = sql * sqr * sgn;
@@ -238,7 +240,7 @@ MHD_HD void hlld(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, R F[
     const R es = fma_(su, e0, fma_(-pt0, u0, fma_(pts, sm, bn * (vb0 - vbs)))) * si;
     const R ess = fma_(sq * sgn, vbs - vbss, es);
     R sa;   // Alfven speed of the side (sq < 0 on the left)
-    if constexpr (F64) sa = fma_(rabs(bn), rcp_(sq), sm);
+    if constexpr (F64) sa = fma_(rabs(bn), rcp_near_(sq), sm);
     else sa = sm + rdiv(rabs(bn), sq);
 
     // region: outer (L, R), star or double star
@@ -296,8 +298,8 @@ MHD_HD void hll(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R F[5]) {
     const R ptl = fma_(half, b2l, pl), ptr = fma_(half, b2r, pr);
     const R el = fma_(pl, gm1i, half * fma_(rl, fma_(ul, ul, fma_(vl, vl, wl * wl)), b2l));
     const R er = fma_(pr, gm1i, half * fma_(rr, fma_(ur, ur, fma_(vr, vr, wr * wr)), b2r));
-    const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
-    const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
+    const R cfl = fast_speed<false>(rcp_near_(rl), gamma * pl, bn, byl, bzl);
+    const R cfr = fast_speed<false>(rcp_near_(rr), gamma * pr, bn, byr, bzr);
     const R vbl = fma_(ul, bn, fma_(vl, byl, wl * bzl)), vbr = fma_(ur, bn, fma_(vr, byr, wr * bzr));
     const R cmax = fmax_(cfl, cfr);
     const R sl = fmin_(ul, ur) - cmax;
@@ -309,7 +311,7 @@ MHD_HD void hll(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R F[5]) {
                      fma_(el + ptl, ul, -bn * vbl)};
     const R FR[5] = {mr, fma_(mr, ur, ptr - bn2), fma_(mr, vr, -byr * bn), fma_(mr, wr, -bzr * bn),
                      fma_(er + ptr, ur, -bn * vbr)};
-    const R di = rcp_(sr - sl);
+    const R di = rcp_near_(sr - sl);
     const R slr = sl * sr;
     const auto gl = nonneg_(sl), gr = nonneg_(sr);
 #pragma unroll
@@ -331,19 +333,19 @@ struct Corner {
 template <typename R>
 MHD_HD void corner_speeds(const Corner<R>& s, R gamma, R& cfa, R& cfb, R& ra, R& rb) {
     if constexpr (sizeof(R) == 8) {
-        const R hri = R(0.5) * rcp_(s.rho), gP4 = R(4) * gamma * s.p;
+        const R hri = R(0.5) * rcp_near_(s.rho), gP4 = R(4) * gamma * s.p;
         const R be2 = s.Be * s.Be;
         const R ta = fma_(s.Bb, s.Bb, be2), tb = fma_(s.Ba, s.Ba, be2);   // transverse to a, to b
         const R b2 = fma_(s.Ba, s.Ba, ta);
         const R sf = fma_(gamma, s.p, b2), df = fma_(gamma, s.p, -b2);
         const R dd = df * df;
-        cfa = rsqrt_(fast_h(gP4, sf, dd, ta, ra) * hri);
-        cfb = rsqrt_(fast_h(gP4, sf, dd, tb, rb) * hri);
+        cfa = rsqrt_near_(fast_h(gP4, sf, dd, ta, ra) * hri);
+        cfb = rsqrt_near_(fast_h(gP4, sf, dd, tb, rb) * hri);
     } else {   // the rounding of fast_speed (see hlld)
         ra = rb = R(0);
-        const R ri = rcp_(s.rho), gP = gamma * s.p;
-        cfa = fast_speed(ri, gP, s.Ba, s.Bb, s.Be);
-        cfb = fast_speed(ri, gP, s.Bb, s.Ba, s.Be);
+        const R ri = rcp_near_(s.rho), gP = gamma * s.p;
+        cfa = fast_speed<false>(ri, gP, s.Ba, s.Bb, s.Be);
+        cfb = fast_speed<false>(ri, gP, s.Bb, s.Ba, s.Be);
     }
 }
 
@@ -376,7 +378,7 @@ MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, co
     const R eNE = fma_(NE.ua, NE.Bb, -NE.ub * NE.Ba);
     // [S_E (S_N E_SW - S_S E_NW) - S_W (S_N E_SE - S_S E_NE)] / (da db)
     const R num = fma_(sE, fma_(sN, eSW, -sS * eNW), -sW * fma_(sN, eSE, -sS * eNE));
-    const R ida = rcp_(da), idb = rcp_(db);
+    const R ida = rcp_near_(da), idb = rcp_near_(db);
     return fma_(sE * sW * ida, SE.Bb - SW.Bb, fma_(num * ida, idb, -(sN * sS * idb) * (NW.Ba - SW.Ba)));
 }
 
@@ -396,14 +398,14 @@ MHD_HD R emf_line(const Corner<R>& s0, const Corner<R>& s1, bool along_a, R gamm
             const R bn = along_a ? s.Ba : s.Bb, bt = along_a ? s.Bb : s.Ba;
             const R bt2 = fma_(bt, bt, s.Be * s.Be), b2 = fma_(bn, bn, bt2);
             const R df = fma_(gamma, s.p, -b2);
-            return rsqrt_(fast_h(R(4) * gamma * s.p, fma_(gamma, s.p, b2), df * df, bt2) * (R(0.5) * rcp_(s.rho)));
+            return rsqrt_near_(fast_h(R(4) * gamma * s.p, fma_(gamma, s.p, b2), df * df, bt2) * (R(0.5) * rcp_near_(s.rho)));
         };
         const R c0 = speed(s0), c1 = speed(s1);
         const R u0 = along_a ? s0.ua : s0.ub, u1 = along_a ? s1.ua : s1.ub;
         const R S1 = fmax_(fmax_(u0 + c0, u1 + c1), R(0)), S0 = fmin_(fmin_(u0 - c0, u1 - c1), R(0));
         const R e0 = fma_(s0.ua, s0.Bb, -s0.ub * s0.Ba), e1 = fma_(s1.ua, s1.Bb, -s1.ub * s1.Ba);
         const R dB = along_a ? s1.Bb - s0.Bb : s0.Ba - s1.Ba;
-        return fma_(S1 * S0, dB, fma_(S1, e0, -S0 * e1)) * rcp_(S1 - S0);
+        return fma_(S1 * S0, dB, fma_(S1, e0, -S0 * e1)) * rcp_near_(S1 - S0);
     }
 }
 

@@ -113,9 +113,9 @@ __global__ void cfl_uniform_kernel(const R* __restrict__ U, int npatch, int nx, 
         R q[8];
         cons_to_prim(c[0], c[vol], c[2 * vol], c[3 * vol], c[4 * vol], bxc, byc, bzc, gm1, q);
         const R ri = rcp_(q[Q_RHO]), gP = gamma * q[Q_P];
-        R rate = (rabs(q[Q_U]) + fast_speed(ri, gP, bxc, byc, bzc)) * dxi0;
-        if (ay) rate += (rabs(q[Q_V]) + fast_speed(ri, gP, byc, bzc, bxc)) * dxi1;
-        if (az) rate += (rabs(q[Q_W]) + fast_speed(ri, gP, bzc, bxc, byc)) * dxi2;
+        R rate = (rabs(q[Q_U]) + fast_speed<true>(ri, gP, bxc, byc, bzc)) * dxi0;
+        if (ay) rate += (rabs(q[Q_V]) + fast_speed<true>(ri, gP, byc, bzc, bxc)) * dxi1;
+        if (az) rate += (rabs(q[Q_W]) + fast_speed<true>(ri, gP, bzc, bxc, byc)) * dxi2;
         if (isfinite((double)rate)) vmax = rate > vmax ? rate : vmax;
         else bad = true;
     }

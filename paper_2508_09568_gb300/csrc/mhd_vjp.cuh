@@ -50,17 +50,17 @@ MHD_HD void slope_vjp(R qm, R q0, R qp, int limiter, R lo, R& lqm, R& lq0, R& lq
 template <typename R>
 MHD_HD void fast_speed_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R lcf, R& lrho, R& lP, R& lbn, R& lbt1,
                            R& lbt2) {
-    const R ri = rcp_(rho);
+    const R ri = rcp_near_(rho);
     const R cs2 = gamma * P * ri;
     const R can2 = bn * bn * ri;
     const R cat2 = (bt1 * bt1 + bt2 * bt2) * ri;
     const R d = cs2 - can2;
     const R disc = d * d + cat2 * (R(2) * (cs2 + can2) + cat2);
-    const R s = rsqrt_(disc);
+    const R s = rsqrt_near_(disc);
     const R h = R(0.5) * (cs2 + can2 + cat2 + s);
-    const R cf = rsqrt_(h);
-    const R lh = positive_(cf) ? R(0.5) * lcf * rcp_(cf) : R(0);
-    const R ldisc = positive_(disc) ? R(0.25) * lh * rcp_(s) : R(0);
+    const R cf = rsqrt_near_(h);
+    const R lh = positive_(cf) ? R(0.5) * lcf * rcp_near_(cf) : R(0);
+    const R ldisc = positive_(disc) ? R(0.25) * lh * rcp_near_(s) : R(0);
     const R lcs2 = R(0.5) * lh + ldisc * (R(2) * d + R(2) * cat2);
     const R lcan2 = R(0.5) * lh + ldisc * (R(-2) * d + R(2) * cat2);
     const R lcat2 = R(0.5) * lh + ldisc * (R(2) * (cs2 + can2) + R(2) * cat2);
@@ -77,11 +77,11 @@ MHD_HD void fast_speed_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R lcf, R& lr
 template <typename R>
 MHD_HD void fast_h_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R cf, R root, R lcf, R& lrho, R& lP, R& lbn, R& lbt1,
                        R& lbt2) {
-    const R hri = R(0.5) * rcp_(rho), gP = gamma * P;
+    const R hri = R(0.5) * rcp_near_(rho), gP = gamma * P;
     const R t = fma_(bt1, bt1, bt2 * bt2), d = gP - fma_(bn, bn, t);
     const R lx = lcf * hri;
-    const R lh = positive_(cf) ? R(0.5) * lx * rcp_(cf) : R(0);      // of s + root
-    const R ld = positive_(root) ? lh * rcp_(root) : R(0);           // of disc, twice
+    const R lh = positive_(cf) ? R(0.5) * lx * rcp_near_(cf) : R(0);      // of s + root
+    const R ld = positive_(root) ? lh * rcp_near_(root) : R(0);           // of disc, twice
     const R lb = fma_(-ld, d, lh);                                   // of B^2
     const R l2 = R(2) * lb, lt = fma_(R(4) * gP, ld, l2);
     lP += gamma * fma_(ld, fma_(R(2), t, d), lh);
@@ -184,14 +184,14 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     if constexpr (sizeof(R) == 8) {
         const R g4 = R(4) * gamma, gpl = gamma * pl, gpr = gamma * pr;
         R rootl, rootr;
-        const R hl = fast_h(g4 * pl, gpl + b2l, (gpl - b2l) * (gpl - b2l), btl, rootl) * rcp_(rl);
-        const R hr = fast_h(g4 * pr, gpr + b2r, (gpr - b2r) * (gpr - b2r), btr, rootr) * rcp_(rr);
+        const R hl = fast_h(g4 * pl, gpl + b2l, (gpl - b2l) * (gpl - b2l), btl, rootl) * rcp_near_(rl);
+        const R hr = fast_h(g4 * pr, gpr + b2r, (gpr - b2r) * (gpr - b2r), btr, rootr) * rcp_near_(rr);
         cl = number_(hl) && !greater_(hr, hl);
-        cmax = rsqrt_(R(0.5) * (cl ? hl : hr));
+        cmax = rsqrt_near_(R(0.5) * (cl ? hl : hr));
         croot = cl ? rootl : rootr;
     } else {
-        const R cfl = fast_speed(rcp_(rl), gamma * pl, bn, byl, bzl);
-        const R cfr = fast_speed(rcp_(rr), gamma * pr, bn, byr, bzr);
+        const R cfl = fast_speed<false>(rcp_near_(rl), gamma * pl, bn, byl, bzl);
+        const R cfr = fast_speed<false>(rcp_near_(rr), gamma * pr, bn, byr, bzr);
         cl = number_(cfl) && !greater_(cfr, cfl);
         cmax = cl ? cfl : cfr;
     }
@@ -201,7 +201,7 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     const R sr = (Ml ? ul : ur) + cmax;
     const R dl = (sl - ul) * rl, dr = (sr - ur) * rr;
     const R den = dr - dl;
-    const R deni = rcp_(den);
+    const R deni = rcp_near_(den);
     const R smn = dr * ur - dl * ul - ptr + ptl;
     const R ptn = dr * ptl - dl * ptr + dl * dr * (ur - ul);
     const R sm = smn * deni;
@@ -214,10 +214,10 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         Side t{W[0], W[1], W[2], W[3], W[4], W[5], W[6], b2, pt, S};
         t.sa = S - t.u;
         t.ssm = S - sm;
-        t.ssmi = rcp_(t.ssm);
+        t.ssmi = rcp_near_(t.ssm);
         t.rs = t.r * t.sa * t.ssmi;
-        t.sq = rsqrt_(t.rs);
-        t.isq = rcp_(t.sq);
+        t.sq = rsqrt_near_(t.rs);
+        t.isq = rcp_near_(t.sq);
         return t;
     };
     const Side A = side(L, b2l, ptl, sl), B = side(Rt, b2r, ptr, sr);
@@ -270,7 +270,7 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
         Star t;
         const R D = T.r * T.sa * T.ssm - bn2;
         t.deg = le_mag_(rabs(D), eps * bn2);
-        t.Di = t.deg ? R(0) : rcp_(D);
+        t.Di = t.deg ? R(0) : rcp_near_(D);
         t.nu = bn * (sm - T.u) * t.Di;
         t.nb = (T.r * T.sa * T.sa - bn2) * t.Di;
         t.vs = t.deg ? T.v : T.v - T.by * t.nu;
@@ -379,7 +379,7 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
                 const Energy Eo = energy(O);
                 const Star F = star(O, Eo);
                 StarGrad k;
-                const R isum = rcp_(N.sq + O.sq), sq2 = N.sq * O.sq * sg;
+                const R isum = rcp_near_(N.sq + O.sq), sq2 = N.sq * O.sq * sg;
                 const R dvs = (F.vs - T.vs) * sg, dws = (F.ws - T.ws) * sg;
                 const R vss = (N.sq * T.vs + O.sq * F.vs + (F.bys - T.bys) * sg) * isum;
                 const R wss = (N.sq * T.ws + O.sq * F.ws + (F.bzs - T.bzs) * sg) * isum;
@@ -513,7 +513,7 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
         const R b2 = bn2 + by * by + bz * bz;
         pt[k] = p + R(0.5) * b2;
         e[k] = p * gm1i + R(0.5) * r * (u * u + v * v + w * w) + R(0.5) * b2;
-        cf[k] = fast_speed(rcp_(r), gamma * p, bn, by, bz);
+        cf[k] = fast_speed<false>(rcp_near_(r), gamma * p, bn, by, bz);
         vb[k] = u * bn + v * by + w * bz;
         U[k][0] = r;
         U[k][1] = r * u;
@@ -538,7 +538,7 @@ MHD_HD void hll_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, const R 
     if (nonneg_(sl)) {
         for (int c = 0; c < 5; ++c) lFs[0][c] = lF[c];
     } else if (nonneg_(sr)) {
-        const R di = rcp_(sr - sl);
+        const R di = rcp_near_(sr - sl);
         for (int c = 0; c < 5; ++c) {
             const R dU = U[1][c] - U[0][c];
             const R fh = (sr * F[0][c] - sl * F[1][c] + sl * sr * dU) * di;
@@ -680,7 +680,7 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
 #pragma unroll
     for (int k = 0; k < 4; ++k) e[k] = st[k]->ua * st[k]->Bb - st[k]->ub * st[k]->Ba;
     const R num = sE * sN * e[0] - sE * sS * e[2] - sW * sN * e[1] + sW * sS * e[3];
-    const R ida = rcp_(da), idb = rcp_(db);
+    const R ida = rcp_near_(da), idb = rcp_near_(db);
     const R t2 = sE * sW * ida, t3 = sN * sS * idb;
     const R jb = SE.Bb - SW.Bb, ja = NW.Ba - SW.Ba;
     // E = num / (da db) + t2 jb - t3 ja

@@ -6,7 +6,7 @@
 using R = REAL;
 using namespace mhd;
 
-enum Op { GREATER, HLLD_VJP, COMPARE, MAX0, EMF2D, EMF2D_VJP };
+enum Op { GREATER, HLLD_VJP, COMPARE, MAX0, EMF2D, EMF2D_VJP, ROOTS };
 
 __device__ Corner<R> corner_of(const R* x) { return Corner<R>{x[0], x[1], x[2], x[3], x[4], x[5], x[6]}; }
 __device__ void to_row(const Corner<R>& c, R* y) {
@@ -38,6 +38,11 @@ __global__ void rows(int op, int nin, int nout, const R* in, R* out, int n) {
     } else if (op == MAX0) {   // four values
         y[0] = max0_(x[0], x[1], x[2], x[3]);
         y[1] = min0_(x[0], x[1], x[2], x[3]);
+    } else if (op == ROOTS) {
+        y[0] = rsqrt_(x[0]);
+        y[1] = rcp_(x[0]);
+        y[2] = rsqrt_near_(x[0]);
+        y[3] = rcp_near_(x[0]);
     } else {   // four corners: rho, p, ua, ub, Ba, Bb, Be each
         Corner<R> c[4];
         for (int v = 0; v < 4; ++v) c[v] = corner_of(x + 7 * v);

@@ -12,7 +12,7 @@ import torch
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-OPS = ["greater", "hlld_vjp", "compare", "max0", "emf2d", "emf2d_vjp"]
+OPS = ["greater", "hlld_vjp", "compare", "max0", "emf2d", "emf2d_vjp", "roots"]
 DTYPES = [torch.float64, torch.float32]
 both = pytest.mark.parametrize("dtype", DTYPES, ids=["f64", "f32"])
 
@@ -122,3 +122,42 @@ def test_edge_emf_beside_a_corner_without_speeds(ops, dtype, bad):
     assert np.all(np.isfinite(e[1])) and np.array_equal(e[0], e[1])
     g = [ops("emf2d_vjp", np.concatenate([r.reshape(n, 28), l], axis=1), 28, dtype) for r in (neg, dense)]
     assert np.all(np.isfinite(g[1])) and np.array_equal(g[0], g[1])
+
+
+def test_fp64_square_root_and_reciprocal(ops):
+    """Over every exponent with random significands, beside the powers of two (significands of few bits
+    and of almost all), at the squares of points half way between two numbers and at reciprocals of
+    numbers, where the rounding is closest; at and beside the ends of the range of the fast forms; and
+    the special values.  rsqrt_ and rcp_: bit for bit the IEEE operations (numpy's).  The near forms:
+    the same bits outside the range, at most the neighbour inside it, and within 0.51 units in the last
+    place of the exact value (0.5 of the rounding and the two forms' remainders, at most 2^-60 and 2^-59
+    of the value, 0.008 and 0.016 units, less than that where they add to 0.5)."""
+    rng = np.random.default_rng(70)
+    n = 1 << 19
+    man = rng.integers(0, 1 << 52, n, dtype=np.uint64)
+    few = rng.integers(0, 1 << 12, n, dtype=np.uint64)
+    one = np.uint64(1) << rng.integers(0, 52, n, dtype=np.uint64)
+    top = np.uint64((1 << 52) - 1)
+    ex = rng.integers(1, 2047, n, dtype=np.uint64) << np.uint64(52)
+    m = ((np.uint64(1023) << np.uint64(52)) | man).view(np.float64)
+    mid = np.ldexp(m * m + m * 2.0 ** -52, 2 * rng.integers(-400, 400, n))
+    inv = np.ldexp(1.0 / m, rng.integers(-800, 800, n))
+    ends = np.array([s for e in (-900, 900, -1022, 0, 1) for s in (2.0 ** e, np.nextafter(2.0 ** e, 0), np.nextafter(2.0 ** e, 9e300))])
+    x = np.concatenate([(ex | v).view(np.float64) for v in (man, few, top - few, one, top - one, np.full(n, top))]
+                       + [mid, inv, ends, np.finfo(float).max * np.ones(1), special(torch.float64)])
+    x = np.concatenate([x, -x])
+    y = ops("roots", x[:, None], 4, torch.float64)
+    with np.errstate(invalid="ignore", divide="ignore", over="ignore"):
+        ref = np.stack([np.sqrt(x), 1.0 / x], axis=1)
+        assert same(y[:, :2], ref)
+        assert np.array_equal(np.signbit(y[:, 1][np.isinf(x)]), np.signbit(x[np.isinf(x)]))
+        inside = (np.abs(x) >= 2.0 ** -900) & (np.abs(x) < 2.0 ** 900)
+        assert same(y[~inside, 2:], ref[~inside])
+        k = inside & (x > 0)
+        assert np.all(np.abs(y[k, 2] - ref[k, 0]) <= np.spacing(ref[k, 0]))
+        assert np.all(np.abs(y[inside, 3] - ref[inside, 1]) <= np.spacing(np.abs(ref[inside, 1])))
+    x, y = x[:n][k[:n]][:100000], y[:n][k[:n]][:100000]
+    xl = x.astype(np.longdouble)   # (64 bits of significand or more)
+    assert np.finfo(np.longdouble).nmant >= 63
+    for c, exact in ((2, np.sqrt(xl)), (3, 1 / xl)):
+        assert np.max(np.abs(y[:, c] - exact) / np.spacing(y[:, c])) <= 0.51
