@@ -247,6 +247,20 @@ MHD_HD float rdiv(float a, float b) {
 }
 MHD_HD double rdiv(double a, double b) { return a / b; }
 
+// a / b from y, the reciprocal of b or a near one.  Double precision on the device: the product and one
+// step on its residual (Markstein), rounded once like the quotient itself, where a y is rounded twice
+// (and y's 0.507 ulp come on top); two operations more.  Single precision: the product.
+MHD_HD float quot_(float a, float b, float y) { return a * y; }
+MHD_HD double quot_(double a, double b, double y) {
+#ifdef __CUDA_ARCH__
+    const double q = __dmul_rn(a, y), q1 = __fma_rn(__fma_rn(-b, q, a), y, q);
+    // (an infinite or zero y, an overflow: the product)
+    return (__double2hiint(q1) & 0x7ff00000) != 0x7ff00000 ? q1 : q;
+#else
+    return a / b;
+#endif
+}
+
 // x is finite (tested in its own precision: no conversion to double)
 MHD_HD bool finite_(float x) { return isfinite(x); }
 MHD_HD bool finite_(double x) { return isfinite(x); }

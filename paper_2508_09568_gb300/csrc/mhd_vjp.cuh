@@ -59,8 +59,8 @@ MHD_HD void fast_speed_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R lcf, R& lr
     const R s = rsqrt_near_(disc);
     const R h = R(0.5) * (cs2 + can2 + cat2 + s);
     const R cf = rsqrt_near_(h);
-    const R lh = positive_(cf) ? R(0.5) * lcf * rcp_near_(cf) : R(0);
-    const R ldisc = positive_(disc) ? R(0.25) * lh * rcp_near_(s) : R(0);
+    const R lh = positive_(cf) ? quot_(R(0.5) * lcf, cf, rcp_near_(cf)) : R(0);
+    const R ldisc = positive_(disc) ? quot_(R(0.25) * lh, s, rcp_near_(s)) : R(0);
     const R lcs2 = R(0.5) * lh + ldisc * (R(2) * d + R(2) * cat2);
     const R lcan2 = R(0.5) * lh + ldisc * (R(-2) * d + R(2) * cat2);
     const R lcat2 = R(0.5) * lh + ldisc * (R(2) * (cs2 + can2) + R(2) * cat2);
@@ -80,8 +80,8 @@ MHD_HD void fast_h_vjp(R rho, R P, R bn, R bt1, R bt2, R gamma, R cf, R root, R 
     const R hri = R(0.5) * rcp_near_(rho), gP = gamma * P;
     const R t = fma_(bt1, bt1, bt2 * bt2), d = gP - fma_(bn, bn, t);
     const R lx = lcf * hri;
-    const R lh = positive_(cf) ? R(0.5) * lx * rcp_near_(cf) : R(0);      // of s + root
-    const R ld = positive_(root) ? lh * rcp_near_(root) : R(0);           // of disc, twice
+    const R lh = positive_(cf) ? quot_(R(0.5) * lx, cf, rcp_near_(cf)) : R(0);      // of s + root
+    const R ld = positive_(root) ? quot_(lh, root, rcp_near_(root)) : R(0);      // of disc, twice
     const R lb = fma_(-ld, d, lh);                                   // of B^2
     const R l2 = R(2) * lb, lt = fma_(R(4) * gP, ld, l2);
     lP += gamma * fma_(ld, fma_(R(2), t, d), lh);
@@ -286,7 +286,7 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
     };
     auto star_rev = [&](const Side& T, const Energy& E, const Star& t, StarGrad h, SideGrad& g) {
         // sq = sqrt(rs)
-        h.rs += R(0.5) * h.sq * T.isq;
+        h.rs += quot_(R(0.5) * h.sq, T.sq, T.isq);
         // es = nes * ssmi
         const R g_nes = h.es * T.ssmi;
         R g_ssm = -g_nes * t.es;
@@ -362,7 +362,9 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
             const Star T = star(N, En);
             // f += S (U* - U), U* = (rs, rs sm, rs vs, rs ws, es)
             const R ls = lF[0] + lF[1] * sm + lF[2] * T.vs + lF[3] * T.ws;
-            gn.S += N.rs * ls - N.r * (lF[0] + lv) + lF[4] * (T.es - En.e);
+            // (difference by difference: of the two sums the larger parts cancel)
+            gn.S += lF[0] * (N.rs - N.r) + lF[1] * (N.rs * sm - ru) + lF[2] * (N.rs * T.vs - N.r * N.v) +
+                    lF[3] * (N.rs * T.ws - N.r * N.w) + lF[4] * (T.es - En.e);
             const R Sr = N.S * N.r, Srs = N.S * N.rs;
             gn.r -= N.S * (lF[0] + lv);
             gn.u -= Sr * lF[1];
@@ -400,10 +402,10 @@ MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, 
                 h.sq -= g_ess * dvb;
                 const R g_vbss = g_ess * N.sq * sg;
                 h.vbs -= g_vbss;
-                const R gsi = gSs * N.isq;
+                const R gsi = quot_(gSs, N.sq, N.isq);
                 g_sm += gSs;
                 g_tabn -= gsi;
-                h.sq += gsi * N.isq * tabn;
+                h.sq += quot_(gsi * tabn, N.sq, N.isq);
                 // vbss = sm bn + vss byss + wss bzss
                 g_sm += g_vbss * bn;
                 g_bn += g_vbss * sm;
@@ -679,33 +681,22 @@ MHD_HD void emf2d_vjp(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>&
     R e[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) e[k] = st[k]->ua * st[k]->Bb - st[k]->ub * st[k]->Ba;
-    const R num = sE * sN * e[0] - sE * sS * e[2] - sW * sN * e[1] + sW * sS * e[3];
-    const R ida = rcp_near_(da), idb = rcp_near_(db);
-    const R t2 = sE * sW * ida, t3 = sN * sS * idb;
+    // E = [sE X - sW Y] / da + sE sW / da jb - sN sS / db ja, X = (sN e0 - sS e2) / db and Y = (sN e1 -
+    // sS e3) / db, and the same with a and b exchanged; so with 1 - sE / da = -sW / da, in which nothing
+    // cancels, dE/dsE = -sW (X - Y + sW jb) / da^2, dE/dsW = sE (X - Y + sE jb) / da^2, and alike along b
+    const R ida = rcp_near_(da), idb = rcp_near_(db), q = da * db;
     const R jb = SE.Bb - SW.Bb, ja = NW.Ba - SW.Ba;
-    // E = num / (da db) + t2 jb - t3 ja
-    const R g_num = lE * ida * idb;
-    const R g_q = -g_num * num * ida * idb;
-    R g_da = g_q * db, g_db = g_q * da;
-    const R g_t2 = lE * jb * ida, g_t3 = -lE * ja * idb;   // cotangents of t2 and t3 over da and db
-    const R g_jb = lE * t2, g_ja = -lE * t3;
-    R g_sE = g_t2 * sW, g_sW = g_t2 * sE;
-    g_da -= g_t2 * t2;
-    R g_sN = g_t3 * sS, g_sS = g_t3 * sN;
-    g_db -= g_t3 * t3;
+    const R g_jb = lE * quot_(sE * sW, da, ida), g_ja = -lE * quot_(sN * sS, db, idb);
     gSE.Bb += g_jb;
     gSW.Bb -= g_jb;
     gNW.Ba += g_ja;
     gSW.Ba -= g_ja;
-    g_sE += g_num * (sN * e[0] - sS * e[2]);
-    g_sN += g_num * (sE * e[0] - sW * e[1]);
-    g_sS += g_num * (-sE * e[2] + sW * e[3]);
-    g_sW += g_num * (-sN * e[1] + sS * e[3]);
-    R g_e[4] = {g_num * sE * sN, -g_num * sW * sN, -g_num * sE * sS, g_num * sW * sS};
-    g_sE += g_da;
-    g_sW -= g_da;
-    g_sN += g_db;
-    g_sS -= g_db;
+    const R xy = (sN * (e[0] - e[1]) - sS * (e[2] - e[3])) * idb, zt = (sE * (e[0] - e[2]) - sW * (e[1] - e[3])) * ida;
+    const R ga = lE * ida * ida, gb = lE * idb * idb;
+    const R g_sE = -ga * sW * (xy + sW * jb), g_sW = ga * sE * (xy + sE * jb);
+    const R g_sN = -gb * sS * (zt - sS * ja), g_sS = gb * sN * (zt - sN * ja);
+    const R g_num = quot_(lE, q, rcp_near_(q));
+    const R g_e[4] = {g_num * sE * sN, -g_num * sW * sN, -g_num * sE * sS, g_num * sW * sS};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         gs[k]->ua += g_e[k] * st[k]->Bb;

@@ -6,7 +6,7 @@
 using R = REAL;
 using namespace mhd;
 
-enum Op { GREATER, HLLD_VJP, COMPARE, MAX0, EMF2D, EMF2D_VJP, ROOTS };
+enum Op { GREATER, HLLD_VJP, COMPARE, MAX0, EMF2D, EMF2D_VJP, ROOTS, HLL_VJP };
 
 __device__ Corner<R> corner_of(const R* x) { return Corner<R>{x[0], x[1], x[2], x[3], x[4], x[5], x[6]}; }
 __device__ void to_row(const Corner<R>& c, R* y) {
@@ -22,9 +22,10 @@ __global__ void rows(int op, int nin, int nout, const R* in, R* out, int n) {
     const R gamma = R(5.0 / 3.0), gm1i = R(1.5), eps = sizeof(R) == 8 ? R(1e-12) : R(1e-6);
     if (op == GREATER) {
         y[0] = greater_(x[0], x[1]);
-    } else if (op == HLLD_VJP) {   // L[7], R[7], bn, cotangents of the flux[5] -> of L, R, bn
+    } else if (op == HLLD_VJP || op == HLL_VJP) {   // L[7], R[7], bn, cotangents of the flux[5] -> of L, R, bn
         for (int v = 0; v < 15; ++v) y[v] = R(0);
-        hlld_vjp(x, x + 7, x[14], gamma, gm1i, eps, x + 15, y, y + 7, y[14]);
+        if (op == HLLD_VJP) hlld_vjp(x, x + 7, x[14], gamma, gm1i, eps, x + 15, y, y + 7, y[14]);
+        else hll_vjp(x, x + 7, x[14], gamma, gm1i, x + 15, y, y + 7, y[14]);
     } else if (op == COMPARE) {   // a, b
         const R a = x[0], b = x[1];
         y[0] = nonneg_(a);

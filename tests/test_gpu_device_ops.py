@@ -9,10 +9,12 @@ import numpy as np
 import pytest
 import torch
 
+import extended_reference as X
+
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-OPS = ["greater", "hlld_vjp", "compare", "max0", "emf2d", "emf2d_vjp", "roots"]
+OPS = ["greater", "hlld_vjp", "compare", "max0", "emf2d", "emf2d_vjp", "roots", "hll_vjp"]
 DTYPES = [torch.float64, torch.float32]
 both = pytest.mark.parametrize("dtype", DTYPES, ids=["f64", "f32"])
 
@@ -161,3 +163,22 @@ def test_fp64_square_root_and_reciprocal(ops):
     assert np.finfo(np.longdouble).nmant >= 63
     for c, exact in ((2, np.sqrt(xl)), (3, 1 / xl)):
         assert np.max(np.abs(y[:, c] - exact) / np.spacing(y[:, c])) <= 0.51
+
+
+@pytest.mark.parametrize("name,bound", [("hlld_vjp", 1.21), ("hll_vjp", 0.664), ("emf2d_vjp", 0.415)])
+def test_fp64_rounding_error_of_the_reverses(ops, name, bound):
+    """Root mean square error of the cotangents, in units of 2^-53 of the row's largest, against the
+    derivative in extended precision.  The bounds are what the reverses with IEEE divisions and square
+    roots throughout give on the same rows (1.208, 0.6626, 0.4143), rounded up."""
+    n = 3000
+    if name == "emf2d_vjp":
+        x = X.edge_rows(n, 81)
+        v = X.inputs(x[:, :28])
+        ref = (x[:, 28].astype(X.LD) * X.edge_emf([v[7 * k:7 * k + 7] for k in range(4)]).d).T
+    else:
+        x = X.face_rows(n, 82)
+        F = X.face_flux(X.inputs(x[:, :15]), name == "hll_vjp")
+        ref = sum(x[:, 15 + k].astype(X.LD) * F[k].d for k in range(5)).T
+    y = ops(name, x, ref.shape[1], torch.float64)
+    err = (np.abs(y - ref) / np.max(np.abs(ref), axis=1, keepdims=True)).astype(float) * 2.0 ** 53
+    assert np.sqrt(np.mean(err ** 2)) <= bound
