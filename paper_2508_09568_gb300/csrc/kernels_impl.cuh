@@ -167,14 +167,12 @@ static cudaError_t launch_fill_interp(void* U0, void* U1, const PatchDev* patche
                                      const double* t_old, const double* t_cur, const FillGeom& fg,
                                      const int64_t* nboff, int Zp, int64_t pstride, unsigned* err, cudaStream_t s) {
     if (nlist <= 0) return cudaSuccess;
-    const int gy = std::min(std::min(nlist, grid_y > 0 ? grid_y : nlist), 65535);
     if (nboff) {
-        const unsigned grid = (unsigned)std::min<int64_t>((int64_t)nlist * Zp, (int64_t)8 * gy);
-        launch_pdl(fill_interp_grid_kernel<R>, grid, 128, 0, s, static_cast<R*>(U0), static_cast<R*>(U1), patches, nboff,
+        launch_pdl(fill_interp_grid_kernel<R>, interp_grid(nlist, Zp, grid_y), 128, 0, s, static_cast<R*>(U0), static_cast<R*>(U1), patches, nboff,
                    list, nlist, nlist_dev, pstride, Zp, slice, t_old, t_cur);
         return cudaGetLastError();
     }
-    dim3 grid(32, gy);
+    dim3 grid(32, std::min(std::min(nlist, grid_y > 0 ? grid_y : nlist), 65535));
     launch_pdl(fill_interp_kernel<R>, grid, 256, 0, s, static_cast<R*>(U0), static_cast<R*>(U1), patches, npatch, list, nlist,
                                                nlist_dev, slice, t_old, t_cur, fg, err);
     return cudaGetLastError();
