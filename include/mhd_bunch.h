@@ -201,7 +201,8 @@ int mhd_bunch_config_info(const mhd_bunch *b, int config, int *tile_x, int *tile
 
 /* Time each tile configuration on the bound state (a few steps each, the state is
  * restored afterwards) and keep the fastest.  If cache_path is not NULL the choice is
- * read from / written to that text file, keyed by device, precision and patch sizes.
+ * read from / written to that text file, keyed by device, precision, patch sizes and the
+ * compiled tile configurations.
  * In MHD_MODE_MIXED every patch-size class is timed with every configuration on its own
  * tiles and takes its fastest (cache_path is not used); *chosen receives the
  * configuration of the class holding the most cells. */

@@ -1314,7 +1314,8 @@ int mhd_bunch_autotune(mhd_bunch* b, const char* cache_path, int* chosen) try {
     if (rc) return rc;
     const int n = (int)b->cfg_index.size();
     if (n == 0) return fail(MHD_EINVAL, "no compiled kernel for this dimensionality");
-    // cache key: device name, precision, dimensionality and the multiset of patch sizes
+    // cache key: device name, precision, dimensionality, mode, the multiset of patch sizes and the tiles
+    // of the compiled configurations (what is stored is an index into them)
     cudaDeviceProp prop;
     int dev = 0;
     CK(cudaGetDevice(&dev));
@@ -1327,7 +1328,11 @@ int mhd_bunch_autotune(mhd_bunch* b, const char* cache_path, int* chosen) try {
         std::sort(sizes.begin(), sizes.end());
         int64_t h = 1469598103934665603LL;
         for (int s : sizes) h = (h ^ s) * 1099511628211LL;
-        key << "|p" << b->npatch << "|h" << (uint64_t)h;
+        key << "|p" << b->npatch << "|h" << (uint64_t)h << "|c";
+        for (int c = 0; c < n; ++c) {
+            const StepLaunch& L = step_cfg(b, c);
+            key << (c ? "," : "") << L.tx << "x" << L.ty << "x" << L.nt;
+        }
     }
     std::string k = key.str();
     for (auto& ch : k)
