@@ -126,6 +126,41 @@ def test_adjoint_in_every_region_of_the_face_flux_fp64(boost, field):
     assert err <= 1e-10, err
 
 
+@pytest.mark.parametrize("boost,field", [((4, -4, 0), (0, 0, 0)), ((0.3, 4, -4), (0, 0, 0)), ((0.1, -0.1, 0.2), (2, -2, 2)),
+                                         ((-0.6, 0.6, 0.6), (0.7, 0.7, -0.7))],
+                         ids=["supersonic_xy", "supersonic_yz", "double_star", "mixed"])
+@pytest.mark.parametrize("dtype,limiter", [(torch.float64, 1), (torch.float32, 0), (torch.float32, 1)],
+                         ids=["f64-mc", "f32-minmod", "f32-mc"])
+def test_adjoint_in_every_region_fp32_and_mc(boost, field, dtype, limiter):
+    """The states of the test above in single precision, whose reverse takes other branches (fast speeds,
+    largest of them), and with the other limiter.  Double precision: the bound above.  Single precision
+    against the FP64 oracle on the rounded state: the bound of the FP32 test below for 97 % of the
+    entries; the others may lie in the stencil of a choice that rounding turns (some 9e4 choices of
+    limiters, speeds and regions, whose arguments differ by a part in 1e2 and are rounded in 1e7: a few
+    turn, each of some hundred of the 13824 entries)."""
+    geom, U, meta = W.small_box(ncell=(12, 12, 12), patch=(12, 6, 12), seed=49)
+    U = U.copy()
+    for c in range(3):
+        mean = 0.5 * (U[5 + c] + np.roll(U[5 + c], -1, axis=2 - c))
+        U[4] += U[1 + c] * boost[c] + 0.5 * U[0] * boost[c] ** 2 + mean * field[c] + 0.5 * field[c] ** 2
+        U[1 + c] += U[0] * boost[c]
+        U[5 + c] += field[c]
+    mask = interior_mask(geom)
+    flat = jitter(W.to_patches(U, geom), mask, 150)
+    if dtype == torch.float32:
+        flat = flat.astype(np.float32).astype(np.float64)
+    ob = O.Bunch(geom, meta["gamma"])
+    dt = ob.cfl_dt(ob.fill_guards(ob.split(flat)))
+    w = np.where(mask, np.random.default_rng(149).normal(size=flat.size), 0.0)
+    ref = oracle_grad(geom, flat, dt, meta["gamma"], w, limiter, eps=O.HLLD_EPS[4 if dtype == torch.float32 else 8])
+    got, _ = gpu_adjoint(geom, flat, dt, meta["gamma"], w, dtype, limiter)
+    err = np.abs(got[mask] - ref[mask]) / np.max(np.abs(ref[mask]))
+    if dtype == torch.float64:
+        assert np.max(err) <= 1e-10, np.max(err)
+    else:
+        assert np.quantile(err, 0.97) <= 1e-4, (np.quantile(err, 0.97), np.max(err))
+
+
 def test_adjoint_fp32_against_fp64_reference():
     geom, flat, gamma, dt, w, mask = setup(43)
     flat32 = flat.astype(np.float32).astype(np.float64)
