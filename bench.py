@@ -44,11 +44,11 @@ OOC_BUDGET = 4 << 30                       # device budget of the out-of-core le
 # DRAM bytes (read + write) per cell-update of the fused step kernel, FP32, 32^3 patches,
 # per tile configuration (the two the autotuner picks between on this machine):
 # dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture of a 192^3 box of the
-# same patches and tiles (7,077,888 cells; 32 x 8: 451.52 MB + 232.33 MB, 16 x 16:
-# 452.88 MB + 235.08 MB).  Traffic scales with the number of patches, so a launch on the
+# same patches and tiles (7,077,888 cells; 32 x 8: 451.67 MB + 232.25 MB, 16 x 16:
+# 452.86 MB + 233.82 MB).  Traffic scales with the number of patches, so a launch on the
 # full box moves this many bytes per cell.  Valid for this kernel version only.
-STEP_DRAM_BYTES_PER_CELL = {(4, 32, (32, 8, 512)): (451.517696e6 + 232.328448e6) / 7077888,
-                            (4, 32, (16, 16, 512)): (452.884992e6 + 235.075072e6) / 7077888}
+STEP_DRAM_BYTES_PER_CELL = {(4, 32, (32, 8, 512)): (451.673600e6 + 232.246784e6) / 7077888,
+                            (4, 32, (16, 16, 512)): (452.862464e6 + 233.822208e6) / 7077888}
 
 
 def peaks():

@@ -171,9 +171,9 @@ int mhd_bunch_step_device_dt(mhd_bunch *b, const void *dt_dev);
  * not meaningful).  max_rounds >= 1; MHD_ESTATE if max_rounds ran out first (*rounds and
  * the record still cover the rounds done); MHD_EPHYS if a patch's dt came out
  * non-positive or non-finite (later rounds are skipped; the state is then not meaningful).
- * The schedule runs on the device: each round is five stream-ordered launches (schedule,
- * guard fill at the patches' own times, per-patch CFL dt, dt clipping, update); the host
- * enqueues 32 rounds at a time and synchronises the bound stream once per 32 rounds to
+ * The schedule runs on the device: each round is six stream-ordered launches (readiness,
+ * list of the ready patches, guard fill at the patches' own times, per-patch CFL dt, dt
+ * clipping, update); the host enqueues 32 rounds at a time and synchronises the bound stream once per 32 rounds to
  * read their record. */
 int mhd_bunch_advance_async(mhd_bunch *b, double t_span, int max_rounds, int *rounds,
                             int64_t *patch_updates);

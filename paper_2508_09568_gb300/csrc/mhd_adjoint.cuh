@@ -9,10 +9,11 @@
 // The last kernel is the transpose of the guard fill: the cotangent that reached a ghost
 // copy is added to the interior cell it copies.
 //
-// Occupancy: the face and edge kernels (the HLLD / 2D-HLL VJPs) are capped at 128
-// registers (two 256-thread blocks per SM) and take their direction from the grid's z
-// index, so each thread handles one face or edge; the slope kernel is capped at 128
-// registers and the other cell kernels at 85.
+// Occupancy: the face and edge kernels (the HLLD / 2D-HLL VJPs) take their direction from the
+// grid's z index, so each thread handles one face or edge; 256-thread blocks, two per SM (128
+// registers) in single precision, one (255) in double, which is bound by the FP64 pipe.  The slope
+// kernel is capped at 128 registers, the predictor's at 85 (double precision 128), the forward
+// slopes at 64 and the other reverse cell kernels at 85.
 //
 // Work arrays (fields of one value per padded cell, index coff[p] + (z*Y + y)*X + x, in blocks of
 // 32 cells, see fat):

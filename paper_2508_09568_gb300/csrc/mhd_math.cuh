@@ -388,7 +388,8 @@ MHD_HD R emf2d(const Corner<R>& SW, const Corner<R>& SE, const Corner<R>& NW, co
 // flux E = [S_1 e_0 - S_0 e_1 + S_1 S_0 dB] / (S_1 - S_0), S_1 = max(0, max u+cf), S_0 = min(0, min u-cf):
 // 2 fast speeds instead of 8.  Single precision keeps emf2d's rounding; the compiler shares the states
 // that are the same (4 speeds).  512^2 box of 32^2 patches: FP64, 2 steps, 1754 -> 1388 us; FP32, 4 steps,
-// 125.8 -> 118.7 us; 1D, 256 cells, FP64, 8 steps, 98.2 -> 82.5 us.
+// 125.8 -> 118.7 us; 1D, 256 cells, FP64, 8 steps, 98.2 -> 82.5 us (FP64 with the short roots throughout;
+// 1429 and 85.8 us with the rounded ones outside the solvers).
 template <typename R>
 MHD_HD R emf_line(const Corner<R>& s0, const Corner<R>& s1, bool along_a, R gamma) {
     if constexpr (sizeof(R) == 4) {

@@ -782,14 +782,15 @@ struct ChunkList {
 // lists come from the parameter bank: with the lists decoded chunk by chunk from memory, or shared out
 // through a counter, the step took 24.7 and 25.7 ms.
 //
-// What bounds it (FP32): the issue slots (61-66 % busy; 16 warps, the registers allow no more), left
-// empty mostly by waits for instructions (of 5.4 warps waiting per issued instruction 1.4: the code of a
-// phase's solvers and prep is more than the instruction cache holds) and at the ends of the phases (1.0);
-// neither HBM (8 %) nor the FP32 pipes (33 %).  Measured on the 512^3 box, 32x8, step and fill: part of
-// the EMFs inside the plane in either phase, a little more even but with their solver in both, 21.36
-// ms; as it is 20.66; one solver per phase behind the state loads of all directions 21.12 (24^3
+// What bounds it (FP32): the issue slots (70 % busy with 32x8 tiles on 32^3 patches, 64 % with 24x8 on
+// 24^3; 16 warps, the registers allow no more).  Of 5.6 warps waiting per issued instruction 1.5 (24x8:
+// 1.3) lost the slot to another, 1.0 (1.1) wait for a fixed latency, 0.6 (0.8) for instructions (the code
+// of a phase's solvers and prep is more than the instruction cache holds) and 0.6 (1.2) at the ends of
+// the phases; neither HBM (9 %) nor the FP32 pipes (34 %) bound it.  Measured on the 512^3 box, 32x8,
+// step and fill: part of the EMFs inside the plane in either phase, a little more even but with their
+// solver in both (instruction waits 1.4 with 24x8), 21.36 ms; as it is 20.64; one solver per phase behind the state loads of all directions 21.12 (24^3
 // patches -1 %), one with offsets chosen at run time 23.5 (a third more instructions); one chunk list
-// per warp and plane with two mbarrier points instead of the barriers, no waits at the ends (1.02 ->
+// per warp and plane with two mbarrier points instead of the barriers, no waits at the ends (then 1.02 ->
 // 0.04) but all code at once (instruction stalls 2.7), 30.4.  The form before this one, three phases
 // (load + update + conversion / prep / fluxes) whose flux phase ended on a half-filled pass and whose
 // prep left four of sixteen warps idle, took 21.0 ms for the step alone, this one 17.9.  FP64 is bound

@@ -1,9 +1,12 @@
 // Hand-written reverse-mode derivatives (vector-Jacobian products) of the per-element
 // arithmetic in mhd_math.cuh, for the discrete adjoint of one bunch step at fixed dt.
 //
-// Each *_vjp function re-evaluates the forward expression it differentiates (the same
-// sequence as the forward code) and then accumulates (+=) the cotangents of its inputs
-// from the cotangent of its output, sweeping the forward assignments in reverse order.
+// Each *_vjp function re-evaluates the values it needs of the forward expression and then
+// accumulates (+=) the cotangents of its inputs from the cotangent of its output, sweeping the
+// assignments in reverse order.  It differentiates the expression, not its rounding: where the
+// forward code of a precision writes the same value in another form (the double-precision HLLD
+// flux, the edge EMF's speeds) the two differ by rounding, also in a choice between branches
+// whose arguments are equal to rounding.
 // Non-differentiable points take the branch the forward took: the limiter passes the
 // cotangent to the argument it selected (ties: the first; none when the arguments differ
 // in sign or one is zero), max/min pass it to the selected argument (ties: the first),
@@ -168,7 +171,9 @@ MHD_HD void hancock_vjp(const R q[8], const R D[3][8], R hdt, R gamma, const R l
     lq[Q_RHO] -= lri * ri * ri;
 }
 
-// d hlld: lF[5] -> lL[7], lR[7], lbn.  Same forward sequence as hlld().
+// d hlld: lF[5] -> lL[7], lR[7], lbn: the derivative of F + S (U* - U) + S* (U** - U*) in the region at
+// x/t = 0, in both precisions (hlld in double precision takes the flux function at the region's state,
+// which the jump conditions make equal).
 template <typename R>
 MHD_HD void hlld_vjp(const R L[7], const R Rt[7], R bn, R gamma, R gm1i, R eps, const R lF[5], R lL[7], R lR[7],
                      R& lbn) {
